@@ -2,13 +2,16 @@
 // images, read-back of populations and macroscopic fields, and the FP64
 // reductions behind Laplace's law (Eq. 22) and the run statistics.
 // None of these is on the per-step path.
+#include <type_traits>
+
 #include "lbm_internal.cuh"
 #include "lbm_init.h"
+#include "lbm_reduce.cuh"
 
 namespace lbm {
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = kRedThreads;
 
 // Lattice weights t_a of the D2Q9 equilibrium (4/9, 1/9, 1/36).
 __device__ __forceinline__ double tw(int a) { return a == 0 ? 4.0 / 9.0 : (a < 5 ? 1.0 / 9.0 : 1.0 / 36.0); }
@@ -148,192 +151,223 @@ __global__ void k_gather(const Inst* __restrict__ I, int parity, int a, double* 
     }
 }
 
-// rho and momentum sum f e of node (x, y), x in [-1, nx], y in [-1, ny].
-template <typename T>
-__device__ __forceinline__ double node_rho(const Inst* I, const T* p, int x, int y, double* jx, double* jy) {
-    double r = 0.0, mx = 0.0, my = 0.0;
+// The nine populations pulled by node (x, y), x in [-1, nx], y in [-1, ny].
+template <typename T> __device__ __forceinline__ void node_pops(const Inst* I, const T* p, int x, int y, T (&v)[9]) {
 #pragma unroll
-    for (int a = 0; a < 9; ++a) {
-        const double v = static_cast<double>(p[at<T>(I, a, x - cx(a), y - cy(a))]);
-        r += v;
-        mx += cx(a) * v;
-        my += cy(a) * v;
-    }
-    if (jx) *jx = mx;
-    if (jy) *jy = my;
-    return r + static_cast<double>(phys<T>(I).rho_ref);
+    for (int a = 0; a < 9; ++a) v[a] = p[at<T>(I, a, x - cx(a), y - cy(a))];
 }
 
-// rho of an FP32 node from its nine deviations: their sum as an unevaluated
-// pair hi + lo (Knuth's TwoSum gives the exact error of each addition; the
-// errors are summed in FP32), then hi + lo + rho_ref in FP64.  Within about
-// 2^-45 of the FP64 sum relative to the deviations' sum, and three FP64
-// operations per node instead of eighteen: GB300's FP64 pipe would
-// otherwise bound the density read-back.
-__device__ __forceinline__ double node_rho_f32(const Inst* I, const float* p, int x, int y) {
-    float hi = 0.0f, lo = 0.0f;
+// Sum of N floats in FP64 accuracy with three FP64 additions: the sum as an
+// unevaluated triple hi + lo + lo2 (Knuth's TwoSum gives the exact error of
+// each addition; the errors' own sum is kept the same way), within 2^-69 of
+// the largest partial sum, closer than adding the N values one after another
+// in FP64.  About 13 FP32 operations per value, which GB300 issues at 64
+// times the rate of FP64 ones.  A sum that leaves FP32's range (an unstable
+// lattice) is formed in FP64.
+template <int N> __device__ __forceinline__ double sum_f32(const float (&v)[N], double plus) {
+    float hi = v[0], lo = 0.0f, lo2 = 0.0f;
+    auto two_sum = [](float a, float b, float& err) {
+        const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+        err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+        return s;
+    };
 #pragma unroll
-    for (int a = 0; a < 9; ++a) {
-        const float v = p[at<float>(I, a, x - cx(a), y - cy(a))];
-        const float sum = __fadd_rn(hi, v);
-        const float bv = __fsub_rn(sum, hi);
-        const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(sum, bv)), __fsub_rn(v, bv));
-        hi = sum;
-        lo = __fadd_rn(lo, err);
+    for (int k = 1; k < N; ++k) {
+        float e, e2;
+        hi = two_sum(hi, v[k], e);
+        lo = two_sum(lo, e, e2);
+        lo2 = __fadd_rn(lo2, e2);
     }
-    return (static_cast<double>(hi) + static_cast<double>(lo)) + static_cast<double>(I->pf.rho_ref);
+    if (!(fabsf(hi) < 3.0e38f)) {
+        double r = 0.0;
+        for (int k = 0; k < N; ++k) r += static_cast<double>(v[k]);
+        return r + plus;
+    }
+    return (static_cast<double>(hi) + plus) + (static_cast<double>(lo) + static_cast<double>(lo2));
 }
 
-__device__ __forceinline__ double psi_of(const Phys<double>& P, double rho) {
-    return sqrt(psi_radicand(P, rho));
+// rho of a node from its nine populations.
+__device__ __forceinline__ double node_rho(const Inst* I, const float (&v)[9]) {
+    return sum_f32<9>(v, static_cast<double>(I->pf.rho_ref));
+}
+__device__ __forceinline__ double node_rho(const Inst* I, const double (&v)[9]) {
+    double r = 0.0;
+#pragma unroll
+    for (int a = 0; a < 9; ++a) r += v[a];
+    return r + I->pd.rho_ref;
+}
+template <typename T> __device__ __forceinline__ double node_rho(const Inst* I, const T* p, int x, int y) {
+    T v[9];
+    node_pops(I, p, x, y, v);
+    return node_rho(I, v);
+}
+// momentum sum f e
+__device__ __forceinline__ void node_j(const float (&v)[9], double& jx, double& jy) {
+    const float sx[6] = {v[1], -v[3], v[5], -v[6], -v[7], v[8]}, sy[6] = {v[2], -v[4], v[5], v[6], -v[7], -v[8]};
+    jx = sum_f32<6>(sx, 0.0);
+    jy = sum_f32<6>(sy, 0.0);
+}
+__device__ __forceinline__ void node_j(const double (&v)[9], double& jx, double& jy) {
+    jx = v[1] - v[3] + v[5] - v[6] - v[7] + v[8];
+    jy = v[2] - v[4] + v[5] + v[6] - v[7] - v[8];
 }
 
-// rho, velocity (Eq. 9 force, rho u = sum f e + F/2) and psi of node (x, y).
-template <typename T>
-__device__ void node_fields(const Inst* I, const T* p, int x, int y, double* rho, double* ux, double* uy,
-                            double* psi) {
+// Tiles of the kernels that need the force (velocity fields, statistics):
+// psi of the tile and its 1-node ring (periodic) goes to shared memory once,
+// so a node costs 1.25 densities and square roots instead of nine, and about
+// 100 FP64 instructions instead of 700 (the FP64 pipe is the bound: 16
+// clocks of an SM per warp instruction).  32 x 16 nodes: two per thread, a
+// ring of 612 nodes in 20 warp passes for 16 of the tile's own.
+// FP32 statistics of 1024^2: 1113 -> 250 us per call, of 256^2: 149 -> 35;
+// the two velocity components of 1531 x 1117: 2 x 1709 -> 396 us, rho and
+// psi with them.
+constexpr int kFlowX = 32, kFlowY = 16, kFlowW = kFlowX + 2, kFlowH = kFlowY + 2;
+struct FlowTile {
+    double psi[kFlowH][kFlowW], rho[kFlowH][kFlowW];
+};
+
+// rho, velocity (rho u = sum f e + F/2, F of Eq. 9) and psi of the nodes
+// of tile (x0, y0), rows below y1, given to use(x, y, rho, ux, uy, psi) by
+// the thread that owns each; every thread of the block (kThreads) calls it.
+template <typename T, typename Use>
+__device__ __forceinline__ void flow_tile(const Inst* I, const T* p, int x0, int y0, int y1, FlowTile& S, Use use) {
     const Phys<double>& P = I->pd;
-    const int nx = I->nx, ny = I->ny;
-    double jx, jy;
-    const double r = node_rho<T>(I, p, x, y, &jx, &jy);
-    double Fx = 0.0, Fy = 0.0, ps = 0.0;
-    if (P.interact) {
-        ps = psi_of(P, r);
-        double gx1 = 0, gy1 = 0, gx2 = 0, gy2 = 0;
-#pragma unroll
-        for (int a = 1; a < 9; ++a) {
-            int xn = x + cx(a), yn = y + cy(a);
-            xn = xn < 0 ? xn + nx : (xn >= nx ? xn - nx : xn);
-            yn = yn < 0 ? yn + ny : (yn >= ny ? yn - ny : yn);
-            const double pn = psi_of(P, node_rho<T>(I, p, xn, yn, nullptr, nullptr));
-            const double w = (a < 5) ? 1.0 / 3.0 : 1.0 / 12.0;
-            gx1 += w * pn * cx(a);
-            gy1 += w * pn * cy(a);
-            gx2 += w * pn * pn * cx(a);
-            gy2 += w * pn * pn * cy(a);
+    const int nx = I->nx, ny = I->ny, interact = P.interact;
+    const int tid = threadIdx.x;
+    if (interact) {
+        const LawFp64 radicand(P, true);
+        const int w = min(kFlowX, nx - x0) + 2, h = min(kFlowY, y1 - y0) + 2;
+        for (int e = tid; e < kFlowW * kFlowH; e += kThreads) {
+            const int j = e / kFlowW, i = e - j * kFlowW;
+            if (i >= w || j >= h) continue;
+            int x = x0 + i - 1, y = y0 + j - 1;
+            x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
+            y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
+            const double r = node_rho<T>(I, p, x, y);
+            S.rho[j][i] = r;
+            S.psi[j][i] = sqrt(radicand(r));
         }
-        Fx = -P.G * (0.5 * P.A * gx2 + (1.0 - P.A) * ps * gx1);
-        Fy = -P.G * (0.5 * P.A * gy2 + (1.0 - P.A) * ps * gy1);
+        __syncthreads();
     }
-    *rho = r;
-    *ux = (jx + 0.5 * Fx) / r;
-    *uy = (jy + 0.5 * Fy) / r;
-    *psi = ps;
+    const double negGw = -P.G * (1.0 / 12.0), hA = 0.5 * P.A, omA = 1.0 - P.A;
+    const int i = tid % kFlowX + 1, x = x0 + i - 1;
+    for (int j = tid / kFlowX + 1; j <= kFlowY; j += kThreads / kFlowX) {
+        const int y = y0 + j - 1;
+        if (x >= nx || y >= y1) continue;
+        T v[9];
+        node_pops(I, p, x, y, v);
+        const double r = interact ? S.rho[j][i] : node_rho(I, v);
+        double jx, jy, ps = 0.0;
+        node_j(v, jx, jy);
+        if (interact) {
+            // Eq. 9 with the weights 12 w_a (4 on the axes, 1 on the diagonals)
+            const double p1 = S.psi[j][i + 1], p2 = S.psi[j + 1][i], p3 = S.psi[j][i - 1], p4 = S.psi[j - 1][i];
+            const double p5 = S.psi[j + 1][i + 1], p6 = S.psi[j + 1][i - 1], p7 = S.psi[j - 1][i - 1],
+                         p8 = S.psi[j - 1][i + 1];
+            ps = S.psi[j][i];
+            const double a57 = p5 - p7, a86 = p8 - p6, b57 = p5 * p5 - p7 * p7, b86 = p8 * p8 - p6 * p6;
+            const double gx1 = 4.0 * (p1 - p3) + (a57 + a86), gy1 = 4.0 * (p2 - p4) + (a57 - a86);
+            const double gx2 = 4.0 * (p1 * p1 - p3 * p3) + (b57 + b86), gy2 = 4.0 * (p2 * p2 - p4 * p4) + (b57 - b86);
+            const double c = omA * ps;
+            jx += 0.5 * (negGw * (c * gx1 + hA * gx2));
+            jy += 0.5 * (negGw * (c * gy1 + hA * gy2));
+        }
+        use(x, y, r, jx / r, jy / r, ps);
+    }
+    if (interact) __syncthreads();   // before the next tile's psi
 }
 
-// One macroscopic field per launch (0 rho, 1 u_x, 2 u_y, 3 psi), each its
-// own kernel: the density read-back keeps the registers of a plain gather.
-// Rows [y0, y1) of the field, at their place in out (row-major nx x ny).
+// rho or psi of the nodes, one field per launch (FIELD 0 rho, 3 psi): the
+// density read-back keeps the registers of a plain gather.  Rows [y0, y1) of
+// the field, at their place in out (row-major nx x ny).
 template <typename T, int FIELD, typename O>
-__global__ void k_field(const Inst* __restrict__ I, int parity, int y0, int y1, O* __restrict__ out) {
+__global__ void k_field(const Inst* __restrict__ I, int parity, int y0, int y1, O* __restrict__ out,
+                        int* status) {
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *status = *I->status;
     const int nx = I->nx;
     const T* p = popk<T>(I, parity);
+    const LawFp64 radicand(I->pd, true);
     for (int y = y0 + static_cast<int>(blockIdx.y); y < y1; y += gridDim.y)
         for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < nx; x += gridDim.x * blockDim.x) {
-            const long long i = static_cast<long long>(y) * nx + x;
-            double v;
-            if constexpr (FIELD == 0 && sizeof(T) == 4) {
-                v = node_rho_f32(I, p, x, y);
-            } else if constexpr (FIELD == 0) {
-                v = node_rho<T>(I, p, x, y, nullptr, nullptr);
-            } else if constexpr (FIELD == 3) {
-                v = I->pd.interact ? psi_of(I->pd, node_rho<T>(I, p, x, y, nullptr, nullptr)) : 0.0;
-            } else {
-                double r, u, w, s;
-                node_fields<T>(I, p, x, y, &r, &u, &w, &s);
-                v = FIELD == 1 ? u : w;
-            }
-            out[i] = static_cast<O>(v);
+            const double r = node_rho<T>(I, p, x, y);
+            double v = r;
+            if constexpr (FIELD == 3) v = I->pd.interact ? sqrt(radicand(r)) : 0.0;
+            out[static_cast<long long>(y) * nx + x] = static_cast<O>(v);
         }
 }
 
-// ---- FP64 block reductions ----------------------------------------------
-// Each block writes kReduceSlots partial sums (slot `max_slot` is a max);
-// k_finish adds the partials in a fixed order, so results are deterministic.
-__device__ __forceinline__ void block_reduce_store(double (&v)[kReduceSlots], int max_slot, double* partials) {
-    __shared__ double red[kThreads / 32][kReduceSlots];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < kReduceSlots; ++k) {
-        double x = v[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double y = __shfl_down_sync(0xffffffffu, x, o);
-            x = (k == max_slot) ? fmax(x, y) : x + y;
-        }
-        if (lane == 0) red[warp][k] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x < kReduceSlots) {
-        const int k = threadIdx.x;
-        double x = red[0][k];
-        for (int w = 1; w < kThreads / 32; ++w) x = (k == max_slot) ? fmax(x, red[w][k]) : x + red[w][k];
-        partials[blockIdx.x * kReduceSlots + k] = x;
-    }
-}
-
-__global__ void k_finish(const double* __restrict__ partials, int nblocks, int max_slot, double* __restrict__ out) {
-    const int k = threadIdx.x;
-    if (k >= kReduceSlots) return;
-    double x = partials[k];
-    for (int b = 1; b < nblocks; ++b) {
-        const double y = partials[b * kReduceSlots + k];
-        x = (k == max_slot) ? fmax(x, y) : x + y;
-    }
-    out[k] = x;
-}
-
-// Sums for Laplace's law: {sum rho, sum p_in, sum rho_in, n_in, sum p_out,
-// sum rho_out, n_out, 0}; p = p_EOS(rho) (equal to rho/3 + G psi^2/2, Eq. 10).
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k_measure(const Inst* __restrict__ I, int parity, double cxc, double cyc,
-                                                       double r_in, double r_out, double* __restrict__ partials) {
-    const int nx = I->nx, ny = I->ny;
-    const long long N = static_cast<long long>(nx) * ny;
+// The velocity components and, where asked for, rho and psi of rows [y0, y1)
+// in one pass (any output may be NULL).
+template <typename T, typename O>
+__global__ void __launch_bounds__(kThreads) k_flow(const Inst* __restrict__ I, int parity, int y0, int y1,
+                                                   O* __restrict__ rho, O* __restrict__ ux, O* __restrict__ uy,
+                                                   O* __restrict__ psi, int* status) {
+    __shared__ FlowTile S;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *status = *I->status;
+    const int nx = I->nx, tiles_x = (nx + kFlowX - 1) / kFlowX, tiles = tiles_x * ((y1 - y0 + kFlowY - 1) / kFlowY);
     const T* p = popk<T>(I, parity);
-    double v[kReduceSlots] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < N;
-         i += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int x = static_cast<int>(i % nx), y = static_cast<int>(i / nx);
-        const double r = node_rho<T>(I, p, x, y, nullptr, nullptr);
-        double dx = x - cxc, dy = y - cyc;
-        dx -= nx * rint(dx / nx);
-        dy -= ny * rint(dy / ny);
-        const double d = sqrt(dx * dx + dy * dy);
-        v[0] += r;
-        if (d <= r_in) {
-            v[1] += p_eos(I->pd, r);
-            v[2] += r;
-            v[3] += 1.0;
-        }
-        if (d >= r_out) {
-            v[4] += p_eos(I->pd, r);
-            v[5] += r;
-            v[6] += 1.0;
-        }
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int ty = t / tiles_x;
+        flow_tile<T>(I, p, (t - ty * tiles_x) * kFlowX, y0 + ty * kFlowY, y1, S,
+                     [&](int x, int y, double r, double u, double w, double ps) {
+                         const long long i = static_cast<long long>(y) * nx + x;
+                         if (rho) rho[i] = static_cast<O>(r);
+                         if (ux) ux[i] = static_cast<O>(u);
+                         if (uy) uy[i] = static_cast<O>(w);
+                         if (psi) psi[i] = static_cast<O>(ps);
+                     });
     }
-    block_reduce_store(v, -1, partials);
+}
+
+// ---- FP64 reductions (lbm_reduce.cuh) -------------------------------------
+// Sums for Laplace's law (LaplaceSums); p = p_EOS(rho) (equal to
+// rho/3 + G psi^2/2, Eq. 10).  The last block puts the totals and the
+// instance's status into *out, which is mapped host memory: the call needs no
+// second launch and no copy.  About 33 FP64 instructions per node (nine
+// additions in FP64, the square root and the divisions by the lattice's size
+// are gone).  Per call, FP32: 256^2 88 -> 24 us, 1024^2 236 -> 85 us.
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_measure(const Inst* __restrict__ I, int parity, Discs D, int rpt,
+                                                       double* __restrict__ partials, unsigned* ticket,
+                                                       Reduced* out) {
+    __shared__ double dy2[kTileRows * kMaxRpt];
+    const T* p = popk<T>(I, parity);
+    LaplaceSums L;
+    laplace_tiles(L, LawFp64(I->pd, false), D, I->nx, I->ny, rpt, dy2,
+                  [&](int x, int y) { return node_rho<T>(I, p, x, y); });
+    double total;
+    if (grid_sum8(L.v, -1, 0.0, partials, ticket, &total)) {
+        out->v[threadIdx.x] = total;
+        if (threadIdx.x == 0) out->status = *I->status;
+    }
 }
 
 // {mass, sum rho u_x, sum rho u_y, sum rho |u|^2 / 2, max |u|, 0, 0, 0}
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_stats(const Inst* __restrict__ I, int parity, double* __restrict__ partials) {
+__global__ void __launch_bounds__(kThreads) k_stats(const Inst* __restrict__ I, int parity, double* __restrict__ partials,
+                                                     unsigned* ticket, Reduced* out) {
+    __shared__ FlowTile S;
     const int nx = I->nx, ny = I->ny;
-    const long long N = static_cast<long long>(nx) * ny;
+    const int tiles_x = (nx + kFlowX - 1) / kFlowX, tiles = tiles_x * ((ny + kFlowY - 1) / kFlowY);
     const T* p = popk<T>(I, parity);
-    double v[kReduceSlots] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < N;
-         i += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int x = static_cast<int>(i % nx), y = static_cast<int>(i / nx);
-        double r, u, w, s;
-        node_fields<T>(I, p, x, y, &r, &u, &w, &s);
-        v[0] += r;
-        v[1] += r * u;
-        v[2] += r * w;
-        v[3] += 0.5 * r * (u * u + w * w);
-        v[4] = fmax(v[4], sqrt(u * u + w * w));
+    double v[8] = {0, 0, 0, 0, 0, 0, 0, 0}, most = 0.0;   // most: max |u|^2 (the root is monotone)
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int ty = t / tiles_x;
+        flow_tile<T>(I, p, (t - ty * tiles_x) * kFlowX, ty * kFlowY, ny, S,
+                     [&](int, int, double r, double u, double w, double) {
+                         const double u2 = u * u + w * w;
+                         v[0] += r;
+                         v[1] += r * u;
+                         v[2] += r * w;
+                         v[3] += 0.5 * r * u2;
+                         most = fmax(most, u2);
+                     });
     }
-    block_reduce_store(v, 4, partials);
+    double total;
+    if (grid_sum8(v, 4, most, partials, ticket, &total)) {
+        out->v[threadIdx.x] = threadIdx.x == 4 ? sqrt(total) : total;
+        if (threadIdx.x == 0) out->status = *I->status;
+    }
 }
 
 int grid_for(long long n) {
@@ -507,45 +541,65 @@ cudaError_t aux_gather_plane(const Inst& h, const Inst* d, int parity, int a, do
 }
 
 template <typename O>
-cudaError_t field_t(const Inst& h, const Inst* d, int parity, int field, int y0, int y1, O* out, cudaStream_t st) {
+cudaError_t field_t(const Inst& h, const Inst* d, int parity, int field, int y0, int y1, O* out, int* status,
+                    cudaStream_t st) {
     const dim3 g = grid_2d(h.nx, y1 - y0);
-    auto go = [&](auto k) { k<<<g, kThreads, 0, st>>>(d, parity, y0, y1, out); };
+    auto go = [&](auto k) { k<<<g, kThreads, 0, st>>>(d, parity, y0, y1, out, status); };
     const bool f32 = h.prec == LBM_FP32;
-    switch (field) {
-    case 0: f32 ? go(k_field<float, 0, O>) : go(k_field<double, 0, O>); break;
-    case 1: f32 ? go(k_field<float, 1, O>) : go(k_field<double, 1, O>); break;
-    case 2: f32 ? go(k_field<float, 2, O>) : go(k_field<double, 2, O>); break;
-    default: f32 ? go(k_field<float, 3, O>) : go(k_field<double, 3, O>); break;
-    }
+    if (field == 0) f32 ? go(k_field<float, 0, O>) : go(k_field<double, 0, O>);
+    else f32 ? go(k_field<float, 3, O>) : go(k_field<double, 3, O>);
     return cudaGetLastError();
 }
 
 cudaError_t aux_field(const Inst& h, const Inst* d, int parity, int field, int y0, int y1, void* out, bool f32out,
-                      cudaStream_t st) {
-    if (f32out) return field_t(h, d, parity, field, y0, y1, static_cast<float*>(out), st);
-    return field_t(h, d, parity, field, y0, y1, static_cast<double*>(out), st);
+                      int* status, cudaStream_t st) {
+    if (field != 0 && field != 3) return cudaErrorInvalidValue;
+    if (f32out) return field_t(h, d, parity, field, y0, y1, static_cast<float*>(out), status, st);
+    return field_t(h, d, parity, field, y0, y1, static_cast<double*>(out), status, st);
 }
 
-cudaError_t aux_measure(const Inst& h, const Inst* d, int parity, double cxc, double cyc, double r_in,
-                        double r_out, double* partials, double* result, cudaStream_t st) {
-    if (h.prec == LBM_FP32)
-        k_measure<float><<<kReduceBlocks, kThreads, 0, st>>>(d, parity, cxc, cyc, r_in, r_out, partials);
-    else
-        k_measure<double><<<kReduceBlocks, kThreads, 0, st>>>(d, parity, cxc, cyc, r_in, r_out, partials);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_finish<<<1, 32, 0, st>>>(partials, kReduceBlocks, -1, result);
+// Blocks of the flow and reduction kernels: one per tile up to what the
+// device holds at once (eight blocks of 256 threads on each of 152 SMs).
+constexpr int kResident = 8 * 152;
+int flow_grid(int nx, int rows) {
+    const long long tiles = static_cast<long long>((nx + kFlowX - 1) / kFlowX) * ((rows + kFlowY - 1) / kFlowY);
+    return static_cast<int>(tiles < kResident ? tiles : kResident);
+}
+
+cudaError_t aux_flow(const Inst& h, const Inst* d, int parity, int y0, int y1, void* const out[4], bool f32out,
+                     int* status, cudaStream_t st) {
+    const int g = flow_grid(h.nx, y1 - y0);
+    auto go = [&](auto k, auto* zero) {
+        using O = typename std::remove_pointer<decltype(zero)>::type;
+        k<<<g, kThreads, 0, st>>>(d, parity, y0, y1, static_cast<O*>(out[0]), static_cast<O*>(out[1]),
+                                  static_cast<O*>(out[2]), static_cast<O*>(out[3]), status);
+    };
+    const bool f32 = h.prec == LBM_FP32;
+    float* zf = nullptr;
+    double* zd = nullptr;
+    if (f32out) f32 ? go(k_flow<float, float>, zf) : go(k_flow<double, float>, zf);
+    else f32 ? go(k_flow<float, double>, zd) : go(k_flow<double, double>, zd);
     return cudaGetLastError();
 }
 
-cudaError_t aux_stats(const Inst& h, const Inst* d, int parity, double* partials, double* result, cudaStream_t st) {
-    if (h.prec == LBM_FP32)
-        k_stats<float><<<kReduceBlocks, kThreads, 0, st>>>(d, parity, partials);
-    else
-        k_stats<double><<<kReduceBlocks, kThreads, 0, st>>>(d, parity, partials);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_finish<<<1, 32, 0, st>>>(partials, kReduceBlocks, 4, result);
+cudaError_t aux_measure(const Inst& h, const Inst* d, int parity, double cxc, double cyc, double r_in,
+                        double r_out, double* partials, int rows, unsigned* ticket, Reduced* out,
+                        cudaStream_t st) {
+    if (rows > kResident) rows = kResident;
+    const Discs D = make_discs(h.nx, h.ny, cxc, cyc, r_in, r_out);
+    const int rpt = tile_rpt(h.nx, h.ny);
+    const long long tiles = tile_count(h.nx, h.ny, rpt);
+    const int g = static_cast<int>(tiles < rows ? tiles : rows);
+    if (h.prec == LBM_FP32) k_measure<float><<<g, kThreads, 0, st>>>(d, parity, D, rpt, partials, ticket, out);
+    else k_measure<double><<<g, kThreads, 0, st>>>(d, parity, D, rpt, partials, ticket, out);
+    return cudaGetLastError();
+}
+
+cudaError_t aux_stats(const Inst& h, const Inst* d, int parity, double* partials, int rows, unsigned* ticket,
+                      Reduced* out, cudaStream_t st) {
+    const int tiles = flow_grid(h.nx, h.ny), g = tiles < rows ? tiles : rows;
+    if (h.prec == LBM_FP32) k_stats<float><<<g, kThreads, 0, st>>>(d, parity, partials, ticket, out);
+    else k_stats<double><<<g, kThreads, 0, st>>>(d, parity, partials, ticket, out);
     return cudaGetLastError();
 }
 

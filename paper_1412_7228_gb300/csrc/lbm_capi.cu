@@ -9,6 +9,7 @@
 #include <cstring>
 #include <string>
 #include <type_traits>
+#include <utility>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -237,6 +238,8 @@ struct lbm_ctx {
     int* d_status = nullptr;
     double* d_partials = nullptr;
     double* d_result = nullptr;
+    unsigned* d_ticket = nullptr;           // of the reductions' last block; zero between launches
+    lbm::Reduced* h_red = nullptr;          // pinned, mapped: the device writes results and the status here
     double* d_scratch = nullptr;
     int parity = 0;
     long long steps = 0, launches = 0;
@@ -629,11 +632,24 @@ int check_idx(lbm_ctx* c, int i) {
     return LBM_OK;
 }
 
+int status_code(int st) {
+    return (st & lbm::ST_UNSTABLE) ? LBM_EUNSTABLE : ((st & lbm::ST_TIMEOUT) ? LBM_ETIMEOUT : LBM_OK);
+}
+
 int status_of(lbm_ctx* c, int i, int* code) {
     int st = 0;
     CK(c, cudaMemcpy(&st, c->d_status + i, sizeof(int), cudaMemcpyDeviceToHost));
-    *code = (st & lbm::ST_UNSTABLE) ? LBM_EUNSTABLE : ((st & lbm::ST_TIMEOUT) ? LBM_ETIMEOUT : LBM_OK);
+    *code = status_code(st);
     return LBM_OK;
+}
+
+// Where a reduction's blocks put their partial sums, and how many rows fit:
+// the field scratch, idle then, unless a small lattice has fewer than
+// the rows that every context keeps.
+std::pair<double*, int> partial_rows(lbm_ctx* c) {
+    const size_t rows = c->L.scratch_elems / lbm::kReduceSlots;
+    if (rows <= lbm::kReduceBlocks) return {c->d_partials, lbm::kReduceBlocks};
+    return {c->d_scratch, static_cast<int>(std::min<size_t>(rows, 1 << 20))};
 }
 
 int sync_all(lbm_ctx* c) {
@@ -843,40 +859,70 @@ template <typename O> int read_fields_t(lbm_ctx* c, int i, O* rho, O* ux, O* uy,
     // a large lattice in row bands: band b's copy to the host overlaps band b + 1's kernel
     const int bands = field_bands(c, i);
     if (bands > 1 && (rc = ensure_copy_stream(c))) return rc;
-    O* outs[4] = {rho, ux, uy, psi};
+    O* const outs[4] = {rho, ux, uy, psi};
     O* const scratch = reinterpret_cast<O*>(c->d_scratch);
     constexpr bool f32 = sizeof(O) == 4;
-    for (int f = 0; f < 4; ++f) {
-        if (!outs[f]) continue;
-        if (bands == 1) {
-            CK(c, lbm::aux_field(c->h[i], c->d_inst + i, c->parity, f, 0, ny, scratch, f32, c->stream));
-            CK(c, cudaMemcpyAsync(outs[f], scratch, N * sizeof(O), cudaMemcpyDeviceToHost, c->stream));
-            CK(c, cudaStreamSynchronize(c->stream));
-            continue;
+    // the fields in groups that the scratch holds side by side: with a
+    // velocity component asked for, everything comes from one pass over the
+    // lattice (four FP64 fields: rho first, by itself); rho or psi alone from
+    // passes of their own, which read less
+    struct Group {
+        bool flow;
+        std::vector<int> f;
+    };
+    std::vector<Group> groups;
+    std::vector<int> want;
+    for (int f = 0; f < 4; ++f)
+        if (outs[f]) want.push_back(f);
+    if (ux || uy) {
+        if (want.size() * N * sizeof(O) > c->L.scratch_elems * sizeof(double)) {
+            groups.push_back({false, {0}});
+            want.erase(want.begin());
         }
-        auto issue_bands = [&]() -> int {
-            for (int b = 0; b < bands; ++b) {
-                const int y0 = static_cast<int>(static_cast<long long>(ny) * b / bands);
-                const int y1 = static_cast<int>(static_cast<long long>(ny) * (b + 1) / bands);
-                const size_t off = static_cast<size_t>(y0) * nx, cnt = static_cast<size_t>(y1 - y0) * nx;
-                CK(c, lbm::aux_field(c->h[i], c->d_inst + i, c->parity, f, y0, y1, scratch, f32, c->stream));
+        groups.push_back({true, want});
+    } else {
+        for (int f : want) groups.push_back({false, {f}});
+    }
+    int* const h_status = &c->h_red->status;
+    *h_status = 0;
+    auto issue = [&](const Group& g) -> int {
+        for (int b = 0; b < bands; ++b) {
+            const int y0 = static_cast<int>(static_cast<long long>(ny) * b / bands);
+            const int y1 = static_cast<int>(static_cast<long long>(ny) * (b + 1) / bands);
+            const size_t off = static_cast<size_t>(y0) * nx, cnt = static_cast<size_t>(y1 - y0) * nx;
+            void* dev[4] = {};
+            for (size_t k = 0; k < g.f.size(); ++k) dev[g.f[k]] = scratch + k * N;
+            if (g.flow)
+                CK(c, lbm::aux_flow(c->h[i], c->d_inst + i, c->parity, y0, y1, dev, f32, h_status, c->stream));
+            else
+                CK(c, lbm::aux_field(c->h[i], c->d_inst + i, c->parity, g.f[0], y0, y1, scratch, f32, h_status, c->stream));
+            cudaStream_t cs = c->stream;
+            if (bands > 1) {
+                cs = c->copy_stream;
                 CK(c, cudaEventRecord(c->band_done[b], c->stream));
-                CK(c, cudaStreamWaitEvent(c->copy_stream, c->band_done[b], 0));
-                CK(c, cudaMemcpyAsync(outs[f] + off, scratch + off, cnt * sizeof(O), cudaMemcpyDeviceToHost,
-                                      c->copy_stream));
+                CK(c, cudaStreamWaitEvent(cs, c->band_done[b], 0));
             }
-            return LBM_OK;
-        };
-        rc = issue_bands();
-        if (rc) {   // no copy into the caller's array may outlive the call
-            cudaStreamSynchronize(c->copy_stream);
+            for (size_t k = 0; k < g.f.size(); ++k)
+                CK(c, cudaMemcpyAsync(outs[g.f[k]] + off, scratch + k * N + off, cnt * sizeof(O), cudaMemcpyDeviceToHost,
+                                      cs));
+        }
+        CK(c, cudaStreamSynchronize(bands > 1 ? c->copy_stream : c->stream));   // before the next group reuses the scratch
+        return LBM_OK;
+    };
+    for (const Group& g : groups) {
+        rc = issue(g);
+        if (rc) {   // no copy into the caller's arrays may outlive the call
+            if (bands > 1) cudaStreamSynchronize(c->copy_stream);
+            cudaStreamSynchronize(c->stream);
             return rc;
         }
-        CK(c, cudaStreamSynchronize(c->copy_stream));   // before the next field reuses the scratch
     }
-    int code = LBM_OK;
-    rc = status_of(c, i, &code);
-    return rc ? rc : code;
+    if (groups.empty()) {
+        int code = LBM_OK;
+        rc = status_of(c, i, &code);
+        return rc ? rc : code;
+    }
+    return status_code(*h_status);
 }
 
 }  // namespace
@@ -1053,6 +1099,13 @@ int lbm_batch_create(lbm_ctx** out, int n, const int* nx, const int* ny, int pre
         c->owns = true;
         c->buf_bytes = c->L.total;
     }
+    void* red = nullptr;
+    if (cudaHostAlloc(&red, sizeof(lbm::Reduced), cudaHostAllocMapped) != cudaSuccess) {
+        cudaGetLastError();
+        lbm_destroy(c);
+        return LBM_ENOMEM;
+    }
+    c->h_red = static_cast<lbm::Reduced*>(red);
     if (cudaMemsetAsync(c->buf, 0, c->L.total, c->stream) != cudaSuccess || cudaStreamSynchronize(c->stream) != cudaSuccess) {
         lbm_destroy(c);
         return LBM_ECUDA;
@@ -1062,6 +1115,7 @@ int lbm_batch_create(lbm_ctx** out, int n, const int* nx, const int* ny, int pre
     c->d_status = reinterpret_cast<int*>(c->buf + c->L.status_off);
     c->d_partials = reinterpret_cast<double*>(c->buf + c->L.partials_off);
     c->d_result = reinterpret_cast<double*>(c->buf + c->L.result_off);
+    c->d_ticket = reinterpret_cast<unsigned*>(c->buf + c->L.result_off + 128);   // in the result's 256-byte slot
     c->d_scratch = reinterpret_cast<double*>(c->buf + c->L.scratch_off);
     c->d_run = c->buf + c->L.run_off;
     c->h.assign(n, Inst{});
@@ -1103,6 +1157,7 @@ void lbm_destroy(lbm_ctx* c) {
     }
     for (auto& e : c->band_done)
         if (e) cudaEventDestroy(e);
+    if (c->h_red) cudaFreeHost(c->h_red);
     if (c->owns && c->buf) cudaFree(c->buf);
     delete c;
 }
@@ -1275,11 +1330,10 @@ int lbm_batch_measure(lbm_ctx* c, int i, double cxc, double cyc, double r_in, do
     if (!c->inited[i] || !c->hp[i].set) return fail(c, LBM_EINVAL, "instance not initialised%s");
     Range range("lbm_batch_measure");
     CK(c, cudaSetDevice(c->device));
-    CK(c, lbm::aux_measure(c->h[i], c->d_inst + i, c->parity, cxc, cyc, r_in, r_out, c->d_partials, c->d_result,
-                           c->stream));
-    double s[lbm::kReduceSlots];
-    CK(c, cudaMemcpyAsync(s, c->d_result, sizeof s, cudaMemcpyDeviceToHost, c->stream));
+    CK(c, lbm::aux_measure(c->h[i], c->d_inst + i, c->parity, cxc, cyc, r_in, r_out, partial_rows(c).first,
+                           partial_rows(c).second, c->d_ticket, c->h_red, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
+    const double* s = c->h_red->v;
     const double N = static_cast<double>(c->nx[i]) * c->ny[i];
     const double p_in = s[3] > 0 ? s[1] / s[3] : NAN, rho_in = s[3] > 0 ? s[2] / s[3] : NAN;
     const double p_out = s[6] > 0 ? s[4] / s[6] : NAN, rho_out = s[6] > 0 ? s[5] / s[6] : NAN;
@@ -1287,9 +1341,7 @@ int lbm_batch_measure(lbm_ctx* c, int i, double cxc, double cyc, double r_in, do
     const double R_eq = std::sqrt(std::max(ex, 0.0) / (M_PI * (rho_in - rho_out)));
     const double vals[LBM_MEASURE_N] = {p_in, p_out, rho_in, rho_out, R_eq, s[0], s[3], s[6]};
     std::memcpy(out, vals, sizeof vals);
-    int code = LBM_OK;
-    rc = status_of(c, i, &code);
-    return rc ? rc : code;
+    return status_code(c->h_red->status);
 }
 
 int lbm_measure_pressure_jump(lbm_ctx* c, double cxc, double cyc, double r_in, double r_out, double* p_in,
@@ -1311,14 +1363,11 @@ int lbm_batch_stats(lbm_ctx* c, int i, double* out5) {
     if (!c->inited[i] || !c->hp[i].set) return fail(c, LBM_EINVAL, "instance not initialised%s");
     Range range("lbm_batch_stats");
     CK(c, cudaSetDevice(c->device));
-    CK(c, lbm::aux_stats(c->h[i], c->d_inst + i, c->parity, c->d_partials, c->d_result, c->stream));
-    double s[lbm::kReduceSlots];
-    CK(c, cudaMemcpyAsync(s, c->d_result, sizeof s, cudaMemcpyDeviceToHost, c->stream));
+    CK(c, lbm::aux_stats(c->h[i], c->d_inst + i, c->parity, partial_rows(c).first, partial_rows(c).second, c->d_ticket,
+                         c->h_red, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
-    std::memcpy(out5, s, 5 * sizeof(double));
-    int code = LBM_OK;
-    rc = status_of(c, i, &code);
-    return rc ? rc : code;
+    std::memcpy(out5, c->h_red->v, 5 * sizeof(double));
+    return status_code(c->h_red->status);
 }
 
 int lbm_stats(lbm_ctx* c, double* mass, double* mom_x, double* mom_y, double* ke, double* umax) {

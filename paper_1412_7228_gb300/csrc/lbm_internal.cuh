@@ -177,26 +177,6 @@ template <typename T> __device__ __forceinline__ const Phys<T>& phys(const Inst*
 template <> __device__ __forceinline__ const Phys<float>& phys<float>(const Inst* I) { return I->pf; }
 template <> __device__ __forceinline__ const Phys<double>& phys<double>(const Inst* I) { return I->pd; }
 
-// Pressure law (Eq. 21 / Eq. 29 / Carnahan-Starling); K scales the whole law.
-template <typename T> __device__ __forceinline__ T p_eos(const Phys<T>& P, T rho) {
-    if (P.eos == LBM_EOS_CS) {
-        T n = P.b4 * rho;
-        T q = T(1) - n;
-        T num = T(1) + n * (T(1) + n * (T(1) - n));
-        return P.K * (rho * P.RT * num / (q * q * q) - P.a * rho * rho);
-    } else if (P.eos == LBM_EOS_VDW) {
-        return P.K * (rho * P.RT / (T(1) - P.b * rho) - P.a * rho * rho);
-    } else {
-        T br = P.b * rho;
-        return P.K * (rho * P.RT / (T(1) - br) - P.aalpha * rho * rho / (T(1) + T(2) * br - br * br));
-    }
-}
-
-// Radicand of Eq. 10 with c = 1: psi^2 = 2 (p_EOS - rho/3) / G.
-template <typename T> __device__ __forceinline__ T psi_radicand(const Phys<T>& P, T rho) {
-    return P.two_over_G * (p_eos(P, rho) - rho * T(1.0 / 3.0));
-}
-
 // Division, reciprocal and square root of the fused step.  FP32 uses the
 // hardware approximations (a couple of ulp, far inside the FP32 error budget
 // of the stored populations).  FP64 refines the hardware estimates
@@ -357,20 +337,33 @@ cudaError_t aux_check_init(const void* rho, const void* ux, const void* uy, bool
                            int* bad, cudaStream_t st);
 cudaError_t aux_gather_plane(const Inst& host, const Inst* d_inst, int parity, int a, double* out,
                              cudaStream_t st);
-// field: 0 rho, 1 ux, 2 uy, 3 psi; rows [y0, y1), written at their place in
-// out (row-major, nx per row)
+// field: 0 rho, 3 psi; rows [y0, y1), written at their place in out
+// (row-major, nx per row)
+// f32out: floats, each the FP64 value rounded to nearest; *status (mapped host
+// memory): the instance's status word
 cudaError_t aux_field(const Inst& host, const Inst* d_inst, int parity, int field, int y0, int y1, void* out,
-                      bool f32out, cudaStream_t st);   // f32out: floats, each the FP64 value rounded to nearest
+                      bool f32out, int* status, cudaStream_t st);
+// rho, ux, uy, psi into out[0..3] (any may be NULL) in one pass; rows and types as above
+cudaError_t aux_flow(const Inst& host, const Inst* d_inst, int parity, int y0, int y1, void* const out[4], bool f32out,
+                     int* status, cudaStream_t st);
 // out: 4 device words (see lbm_fp64_math_check); default stream.
 cudaError_t aux_math_check(long long n, double lo, double hi, unsigned long long* out);
 // FP64 FMA throughput of the current device (see lbm_fp64_fma_rate).
 cudaError_t aux_fp64_fma_rate(int iters, cudaStream_t st, double* flops_per_s, double* seconds);
-constexpr int kReduceBlocks = 304;   // 2 CTAs per SM of a 152-SM GB300: partial sums of FP64 reductions
+constexpr int kReduceBlocks = 304;   // rows of partial sums that every context has; larger lattices use their field scratch
 constexpr int kReduceSlots = 8;
+// What a reduction returns: its sums and the instance's status word, written
+// by the device (into host memory mapped for it).
+struct Reduced {
+    double v[kReduceSlots];
+    int status;
+};
+// partials: device doubles for the partial sums of `rows` blocks
+// (kReduceSlots each); ticket: a device word that is zero between launches
 cudaError_t aux_measure(const Inst& host, const Inst* d_inst, int parity, double cx, double cy,
-                        double r_in, double r_out, double* partials, double* result,
+                        double r_in, double r_out, double* partials, int rows, unsigned* ticket, Reduced* out,
                         cudaStream_t st);
-cudaError_t aux_stats(const Inst& host, const Inst* d_inst, int parity, double* partials,
-                      double* result, cudaStream_t st);
+cudaError_t aux_stats(const Inst& host, const Inst* d_inst, int parity, double* partials, int rows, unsigned* ticket,
+                      Reduced* out, cudaStream_t st);
 
 }  // namespace lbm

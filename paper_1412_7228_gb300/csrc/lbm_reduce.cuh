@@ -1,0 +1,238 @@
+// lbm_reduce.cuh -- FP64 sums over a lattice or a field in one launch: the
+// per-block reduction, the last block's sum of the blocks' partial sums, and
+// the disc tests of the Laplace sampling.  Shared by lbm_aux.cu and
+// lbm_static.cu.
+//
+// GB300's FP64 pipe (two thread operations per clock and SM) bounds all of
+// these, so the code around the sums spends as few FP64 instructions as it
+// can: an FP64 instruction of one warp holds the pipe for 16 clocks however
+// many of its lanes carry data.
+#pragma once
+
+#include <cmath>
+
+#include "lbm_internal.cuh"
+
+namespace lbm {
+namespace {
+
+constexpr int kRedThreads = 256;   // threads per block of every reduction kernel
+
+// Sums of eight values over a warp.  A shuffle tree per value costs 8 x 5
+// FP64 additions per warp; here each exchange halves the values a lane
+// still carries (4 + 2 + 1 additions for the eight values, then two more),
+// nine in all.  The sum of slot k ends in the four lanes 4k .. 4k + 3.
+__device__ __forceinline__ double warp_sum8(const double (&v)[8]) {
+    const int lane = threadIdx.x & 31;
+    double a[4], b[2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const bool up = lane & 16;   // this half keeps slots 4..7
+        const double keep = up ? v[k + 4] : v[k], give = up ? v[k] : v[k + 4];
+        a[k] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const bool up = lane & 8;
+        const double keep = up ? a[k + 2] : a[k], give = up ? a[k] : a[k + 2];
+        b[k] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+    }
+    const bool up = lane & 4;
+    double x = (up ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, up ? b[0] : b[1], 4);
+    x += __shfl_xor_sync(0xffffffffu, x, 2);
+    return x + __shfl_xor_sync(0xffffffffu, x, 1);
+}
+
+// The blocks' sums (slot max_slot: maximum; -1: none) of v over all threads
+// of the grid, written by the last block to finish: every block stores its
+// eight partial sums and draws a ticket; the block that draws the last one
+// adds the partial sums in an order fixed by the grid alone, so the result
+// does not depend on which block that is.  Returns true in threads 0..7 of
+// the last block only, with slot threadIdx.x in *total; *ticket is back at
+// zero for the next launch on the stream.  vmax: the maximum's candidate of
+// this thread when max_slot >= 0 (its own v entry is ignored).
+//
+// The former second launch (one warp adding 304 rows one after another)
+// took 45 us by itself; here the last block's 32 groups of 8 threads take
+// the rows in turn.
+__device__ __forceinline__ bool grid_sum8(const double (&v)[8], int max_slot, double vmax, double* partials,
+                                          unsigned* ticket, double* total) {
+    constexpr int kWarps = kRedThreads / 32, kGroups = kRedThreads / 8;
+    __shared__ double red[kWarps][8];
+    __shared__ unsigned s_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const double x = warp_sum8(v);
+    if ((lane & 3) == 0) red[warp][lane >> 2] = x;
+    if (max_slot >= 0) {
+        double m = vmax;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        __syncwarp();
+        if (lane == 0) red[warp][max_slot] = m;
+    }
+    __syncthreads();
+    auto add = [&](double a, double b, int slot) { return slot == max_slot ? fmax(a, b) : a + b; };
+    if (tid < 8) {
+        double s = red[0][tid];
+        for (int w = 1; w < kWarps; ++w) s = add(s, red[w][tid], tid);
+        partials[blockIdx.x * 8 + tid] = s;
+        __threadfence();   // before the ticket: whoever draws the last one sees this block's row
+    }
+    __syncwarp();          // threads 0..7 are all of the writers, in warp 0
+    if (tid == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return false;
+    __threadfence();
+    const int slot = tid & 7, group = tid >> 3, n = static_cast<int>(gridDim.x);
+    double s = slot == max_slot ? -INFINITY : 0.0;
+    for (int b = group; b < n; b += kGroups) s = add(s, __ldcg(partials + b * 8 + slot), slot);
+    s = add(s, __shfl_xor_sync(0xffffffffu, s, 8), slot);
+    s = add(s, __shfl_xor_sync(0xffffffffu, s, 16), slot);
+    __syncthreads();       // red is read no more
+    if (lane < 8) red[warp][lane] = s;
+    __syncthreads();
+    if (tid == 0) *ticket = 0;
+    if (tid >= 8) return false;
+    double t = red[0][tid];
+    for (int w = 1; w < kWarps; ++w) t = add(t, red[w][tid], tid);
+    *total = t;
+    return true;
+}
+
+// The Laplace discs around (cx, cy), prepared on the host: a node at
+// distance d (periodic minimum image) is inside for d <= r_in and outside
+// for d >= r_out, tested on d^2 against in2, the largest number whose
+// correctly rounded square root is <= r_in, and out2, the smallest whose
+// root is >= r_out.  Square roots are monotone, so the tests decide as
+// those on d = sqrt(d^2) do, without the root.  A centre that is not finite
+// puts no node in either (every d is NaN).
+struct Discs {
+    double cx, cy, inv_nx, inv_ny;
+    long long in2, out2;   // bit patterns: d^2 >= 0, and such doubles order as their patterns
+};
+inline Discs make_discs(int nx, int ny, double cx, double cy, double r_in, double r_out) {
+    Discs D;
+    D.cx = cx;
+    D.cy = cy;
+    D.inv_nx = 1.0 / nx;
+    D.inv_ny = 1.0 / ny;
+    double a = r_in * r_in;
+    while (std::sqrt(a) > r_in) a = std::nextafter(a, 0.0);
+    while (std::sqrt(std::nextafter(a, INFINITY)) <= r_in && a < INFINITY) a = std::nextafter(a, INFINITY);
+    double b = r_out * r_out;
+    while (std::sqrt(b) < r_out) b = std::nextafter(b, INFINITY);
+    while (b > 0.0 && std::sqrt(std::nextafter(b, 0.0)) >= r_out) b = std::nextafter(b, 0.0);
+    if (!std::isfinite(cx) || !std::isfinite(cy)) {
+        D.cx = D.cy = 0.0;
+        D.in2 = -1;                        // no d^2 is below it
+        D.out2 = 0x7fffffffffffffffll;     // and none above this
+        return D;
+    }
+    auto bits = [](double v) {
+        long long i;
+        static_assert(sizeof i == sizeof v, "64-bit patterns");
+        __builtin_memcpy(&i, &v, sizeof i);
+        return i;
+    };
+    D.in2 = bits(a);
+    D.out2 = bits(b);
+    return D;
+}
+// Distance along one axis from the centre, minimum image, squared.  The
+// multiplication by 1/n stands for a division: where the two round apart, v
+// is half a period from the centre on either side, and the square is the same.
+__device__ __forceinline__ double axis2(int v, double c, int n, double inv_n) {
+    double d = v - c;
+    d -= n * rint(d * inv_n);
+    return d * d;
+}
+
+// The pressure law with its constants folded, p = rho [K R T h(rho) - K a rho]
+// (h = num / q^3 for Carnahan-Starling), and Eq. 10's radicand
+// (2/G)(p - rho/3) in the same form: 18 and 19 FP64 instructions instead of
+// 22 and 25.
+struct LawFp64 {
+    int eos;
+    double b, c1, c2, c3;   // p: K R T, K a (K a alpha), 0; radicand: those and 1/3, times 2/G
+    __device__ __forceinline__ LawFp64(const Phys<double>& P, bool radicand) {
+        const double s = radicand ? P.two_over_G : 1.0;
+        eos = P.eos;
+        b = P.eos == LBM_EOS_CS ? P.b4 : P.b;
+        c1 = s * (P.K * P.RT);
+        c2 = s * (P.K * (P.eos == LBM_EOS_PR ? P.aalpha : P.a));
+        c3 = radicand ? s * (1.0 / 3.0) : 0.0;
+    }
+    __device__ __forceinline__ double operator()(double rho) const {
+        const double n = b * rho, q = 1.0 - n;
+        if (eos == LBM_EOS_CS) return rho * (c1 * fma(n, fma(n, q, 1.0), 1.0) / (q * q * q) - fma(c2, rho, c3));
+        if (eos == LBM_EOS_VDW) return rho * (c1 / q - fma(c2, rho, c3));
+        return rho * (c1 / q - fma(c2, rho / fma(n, 2.0 - n, 1.0), c3));
+    }
+};
+
+// Laplace sums of one thread: {sum rho, sum p_in, sum rho_in, n_in,
+// sum p_out, sum rho_out, n_out, 0}; p = p_EOS(rho).  A node's density is
+// added once: to the disc it belongs to, or to `rest` when it belongs to
+// neither (taken off it when it belongs to both).
+struct LaplaceSums {
+    double v[8] = {0, 0, 0, 0, 0, 0, 0, 0}, rest = 0.0;
+    int n_in = 0, n_out = 0;
+    __device__ __forceinline__ void add(const LawFp64& p_eos, const Discs& D, double r, double d2) {
+        const long long b = __double_as_longlong(d2);
+        const bool in = b <= D.in2, out = b >= D.out2;
+        if (in == out) rest += in ? -r : r;
+        if (!in && !out) return;
+        const double p = p_eos(r);
+        if (in) {
+            v[1] += p;
+            v[2] += r;
+            ++n_in;
+        }
+        if (out) {
+            v[4] += p;
+            v[5] += r;
+            ++n_out;
+        }
+    }
+    __device__ __forceinline__ void close() {
+        v[0] = (v[2] + v[5]) + rest;
+        v[3] = n_in;
+        v[6] = n_out;
+    }
+};
+
+// Tiles of the Laplace sums: kTileX columns by kTileRows * rpt rows, a
+// thread taking rpt nodes of one column.
+constexpr int kTileX = 64, kTileRows = kRedThreads / kTileX, kMaxRpt = 8;
+inline long long tile_count(int nx, int ny, int rpt) {
+    return static_cast<long long>((nx + kTileX - 1) / kTileX) * ((ny + rpt * kTileRows - 1) / (rpt * kTileRows));
+}
+// Rows per thread: as many as leave two tiles per SM.  The distance along x
+// and the block's reduction are then paid once for them.
+inline int tile_rpt(int nx, int ny) {
+    int rpt = 1;
+    while (rpt < kMaxRpt && tile_count(nx, ny, 2 * rpt) >= kReduceBlocks) rpt *= 2;
+    return rpt;
+}
+// The sums over the tiles of this block; rho_at(x, y) gives a node's density.
+// dy2 (kTileRows * kMaxRpt doubles of shared memory): the squared distances
+// along y of a tile's rows, formed once per tile.
+template <typename F>
+__device__ __forceinline__ void laplace_tiles(LaplaceSums& L, const LawFp64& p_eos, const Discs& D, int nx, int ny,
+                                              int rpt, double* dy2, F rho_at) {
+    const int rows = kTileRows * rpt, tx = threadIdx.x % kTileX, ty = threadIdx.x / kTileX;
+    const int tiles_x = (nx + kTileX - 1) / kTileX, tiles = tiles_x * ((ny + rows - 1) / rows);
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int row = t / tiles_x, x = (t - row * tiles_x) * kTileX + tx, y0 = row * rows;
+        __syncthreads();   // the tile before is done with dy2
+        if (static_cast<int>(threadIdx.x) < rows) dy2[threadIdx.x] = axis2(y0 + threadIdx.x, D.cy, ny, D.inv_ny);
+        __syncthreads();
+        if (x >= nx) continue;
+        const double dx2 = axis2(x, D.cx, nx, D.inv_nx);
+        for (int k = ty; k < rows && y0 + k < ny; k += kTileRows) L.add(p_eos, D, rho_at(x, y0 + k), dx2 + dy2[k]);
+    }
+    L.close();
+}
+
+}  // namespace
+}  // namespace lbm
