@@ -673,11 +673,10 @@ int sync_all(lbm_ctx* c) {
 }
 
 // n steps of a lattice held in one cluster's shared memory (schedule 4):
-// one launch, then the ghost cells of the time level it wrote last.
+// one launch, which also writes the ghost cells of the last time level.
 int cluster_steps(lbm_ctx* c, int n) {
     if (n <= 0) return LBM_OK;
     CK(c, lbm::cluster_run(c->h[0], c->parity, n, c->stream));
-    CK(c, lbm::aux_fill_ghosts(c->h[0], c->d_inst, c->parity ^ (n & 1), c->stream));
     c->parity ^= (n & 1);
     c->steps += n;
     c->launches += 1;

@@ -12,16 +12,16 @@
 //   2. collides and streams every owned node into the output box (the same
 //      collide_rows, with the output addressed into shared memory);
 //   3. writes the periodic images of the output's edge columns (x) into its
-//      halo columns, and stores its first two output rows into the bottom
-//      halo rows of the CTA above it and its last two into the top halo rows
-//      of the CTA below it (periodic in y through the cluster ranks), in
-//      their shared memory (distributed shared memory of the cluster);
+//      halo columns, then stores its first two output rows (images included)
+//      into the bottom halo rows of the CTA above it and its last two into
+//      the top halo rows of the CTA below it (periodic in y through the
+//      cluster ranks), in their shared memory (distributed shared memory of
+//      the cluster), 16 bytes per store;
 //   4. waits at a cluster barrier, after which every output box is complete.
 // The per-node arithmetic is that of the one-step kernels on the same box
 // contents, so every schedule gives the same bits.  Nothing goes to global
 // memory between steps: the populations are read once at the start and
-// written once at the end (their ghost cells are then refilled by the
-// caller).  No wait in this kernel spins in software: the cluster barrier
+// written once at the end, ghost cells included.  No wait in this kernel spins in software: the cluster barrier
 // is the hardware's, every CTA of the cluster runs the same number of steps
 // and none leaves early, and a CTA's shared memory is only written by the
 // others between two barriers that it takes part in.
@@ -55,11 +55,20 @@ __device__ __forceinline__ uint32_t cluster_map(uint32_t addr, unsigned rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void st_cluster(uint32_t addr, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster(uint32_t addr, double v) {
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
+// 16 bytes: four floats or two doubles.
+template <typename T> struct Vec;
+template <> struct Vec<float> {
+    using type = float4;
+    static constexpr int N = 4;
+};
+template <> struct Vec<double> {
+    using type = double2;
+    static constexpr int N = 2;
+};
+template <typename V> __device__ __forceinline__ void st_cluster16(uint32_t addr, const V& v) {
+    const uint4 w = reinterpret_cast<const uint4&>(v);
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(w.x), "r"(w.y), "r"(w.z), "r"(w.w)
+                 : "memory");
 }
 
 template <typename T> struct ClusterArgs {
@@ -91,18 +100,29 @@ __global__ void __launch_bounds__(NT, 1) k_cluster(const __grid_constant__ Clust
     const int h_up = up == C - 1 ? h_last : BY;           // rows of the strip above
     const Phys<T>& P = a.P;
     const int interact = P.interact;
-    const bool fast = interact && !P.var_visc && nx == BX && h == BY;
+    const int path = !interact ? kGeneral : (P.var_visc ? kVisc : (nx == BX && h == BY ? kFast : kRagged));
     const EosRegs<T> E(P);
     const T rho_ref = P.rho_ref;
-    const int wcols = nx + 4;                             // columns -2 .. nx + 1 carry data
+    // rows move as 16-byte vectors from column -V on, one row of one plane per
+    // warp: columns -2 .. nx + 1 carry data
+    using Vt = typename Vec<T>::type;
+    constexpr int V = Vec<T>::N, kWarps = NT / 32;
+    static_assert(HX == V, "a box row starts one vector before its node 0");
+    const int nv = (nx + 2 + V - 1) / V + 1, lane = tid & 31, warp = tid >> 5;
 
     // the input box of the first step: rows y0 - 2 .. y0 + h + 1 and columns
     // -2 .. nx + 1 of the global array (its ghost cells are current)
-    for (int e = tid; e < 9 * (h + 4) * wcols; e += NT) {
-        const int c = e % wcols, r = (e / wcols) % (h + 4), q = e / (wcols * (h + 4));
-        box0[q * PB + r * WB + (HX - 2 + c)] =
-            a.src[q * a.plane + static_cast<long long>(y0 - GY + r + GY) * a.pitch + (GXg - 2 + c)];
+    for (int k = warp; k < 9 * (h + 4); k += kWarps) {
+        const int r = k / 9, q = k - 9 * r;
+        const T* const g = a.src + q * a.plane + static_cast<long long>(y0 + r) * a.pitch + (GXg - V);
+        T* const o = box0 + q * PB + r * WB;
+        for (int v = lane; v < nv; v += 32)   // all of them in flight at once
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(o + v * V)), "l"(g + v * V)
+                         : "memory");
     }
+    // the other box's padding columns travel with its rows: zeros, as in the global arrays
+    for (int e = tid; e < 9 * PB / V; e += NT) reinterpret_cast<uint4*>(box1)[e] = make_uint4(0, 0, 0, 0);
+    asm volatile("cp.async.wait_all;" ::: "memory");
     cluster_barrier();   // also: every CTA of the cluster has started before any remote store
 
     bool bad = false;
@@ -110,51 +130,81 @@ __global__ void __launch_bounds__(NT, 1) k_cluster(const __grid_constant__ Clust
     for (int s = 0; s < a.nsteps; ++s) {
         const T* bi = (s & 1) ? box1 : box0;
         T* bo = (s & 1) ? box0 : box1;
-        if (interact) ring_dispatch<Gm>(fast, P.eos, bi, sp, E, rho_ref, tid, tx, ty);
+        if (interact) ring_dispatch<Gm, true>(true, P.eos, bi, sp, E, rho_ref, tid, tx, ty);
         __syncthreads();
         // the output of node (x, y) of the strip goes to box row GY + y,
         // column HX + x: collide_rows addresses (y + GY) * pitch + x + GX
         const Regs<T> R(P);
         T* const o = bo - (Gm::GX - HX);
-        if (fast)
-            bad |= collide_rows<Gm, true, false>(bi, sp, P, R, o, PB, WB, 0, 0, nx, h, false, interact, tx, ty);
+        if (path == kFast)
+            bad |= collide_rows<Gm, kFast, false>(bi, sp, P, R, o, PB, WB, 0, 0, nx, h, false, true, tx, ty);
+        else if (path == kRagged)
+            bad |= collide_rows<Gm, kRagged, false>(bi, sp, P, R, o, PB, WB, 0, 0, nx, h, false, true, tx, ty);
+        else if (path == kVisc)
+            bad |= collide_rows<Gm, kVisc, false>(bi, sp, P, R, o, PB, WB, 0, 0, nx, h, false, true, tx, ty);
         else
-            bad |= collide_rows<Gm, false, false>(bi, sp, P, R, o, PB, WB, 0, 0, nx, h, false, interact, tx, ty);
+            bad |= collide_rows<Gm, kGeneral, false>(bi, sp, P, R, o, PB, WB, 0, 0, nx, h, false, false, tx, ty);
         __syncthreads();
-        // from the collision's outputs only, so neither waits for the other:
         // periodic images in x (columns -2, -1 <- nx - 2, nx - 1; nx, nx + 1
-        // <- 0, 1), one thread per (column, row); and the edge rows (their x
-        // images read at the source) to the neighbours' halo rows, thread
-        // row k < 4: rows GY, GY + 1 to rows GY + h_up, GY + h_up + 1 of the
-        // CTA above, rows GY + h - 2, GY + h - 1 to rows 0, 1 of the CTA below
-        if (tx < 4 && ty < h) {
-            const int to = tx < 2 ? tx - 2 : nx + tx - 2;
-            const int from = tx < 2 ? nx + tx - 2 : tx - 2;
-            T* row = bo + (GY + ty) * WB + HX;
-#pragma unroll
-            for (int q = 0; q < 9; ++q) row[q * PB + to] = row[q * PB + from];
+        // <- 0, 1), one (row, plane, column) per thread
+        for (int k = tid; k < 36 * h; k += NT) {
+            const int r = k / 36, e = k - 36 * r, j = e & 3;
+            T* const row = bo + (e >> 2) * PB + (GY + r) * WB + HX;
+            row[j < 2 ? j - 2 : nx + j - 2] = row[j < 2 ? nx + j - 2 : j - 2];
         }
-        if (ty < 4) {
-            const int from = ty < 2 ? GY + ty : GY + h - 4 + ty;
-            const int to = ty < 2 ? GY + h_up + ty : ty - 2;
-            const uint32_t rbase = cluster_map(smem_u32(bo), ty < 2 ? up : down);
-            for (int c = tx; c < wcols; c += BX) {
-                const int x = c - 2, xs = x < 0 ? x + nx : (x >= nx ? x - nx : x);
+        __syncthreads();
+        // the edge rows with their images to the neighbours' halo rows, one
+        // (row k < 4, plane) per warp: rows GY, GY + 1 to rows GY + h_up, GY +
+        // h_up + 1 of the CTA above, rows GY + h - 2, GY + h - 1 to rows 0, 1 of
+        // the CTA below.  (A lane that forms an image itself makes its whole
+        // warp wait for the gather: 1290 clocks per step instead of 350.)
+        auto edge_row = [&](int k, const T*& from, uint32_t& to) {
+            const int row = k / 9, q = k - 9 * row;
+            from = bo + q * PB + (row < 2 ? GY + row : GY + h - 4 + row) * WB;
+            to = cluster_map(smem_u32(bo + q * PB + (row < 2 ? GY + h_up + row : row - 2) * WB), row < 2 ? up : down);
+        };
+        if (lane < nv) {
+            constexpr int kPairs = (36 + kWarps - 1) / kWarps;   // loaded together, then sent
+            Vt w[kPairs];
+            uint32_t to[kPairs];
 #pragma unroll
-                for (int q = 0; q < 9; ++q)
-                    st_cluster(rbase + static_cast<uint32_t>((q * PB + to * WB + HX + x) * sizeof(T)),
-                               bo[q * PB + from * WB + HX + xs]);
+            for (int i = 0; i < kPairs; ++i) {
+                const T* from;
+                if (warp + i * kWarps < 36) {
+                    edge_row(warp + i * kWarps, from, to[i]);
+                    w[i] = *reinterpret_cast<const Vt*>(from + lane * V);
+                }
             }
+#pragma unroll
+            for (int i = 0; i < kPairs; ++i)
+                if (warp + i * kWarps < 36) st_cluster16(to[i] + lane * 16u, w[i]);
+        }
+        const int rest = nv - 32;   // vectors beyond the lanes: few, one per thread
+        for (int k = tid; k < 36 * rest; k += NT) {
+            const T* from;
+            uint32_t to;
+            const int v = 32 + k / 36;
+            edge_row(k % 36, from, to);
+            st_cluster16(to + v * 16u, *reinterpret_cast<const Vt*>(from + v * V));
         }
         cluster_barrier();
     }
 
-    // the last output box's strip to the global array (ghost cells: the caller)
+    // the last output box's strip to the global array, with its ghost cells:
+    // the strip's rows carry their x images, and the lattice's first and last
+    // two rows also go to the ghost rows opposite
     const T* fin = (a.nsteps & 1) ? box1 : box0;
-    for (int e = tid; e < 9 * h * nx; e += NT) {
-        const int x = e % nx, r = (e / nx) % h, q = e / (nx * h);
-        a.dst[q * a.plane + static_cast<long long>(y0 + r + GY) * a.pitch + (GXg + x)] =
-            fin[q * PB + (GY + r) * WB + HX + x];
+    const long long wrap = static_cast<long long>(ny) * a.pitch;
+    for (int k = warp; k < 9 * h; k += kWarps) {
+        const int r = k / 9, q = k - 9 * r, y = y0 + r;
+        const T* const g = fin + q * PB + (GY + r) * WB;
+        T* const d = a.dst + q * a.plane + static_cast<long long>(y + GY) * a.pitch + (GXg - V);
+        for (int v = lane; v < nv; v += 32) {
+            const Vt w = *reinterpret_cast<const Vt*>(g + v * V);
+            *reinterpret_cast<Vt*>(d + v * V) = w;
+            if (y < 2) *reinterpret_cast<Vt*>(d + wrap + v * V) = w;
+            if (y >= ny - 2) *reinterpret_cast<Vt*>(d - wrap + v * V) = w;
+        }
     }
     if (__syncthreads_or(bad) && tid == 0) atomicOr(a.status, ST_UNSTABLE);
 }
@@ -169,11 +219,8 @@ template <typename T, int BX, int BY, int NT> struct ClusterCfg {
         const int C = (ny + BY - 1) / BY;
         return nx >= 2 && nx <= BX && C <= max_ctas && ny - (C - 1) * BY >= 2;
     }
-    // the launch of one cluster of C CTAs (attributes set on the kernel first)
-    static cudaError_t config(unsigned C, cudaStream_t st, cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr) {
-        const auto fn = &k_cluster<T, BX, BY, NT>;
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    // the launch of one cluster of C CTAs
+    static void config(unsigned C, cudaStream_t st, cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr) {
         cfg = {};
         cfg.gridDim = dim3(C);
         cfg.blockDim = dim3(NT);
@@ -185,30 +232,39 @@ template <typename T, int BX, int BY, int NT> struct ClusterCfg {
         attr.val.clusterDim.z = 1;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        return e;
     }
-    // whether the device can hold a cluster of this lattice's CTAs at all
+    // whether the device can hold a cluster of this lattice's CTAs at all; sets
+    // the kernel's attributes, which every later launch on the device needs
     static bool launchable(int ny) {
+        const auto fn = &k_cluster<T, BX, BY, NT>;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess ||
+            cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+            return false;
         const unsigned C = static_cast<unsigned>((ny + BY - 1) / BY);
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr;
         int n = 0;
-        if (config(C, nullptr, cfg, attr) != cudaSuccess) return false;
+        config(C, nullptr, cfg, attr);
         return cudaOccupancyMaxActiveClusters(&n, &k_cluster<T, BX, BY, NT>, &cfg) == cudaSuccess && n > 0;
     }
     static cudaError_t run(const ClusterArgs<T>& args, cudaStream_t st) {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr;
-        cudaError_t e = config(static_cast<unsigned>((args.ny + BY - 1) / BY), st, cfg, attr);
-        if (e != cudaSuccess) return e;
+        config(static_cast<unsigned>((args.ny + BY - 1) / BY), st, cfg, attr);
         return cudaLaunchKernelEx(&cfg, &k_cluster<T, BX, BY, NT>, args);
     }
 };
 
-// One node per thread.  FP32: strips of 16 rows up to 64 nodes wide, or of
-// 8 rows up to 128 wide; FP64, bound by its FP64 pipe, on as many SMs as a
-// cluster has: strips of 4 rows up to 64 high, else of 8 rows, up to 64
-// nodes wide.
+// One node per thread.  FP32, up to 64 nodes wide: strips of 4 rows up to 64
+// high, of 8 up to 128, else of 16, so that a small lattice is spread over as
+// many SMs as a cluster may have (64^2: 16 CTAs of 256 threads 1.41 us per
+// step, four CTAs of 1024 threads 2.85 us; 64 x 100: 1.63 and 2.85); up to
+// 128 wide: strips of 8 rows.  FP64, bound by its FP64 pipe, likewise: 4 rows
+// up to 64 high, else 8, up to 64 nodes wide.  Clocks of a 64^2 FP32 step:
+// psi ring 610, collision 590, images and edge rows 590, cluster barrier with
+// the remote stores' arrival 1000.
+using CF32s = ClusterCfg<float, 64, 4, 256>;
+using CF32m = ClusterCfg<float, 64, 8, 512>;
 using CF32a = ClusterCfg<float, 64, 16, 1024>;
 using CF32b = ClusterCfg<float, 128, 8, 1024>;
 using CF64a = ClusterCfg<double, 64, 4, 256>;
@@ -233,6 +289,8 @@ ClusterArgs<T> cluster_args(const Inst& h, const Phys<T>& P, int parity, int nst
 
 bool cluster_supported(int prec, int nx, int ny) {
     if (prec == LBM_FP32) {
+        if (CF32s::fits(nx, ny)) return CF32s::launchable(ny);
+        if (CF32m::fits(nx, ny)) return CF32m::launchable(ny);
         if (CF32a::fits(nx, ny)) return CF32a::launchable(ny);
         return CF32b::fits(nx, ny) && CF32b::launchable(ny);
     }
@@ -244,6 +302,8 @@ cudaError_t cluster_run(const Inst& h, int parity, int nsteps, cudaStream_t st) 
     if (nsteps <= 0) return cudaSuccess;
     if (h.prec == LBM_FP32) {
         const ClusterArgs<float> a = cluster_args<float>(h, h.pf, parity, nsteps);
+        if (CF32s::fits(h.nx, h.ny)) return CF32s::run(a, st);
+        if (CF32m::fits(h.nx, h.ny)) return CF32m::run(a, st);
         if (CF32a::fits(h.nx, h.ny)) return CF32a::run(a, st);
         if (CF32b::fits(h.nx, h.ny)) return CF32b::run(a, st);
         return cudaErrorInvalidValue;

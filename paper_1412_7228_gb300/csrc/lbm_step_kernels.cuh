@@ -299,7 +299,8 @@ __device__ __forceinline__ const Phys<double>& phys_of(const BatchArgs<double>&,
 // (square root), which reaches every output of the owned node (F and Q are
 // linear in psi, 0 x NaN is NaN): the collision's NaN check records it.
 // Ring nodes beyond the lattice's ghost images feed no owned node.
-template <typename Gm, int EOSK, typename T>
+// MERGE: unrolled row passes, the extra columns in the last one's idle threads.
+template <typename Gm, int EOSK, bool MERGE, typename T>
 __device__ __forceinline__ void psi_ring(const T* sf, T* sp, const EosRegs<T>& E, T rho_ref, int tid, int tx,
                                          int ty) {
     constexpr int BX = Gm::BX;
@@ -321,14 +322,14 @@ __device__ __forceinline__ void psi_ring(const T* sf, T* sp, const EosRegs<T>& E
         }
         sp[j * Gm::WP + i] = psi;
     };
-    // rows ty, ty + TY, ... (unrolled where a thread owns several rows; the
-    // one-row shapes run under a tighter register bound); the two right-hand
-    // ring columns go to the threads the last row pass leaves idle when there
-    // are enough, so that no warp evaluates more ring nodes than the busiest
-    // row pass gives it
+    // rows ty, ty + TY, ... (unrolled where a thread owns several rows and in
+    // the cluster kernel; the one-step kernels' one-row shapes run under a
+    // tighter register bound); the two right-hand ring columns go to the
+    // threads the last row pass leaves idle when there are enough, so that no
+    // warp evaluates more ring nodes than the busiest row pass gives it
     constexpr int K = (Gm::HP + Gm::TY - 1) / Gm::TY;
-    constexpr bool kMerge = Gm::ROWS > 1 && (K * Gm::TY - Gm::HP) * BX >= 2 * Gm::HP;
-    if constexpr (Gm::ROWS > 1) {
+    constexpr bool kMerge = MERGE && (K * Gm::TY - Gm::HP) * BX >= 2 * Gm::HP;
+    if constexpr (MERGE) {
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const int j = ty + k * Gm::TY;
@@ -346,17 +347,26 @@ __device__ __forceinline__ void psi_ring(const T* sf, T* sp, const EosRegs<T>& E
         for (int e = tid; e < 2 * Gm::HP; e += Gm::NT) ring(BX + (e & 1), e >> 1);
 }
 
+// The code path of a tile, chosen once per tile from uniform values.  kFast:
+// every node inside the lattice, G != 0 and fixed shear rates (no checks per
+// node).  kGeneral: bounds, G = 0 and the viscosity law checked per node.
+// kRagged and kVisc: bounds checked, G != 0, and fixed shear rates or the
+// viscosity law, for the cluster kernel (120^2, Peng-Robinson, with the law:
+// 3.64 -> 2.84 us per step); the one-step kernels lose more to the larger
+// code (4096^2 187.0 -> 189.7 us, 256^2 3.80 -> 4.22 us) than their few such
+// tiles gain.  All compute the same bits.
+enum Path { kFast, kRagged, kVisc, kGeneral };
+
 // Force, modifying tensor, collision and store of the thread's ROWS nodes
 // (consecutive rows of column tx).  Returns true when a node's results are
-// NaN.  FAST: every node of the tile lies inside the lattice (no bounds
-// checks), G != 0 and the shear rates are fixed; GHOST: the tile is within
-// two rows or columns of the lattice's edge, so its nodes there also write
-// their periodic images.  Both are decided once per tile.
-template <typename Gm, bool FAST, bool GHOST, typename T, typename RP>
+// NaN.  GHOST: the tile is within two rows or columns of the lattice's edge,
+// so its nodes there also write their periodic images; decided once per tile
+// as PATH is.
+template <typename Gm, int PATH, bool GHOST, typename T, typename RP>
 __device__ __forceinline__ bool collide_rows(const T* sf, const T* sp, const Phys<T>& P, const RP& R, T* __restrict__ dst,
                                              long long plane, int pitch, int x0, int y0, int nx, int ny, bool border,
                                              bool interact_rt, int tx, int ty) {
-    const bool interact = FAST || interact_rt;
+    const bool interact = PATH != kGeneral || interact_rt;
     // periodic images in the ghost cells read by the neighbouring tiles
     auto ghost = [&](T* o, int x, int y, const T (&v)[9]) {
         const bool xl = x < 2, xr = x >= nx - 2, yl = y < 2, yr = y >= ny - 2;
@@ -422,7 +432,7 @@ __device__ __forceinline__ bool collide_rows(const T* sf, const T* sp, const Phy
                 qp2 = mul_rn(wp2, wp2);
             }
         }
-        if (FAST || (x < nx && y < ny)) {
+        if (PATH == kFast || (x < nx && y < ny)) {
             const T* q = sf + (ly + GY) * Gm::WB + (tx + Gm::HX);
             T f[9];
 #pragma unroll
@@ -446,7 +456,7 @@ __device__ __forceinline__ bool collide_rows(const T* sf, const T* sp, const Phy
             }
 
             T out[9];
-            collide<T, !FAST>(R, f, Fx, Fy, Qxx, Qyy, Qxy, out);
+            collide<T, (PATH >= kVisc)>(R, f, Fx, Fy, Qxx, Qyy, Qxy, out);
             if (!(out[0] == out[0])) bad = true;
 
 #pragma unroll
@@ -461,14 +471,15 @@ __device__ __forceinline__ bool collide_rows(const T* sf, const T* sp, const Phy
     return bad;
 }
 
-// The tile's psi ring on the path chosen for it (see step_body).
-template <typename Gm, typename T>
-__device__ __forceinline__ void ring_dispatch(bool fast, int eos, const T* sf, T* sp, const EosRegs<T>& E, T rho_ref,
+// The tile's psi ring: with the law fixed at compile time (fixed), or read
+// at run time.
+template <typename Gm, bool MERGE = (Gm::ROWS > 1), typename T>
+__device__ __forceinline__ void ring_dispatch(bool fixed, int eos, const T* sf, T* sp, const EosRegs<T>& E, T rho_ref,
                                               int tid, int tx, int ty) {
-    if (fast && eos == LBM_EOS_CS) psi_ring<Gm, LBM_EOS_CS>(sf, sp, E, rho_ref, tid, tx, ty);
-    else if (fast && eos == LBM_EOS_VDW) psi_ring<Gm, LBM_EOS_VDW>(sf, sp, E, rho_ref, tid, tx, ty);
-    else if (fast && eos == LBM_EOS_PR) psi_ring<Gm, LBM_EOS_PR>(sf, sp, E, rho_ref, tid, tx, ty);
-    else psi_ring<Gm, 0>(sf, sp, E, rho_ref, tid, tx, ty);
+    if (fixed && eos == LBM_EOS_CS) psi_ring<Gm, LBM_EOS_CS, MERGE>(sf, sp, E, rho_ref, tid, tx, ty);
+    else if (fixed && eos == LBM_EOS_VDW) psi_ring<Gm, LBM_EOS_VDW, MERGE>(sf, sp, E, rho_ref, tid, tx, ty);
+    else if (fixed && eos == LBM_EOS_PR) psi_ring<Gm, LBM_EOS_PR, MERGE>(sf, sp, E, rho_ref, tid, tx, ty);
+    else psi_ring<Gm, 0, MERGE>(sf, sp, E, rho_ref, tid, tx, ty);
 }
 
 // The tile's collision and store on the path chosen for it; true when a
@@ -478,12 +489,12 @@ __device__ __forceinline__ bool collide_dispatch(bool fast, bool border, const T
                                                  const RP& R, T* dst, long long plane, int pitch, int x0, int y0,
                                                  int nx, int ny, bool interact, int tx, int ty) {
     if (fast && !border)
-        return collide_rows<Gm, true, false>(sf, sp, P, R, dst, plane, pitch, x0, y0, nx, ny, border, interact, tx,
-                                             ty);
+        return collide_rows<Gm, kFast, false>(sf, sp, P, R, dst, plane, pitch, x0, y0, nx, ny, border, interact, tx,
+                                              ty);
     if (fast)
-        return collide_rows<Gm, true, true>(sf, sp, P, R, dst, plane, pitch, x0, y0, nx, ny, border, interact, tx,
-                                            ty);
-    return collide_rows<Gm, false, true>(sf, sp, P, R, dst, plane, pitch, x0, y0, nx, ny, border, interact, tx, ty);
+        return collide_rows<Gm, kFast, true>(sf, sp, P, R, dst, plane, pitch, x0, y0, nx, ny, border, interact, tx,
+                                             ty);
+    return collide_rows<Gm, kGeneral, true>(sf, sp, P, R, dst, plane, pitch, x0, y0, nx, ny, border, interact, tx, ty);
 }
 
 // One kernel, two ways to find the work, both from a __grid_constant__
