@@ -599,7 +599,31 @@ int apply_schedule(lbm_ctx* c, int cfg, int sched) {
     return build_tiles(c);
 }
 
+inline void fill_node(lbm::NodeConsts<float>&, const HostParams&) {}
+inline void fill_node(lbm::NodeConsts<double>& N, const HostParams& hp) {
+    const double w = -hp.G / 12.0, kq = hp.G != 0.0 ? -0.5 * hp.kappa : 0.0;
+    const double s1 = hp.s[1], s2 = hp.s[2], s4 = hp.s[4], s6 = hp.s[6];
+    N.cF = w * (1.0 - hp.A);
+    N.hF = w * (0.5 * hp.A);
+    N.k1[0] = 2.0 * s1 - 4.0;
+    N.k1[1] = -1.0 - s1;
+    N.k1[2] = 2.0 - 4.0 * s1;
+    N.k1r = 3.0 * s1;
+    N.k1q = 1.5 * s1 * (2.0 * kq);
+    N.k2[0] = 4.0 - 3.0 * s2;
+    N.k2[1] = 3.0 * s2 - 2.0;
+    N.k2r = -3.0 * s2;
+    N.k2q = (hp.flags & LBM_FLAG_LI_EPS) ? -1.5 * s2 * (2.0 * kq) : 0.0;
+    N.k4[0] = s4 - 2.0;
+    N.k4[1] = 1.0 - 2.0 * s4;
+    N.k6[0] = s6 - 2.0;
+    N.k6[1] = 1.0 - 2.0 * s6;
+    N.k7q = -hp.s[7] * (4.0 * kq);
+    N.k8q = -hp.s[8] * kq;
+}
+
 template <typename T> void fill_phys(lbm::Phys<T>& P, const HostParams& hp) {
+    fill_node(P, hp);
     lbm::fill_eos(P, hp.eos);
     P.flags = hp.flags;
     P.A = T(hp.A);

@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(NT, 1) k_cluster(const __grid_constant__ Clust
     for (int s = 0; s < a.nsteps; ++s) {
         const T* bi = (s & 1) ? box1 : box0;
         T* bo = (s & 1) ? box0 : box1;
-        if (interact) ring_dispatch<Gm, true>(true, P.eos, bi, sp, E, rho_ref, tid, tx, ty);
+        if (interact) ring_dispatch<Gm, true>(true, P, bi, sp, E, rho_ref, tid, tx, ty);
         __syncthreads();
         // the output of node (x, y) of the strip goes to box row GY + y,
         // column HX + x: collide_rows addresses (y + GY) * pitch + x + GX

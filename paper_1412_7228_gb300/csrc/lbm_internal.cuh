@@ -40,8 +40,19 @@ __host__ __device__ constexpr int cy(int a) {
 constexpr int ST_UNSTABLE = 1;
 constexpr int ST_TIMEOUT = 2;
 
+// Constants of the FP64 node (collide64 in lbm_step_kernels.cuh), formed once
+// on the host.
+template <typename T> struct NodeConsts {};
+template <> struct NodeConsts<double> {
+    double cF, hF;               // -(G/12) (1 - A), -(G/12) A/2
+    double k1[3], k1r, k1q;      // e*: f_0, axis sum, diagonal sum; rho|v|^2; tr Q's sum
+    double k2[2], k2r, k2q;      // eps*: f_0, axis sum (diagonal sum: 1); likewise
+    double k4[2], k6[2];         // q_x*, q_y*: axis and diagonal fluxes
+    double k7q, k8q;             // p_xx*, p_xy*: the sums of Q_xx - Q_yy and Q_xy
+};
+
 // Physics parameters in the kernel's precision.
-template <typename T> struct Phys {
+template <typename T> struct Phys : NodeConsts<T> {
     int eos;            // LBM_EOS_*
     unsigned flags;     // LBM_FLAG_*
     T K, a, b, b4, RT, aalpha;   // EOS; b4 = b/4 (CS), aalpha = a alpha(T) (PR)
@@ -180,9 +191,9 @@ template <> __device__ __forceinline__ const Phys<double>& phys<double>(const In
 // Division, reciprocal and square root of the fused step.  FP32 uses the
 // hardware approximations (a couple of ulp, far inside the FP32 error budget
 // of the stored populations).  FP64 refines the hardware estimates
-// (rcp.approx / rsqrt.approx, accurate to about 2^-22) with two steps of a
-// quadratically converging iteration, which leaves only the rounding of the
-// last step: 1/d by Newton-Raphson (e = 1 - d r, r <- r + r e), sqrt(x) by
+// (rcp.approx / rsqrt.approx, accurate to about 2^-22) until only the rounding
+// of the last step is left: 1/d by one third-order step (e = 1 - d r,
+// r <- r + r (e + e^2), which leaves e^3), sqrt(x) by two steps of
 // Goldschmidt's coupled iteration (g -> sqrt(x), h -> 1/(2 sqrt(x)):
 // r = 1/2 - g h, g <- g + g r, h <- h + h r).  Both stay within 1 ulp of the
 // IEEE-rounded 1/d and sqrt(x), a * rcp(d) within 1 ulp of a/d
@@ -203,10 +214,8 @@ template <> struct Fast<double> {
     static __device__ __forceinline__ double rcp(double d) {
         double r;
         asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-        double e = fma(-d, r, 1.0);
-        r = fma(r, e, r);
-        e = fma(-d, r, 1.0);
-        return fma(r, e, r);
+        const double e = fma(-d, r, 1.0);
+        return fma(r, fma(e, e, e), r);
     }
     static __device__ __forceinline__ double div(double a, double b) { return a * rcp(b); }
     static __device__ __forceinline__ double sqrt(double x) {

@@ -42,7 +42,12 @@ template <typename T, int BX_, int BY_, int NT_, int NBUF_> struct Geom {
     static constexpr size_t box_bytes = size_t(9) * PB * sizeof(T);
     static constexpr size_t buf_stride = (box_bytes + 127) / 128 * 128;      // box buffers
     static constexpr size_t psi_off = NBUF * buf_stride;
-    static constexpr size_t psi_stride = (size_t(WP) * HP * sizeof(T) + 127) / 128 * 128;   // psi tiles
+    static constexpr size_t psi_bytes = size_t(WP) * HP * sizeof(T);
+    // FP64 also keeps each ring node's share of Eq. 9's psi^2 term (see
+    // psi_ring), unless two CTAs would no longer fit on an SM with it
+    static constexpr bool kKeepSquares =
+        sizeof(T) == 8 && 2 * (NBUF * (buf_stride + 2 * psi_bytes + 128) + 1024) <= 233472;
+    static constexpr size_t psi_stride = ((kKeepSquares ? 2 : 1) * psi_bytes + 127) / 128 * 128;   // psi tiles
     static constexpr size_t smem = psi_off + NBUF * psi_stride;
     static_assert(NT % BX == 0 && BY % TY == 0, "thread layout must tile the block");
     static_assert(WB <= 256 && HB <= 256, "TMA box dimensions are limited to 256");
@@ -72,33 +77,32 @@ template <typename T> __device__ __forceinline__ T rho_dev(const T (&f)[9]) {
 // fma(a, a, -b*b) is not antisymmetric in a and b, a difference of two
 // rounded products is.
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
-// The parameters one node needs, copied into registers once per tile (the
-// descriptor lives in global memory, and the compiler may not keep values
-// read through it across the node loop's stores).
-// FP32 keeps them as values; FP64, bound by its FP64 pipe rather than by
-// issue slots, keeps references and spends its registers on occupancy.
-template <typename T, typename V> struct RegsOf {
-    V ns1, ns2, ns4, ns6, ns7, ns8, h6s1, nh6s2, nhs4, nhs6, h2s7, hs8, c1, c2, rho_ref;   // ns = -s, nhs = -hs
+// The parameters one FP32 node needs, copied into registers once per tile
+// (the compiler may not keep values read through the argument block across
+// the node loop's stores).  FP64, bound by its FP64 pipe rather than by
+// issue slots, reads its constants where it needs them and spends its
+// registers on occupancy.
+template <typename T> struct Regs {
+    __device__ __forceinline__ explicit Regs(const Phys<T>&) {}
+};
+template <> struct Regs<float> {
+    float ns1, ns2, ns4, ns6, ns7, ns8, h6s1, nh6s2, nhs4, nhs6, h2s7, hs8, c1, c2, rho_ref;   // ns = -s, nhs = -hs
     int var_visc;
-    V nu_g, dnu, visc_rho_g, visc_inv_drho;
-    __device__ __forceinline__ explicit RegsOf(const Phys<T>& P)
+    float nu_g, dnu, visc_rho_g, visc_inv_drho;
+    __device__ __forceinline__ explicit Regs(const Phys<float>& P)
         : ns1(P.ns[1]), ns2(P.ns[2]), ns4(P.ns[4]), ns6(P.ns[6]), ns7(P.ns[7]), ns8(P.ns[8]), h6s1(P.h6s1),
           nh6s2(P.nh6s2), nhs4(P.nhs[4]), nhs6(P.nhs[6]), h2s7(P.h2s7), hs8(P.hs[8]), c1(P.c1), c2(P.c2),
           rho_ref(P.rho_ref), var_visc(P.var_visc), nu_g(P.nu_g), dnu(P.dnu), visc_rho_g(P.visc_rho_g),
           visc_inv_drho(P.visc_inv_drho) {}
 };
-template <typename T> struct RegsSel { using type = RegsOf<T, const T&>; };
-template <> struct RegsSel<float> { using type = RegsOf<float, float>; };
-template <typename T> using Regs = typename RegsSel<T>::type;
 
-// Moment-space collision of one node in deviation form (Eqs. 2-6, 25, 26).
+// Moment-space collision of one FP32 node in deviation form (Eqs. 2-6, 25,
+// 26); FP64: collide64.
 // Every expression maps onto itself (or its negative) under the mirrors
 // above, which keeps symmetric states symmetric to the last bit.
 // f: pre-collision f_a - t_a rho_ref; out: post-collision, same form.
-// P: the relaxation constants (register copies for FP32, references into the
-// descriptor for FP64).
+// P: the relaxation constants.
 // VISC = false: the tile's lattice has fixed shear rates (no per-node
 // viscosity law), decided once per tile by the caller.
 template <typename T, bool VISC, typename RP>
@@ -217,20 +221,19 @@ template <int EOSK, typename T> __device__ __forceinline__ T radicand_step(const
 //   Peng-Robinson      D = d e, e = 1 + 2 b rho - (b rho)^2,
 //                      W = rho [kR e - (kAa rho + k3 e) d];
 // with kR = (2/G) K R T, kA = (2/G) K a, kAa = (2/G) K a alpha(T),
-// k3 = (2/G)/3.  Then psi = W / sqrt(W D); 1/(2 sqrt(x)) comes from the
-// hardware estimate refined by two Goldschmidt steps, as in
-// Fast<double>::sqrt.  A negative radicand gives NaN (as the square root
-// does), psi(W = 0) = 0.
+// k3 = (2/G)/3.  Then psi = W / sqrt(W D); 1 / sqrt(x) comes from the hardware
+// estimate y refined by one third-order step (Householder's iteration):
+// with d = 1 - x y^2, y + y d (1/2 + 3/8 d) leaves an error of 5/16 d^3, far
+// below the last place from an estimate good to 2^-20; three FP64
+// instructions fewer than two second-order steps.  A negative radicand gives
+// NaN (as the square root does), psi(W = 0) = 0.
 __device__ __forceinline__ double psi_fold_fp64(double W, double D) {
     const double x = W * D;
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double g0 = x * y, h0 = 0.5 * y;
-    const double r0 = fma(-g0, h0, 0.5);
-    const double g1 = fma(g0, r0, g0), h1 = fma(h0, r0, h0);
-    const double r1 = fma(-g1, h1, 0.5);
-    const double h2 = fma(h1, r1, h1);
-    return W == 0.0 ? 0.0 : (W + W) * h2;
+    const double d = fma(-(x * y), y, 1.0);
+    const double r = fma(y * d, fma(d, 0.375, 0.5), y);
+    return W == 0.0 ? 0.0 : W * r;
 }
 
 template <int EOSK>
@@ -239,7 +242,7 @@ __device__ __forceinline__ double psi_fp64(const EosRegs<double>& E, double kR, 
     const int eos = EOSK ? EOSK : E.eos;
     if (eos == LBM_EOS_CS) {
         const double n = E.b4 * rho, q = 1.0 - n;
-        const double num = fma(n, fma(n, 1.0 - n, 1.0), 1.0);
+        const double num = fma(n, fma(n, q, 1.0), 1.0);   // 1 + n + n^2 - n^3
         const double q3 = q * q * q;
         return psi_fold_fp64(rho * fma(-fma(kA, rho, k3), q3, kR * num), q3);
     }
@@ -249,13 +252,12 @@ __device__ __forceinline__ double psi_fp64(const EosRegs<double>& E, double kR, 
     return psi_fold_fp64(rho * fma(-fma(kAa, rho, k3 * e), d, kR * e), d * e);
 }
 
-// Hybrid force (Eq. 9) and modifying tensor (Eq. 23, x G/2) of one node
+// Hybrid force (Eq. 9) and modifying tensor (Eq. 23, x G/2) of one FP32 node
 // from psi at the node (p0) and its eight neighbours (p_a at x + e_a).
 // The lattice sums are formed with the integer weights 12 w_a (4 on the
 // axes, 1 on the diagonals) and the common factor 1/12 is folded into the
 // constants: negGw = -G/12, kGw = kappa G/24; hA = A/2, omA = 1 - A.
-// q_a = p_a^2, rounded on their own (the caller slides them down a column
-// with the psi values, so each square is formed once).
+// q_a = p_a^2, rounded on their own.
 template <typename T>
 __device__ __forceinline__ void force_q(T negGw, T hA, T omA, T kGw, T p0, T p1, T p2, T p3, T p4, T p5, T p6,
                                         T p7, T p8, T q0, T q1, T q2, T q3, T q4, T q5, T q6, T q7, T q8, T& Fx,
@@ -298,10 +300,11 @@ __device__ __forceinline__ const Phys<double>& phys_of(const BatchArgs<double>&,
 // outside the EOS's psi domain gives a negative radicand and a NaN psi
 // (square root), which reaches every output of the owned node (F and Q are
 // linear in psi, 0 x NaN is NaN): the collision's NaN check records it.
-// Ring nodes beyond the lattice's ghost images feed no owned node.
+// Ring nodes beyond the lattice's ghost images feed no owned node.  FP64
+// (kKeepSquares): also hF psi^2, hF = -(G/12) A/2, behind the psi tile.
 // MERGE: unrolled row passes, the extra columns in the last one's idle threads.
 template <typename Gm, int EOSK, bool MERGE, typename T>
-__device__ __forceinline__ void psi_ring(const T* sf, T* sp, const EosRegs<T>& E, T rho_ref, int tid, int tx,
+__device__ __forceinline__ void psi_ring(const T* sf, T* sp, const EosRegs<T>& E, T rho_ref, T hF, int tid, int tx,
                                          int ty) {
     constexpr int BX = Gm::BX;
     // FP64: psi_fp64 on every path (the law fixed at compile time or read at
@@ -321,6 +324,7 @@ __device__ __forceinline__ void psi_ring(const T* sf, T* sp, const EosRegs<T>& E
             psi = Fast<T>::sqrt(radicand_step<EOSK>(E, rho));
         }
         sp[j * Gm::WP + i] = psi;
+        if constexpr (Gm::kKeepSquares) sp[Gm::WP * Gm::HP + j * Gm::WP + i] = (hF * psi) * psi;
     };
     // rows ty, ty + TY, ... (unrolled where a thread owns several rows and in
     // the cluster kernel; the one-step kernels' one-row shapes run under a
@@ -357,33 +361,38 @@ __device__ __forceinline__ void psi_ring(const T* sf, T* sp, const EosRegs<T>& E
 // tiles gain.  All compute the same bits.
 enum Path { kFast, kRagged, kVisc, kGeneral };
 
+// The periodic images of node (x, y), whose values v are at o, in the ghost
+// cells read by the neighbouring tiles.
+template <typename T>
+__device__ __forceinline__ void ghost_images(T* o, long long plane, int pitch, int x, int y, int nx, int ny,
+                                             const T (&v)[9]) {
+    const bool xl = x < 2, xr = x >= nx - 2, yl = y < 2, yr = y >= ny - 2;
+    if (!(xl || xr || yl || yr)) return;
+    const int oxs[3] = {0, xl ? nx : 0, xr ? -nx : 0};
+    const int oys[3] = {0, yl ? ny : 0, yr ? -ny : 0};
+    const bool hx[3] = {true, xl, xr};
+    const bool hy[3] = {true, yl, yr};
+    for (int iy = 0; iy < 3; ++iy)
+        for (int ix = 0; ix < 3; ++ix) {
+            if (!(hx[ix] && hy[iy]) || (ix == 0 && iy == 0)) continue;
+            T* g = o + static_cast<long long>(oys[iy]) * pitch + oxs[ix];
+#pragma unroll
+            for (int a = 0; a < 9; ++a) g[a * plane] = v[a];
+        }
+}
+
 // Force, modifying tensor, collision and store of the thread's ROWS nodes
 // (consecutive rows of column tx).  Returns true when a node's results are
 // NaN.  GHOST: the tile is within two rows or columns of the lattice's edge,
 // so its nodes there also write their periodic images; decided once per tile
-// as PATH is.
-template <typename Gm, int PATH, bool GHOST, typename T, typename RP>
-__device__ __forceinline__ bool collide_rows(const T* sf, const T* sp, const Phys<T>& P, const RP& R, T* __restrict__ dst,
+// as PATH is.  FP32.
+template <typename Gm, int PATH, bool GHOST, typename RP>
+__device__ __forceinline__ bool collide_rows(const float* sf, const float* sp, const Phys<float>& P, const RP& R,
+                                             float* __restrict__ dst,
                                              long long plane, int pitch, int x0, int y0, int nx, int ny, bool border,
                                              bool interact_rt, int tx, int ty) {
+    using T = float;
     const bool interact = PATH != kGeneral || interact_rt;
-    // periodic images in the ghost cells read by the neighbouring tiles
-    auto ghost = [&](T* o, int x, int y, const T (&v)[9]) {
-        const bool xl = x < 2, xr = x >= nx - 2, yl = y < 2, yr = y >= ny - 2;
-        if (!(xl || xr || yl || yr)) return;
-        const int oxs[3] = {0, xl ? nx : 0, xr ? -nx : 0};
-        const int oys[3] = {0, yl ? ny : 0, yr ? -ny : 0};
-        const bool hx[3] = {true, xl, xr};
-        const bool hy[3] = {true, yl, yr};
-        for (int iy = 0; iy < 3; ++iy)
-            for (int ix = 0; ix < 3; ++ix) {
-                if (!(hx[ix] && hy[iy]) || (ix == 0 && iy == 0)) continue;
-                T* g = o + static_cast<long long>(oys[iy]) * pitch + oxs[ix];
-#pragma unroll
-                for (int a = 0; a < 9; ++a) g[a * plane] = v[a];
-            }
-    };
-
     // each thread owns ROWS consecutive rows of one column; the 3x3 psi
     // neighbourhood slides down with it (three new loads per node)
     const T G = P.G, A = P.A;
@@ -391,12 +400,9 @@ __device__ __forceinline__ bool collide_rows(const T* sf, const T* sp, const Phy
     const T kGw = P.kappa * G * T(1.0 / 24.0);
     const int ly0 = ty * Gm::ROWS;
     const T* s0 = sp + (ly0 + 1) * Gm::WP + (tx + 1);   // psi of node (tx, ly0)
-    // FP64 slides the squares of the window too (six FP64 products fewer
-    // per node); FP32 forms them per node, which keeps it to fewer
-    // registers and measured faster
-    constexpr bool kSlideSquares = sizeof(T) == 8;
+    // the window's squares are formed per node, which keeps it to fewer
+    // registers than sliding them and measured faster
     T wm0 = T(0), wm1 = T(0), wm2 = T(0), w00 = T(0), w01 = T(0), w02 = T(0);
-    T qm0 = T(0), qm1 = T(0), qm2 = T(0), q00 = T(0), q01 = T(0), q02 = T(0);   // their squares
     if (interact) {
         wm0 = s0[-Gm::WP - 1];
         wm1 = s0[-Gm::WP];
@@ -404,14 +410,6 @@ __device__ __forceinline__ bool collide_rows(const T* sf, const T* sp, const Phy
         w00 = s0[-1];
         w01 = s0[0];
         w02 = s0[1];
-        if (kSlideSquares) {
-            qm0 = mul_rn(wm0, wm0);
-            qm1 = mul_rn(wm1, wm1);
-            qm2 = mul_rn(wm2, wm2);
-            q00 = mul_rn(w00, w00);
-            q01 = mul_rn(w01, w01);
-            q02 = mul_rn(w02, w02);
-        }
     }
 
     bool bad = false;
@@ -420,17 +418,12 @@ __device__ __forceinline__ bool collide_rows(const T* sf, const T* sp, const Phy
     for (int r = 0; r < Gm::ROWS; ++r, o += pitch) {
         const int ly = ly0 + r;
         const int x = x0 + tx, y = y0 + ly;
-        T wp0 = T(0), wp1 = T(0), wp2 = T(0), qp0 = T(0), qp1 = T(0), qp2 = T(0);
+        T wp0 = T(0), wp1 = T(0), wp2 = T(0);
         if (interact) {
             const T* sr = s0 + (r + 1) * Gm::WP;
             wp0 = sr[-1];
             wp1 = sr[0];
             wp2 = sr[1];
-            if (kSlideSquares) {
-                qp0 = mul_rn(wp0, wp0);
-                qp1 = mul_rn(wp1, wp1);
-                qp2 = mul_rn(wp2, wp2);
-            }
         }
         if (PATH == kFast || (x < nx && y < ny)) {
             const T* q = sf + (ly + GY) * Gm::WB + (tx + Gm::HX);
@@ -440,17 +433,9 @@ __device__ __forceinline__ bool collide_rows(const T* sf, const T* sp, const Phy
 
             T Fx = T(0), Fy = T(0), Qxx = T(0), Qyy = T(0), Qxy = T(0);
             if (interact) {
-                if (!kSlideSquares) {
-                    qp0 = mul_rn(wp0, wp0);
-                    qp1 = mul_rn(wp1, wp1);
-                    qp2 = mul_rn(wp2, wp2);
-                    qm0 = mul_rn(wm0, wm0);
-                    qm1 = mul_rn(wm1, wm1);
-                    qm2 = mul_rn(wm2, wm2);
-                    q00 = mul_rn(w00, w00);
-                    q01 = mul_rn(w01, w01);
-                    q02 = mul_rn(w02, w02);
-                }
+                const T qp0 = mul_rn(wp0, wp0), qp1 = mul_rn(wp1, wp1), qp2 = mul_rn(wp2, wp2);
+                const T qm0 = mul_rn(wm0, wm0), qm1 = mul_rn(wm1, wm1), qm2 = mul_rn(wm2, wm2);
+                const T q00 = mul_rn(w00, w00), q01 = mul_rn(w01, w01), q02 = mul_rn(w02, w02);
                 force_q<T>(negGw, hA, omA, kGw, w01, w02, wp1, w00, wm1, wp2, wp0, wm0, wm2, q01, q02, qp1, q00,
                            qm1, qp2, qp0, qm0, qm2, Fx, Fy, Qxx, Qyy, Qxy);
             }
@@ -461,12 +446,156 @@ __device__ __forceinline__ bool collide_rows(const T* sf, const T* sp, const Phy
 
 #pragma unroll
             for (int a = 0; a < 9; ++a) o[a * plane] = out[a];
-            if (GHOST && border) ghost(o, x, y, out);
+            if (GHOST && border) ghost_images(o, plane, pitch, x, y, nx, ny, out);
         }
         wm0 = w00; wm1 = w01; wm2 = w02;
         w00 = wp0; w01 = wp1; w02 = wp2;
-        qm0 = q00; qm1 = q01; qm2 = q02;
-        q00 = qp0; q01 = qp1; q02 = qp2;
+    }
+    return bad;
+}
+
+// ---- the FP64 node ---------------------------------------------------------
+// FP64 is bound by its pipe (19 clocks of an SM per warp instruction, an
+// addition, a product or a fused one alike), so its node is written for the
+// fewest FP64 instructions rather than for the mirror symmetry that the FP32
+// node keeps to the last bit: about 146 with the psi ring's share instead of
+// 205 (FP64, 1024^2, per step: 410 -> 289 us multi-step with 32 x 32 tiles, 447 ->
+// 315 us one-step with 32 x 8; 64^2 in a cluster 18.7 -> 13.5 us).  The method is
+// the same:
+//  - Eq. 9 and Eq. 23 are linear in g_a = -(G/12) [(1-A) psi(x) psi_a + (A/2)
+//    psi_a^2], so the nine g_a are formed first and each lattice sum once:
+//    F = sum 12 w_a g_a e_a, and Q from the same g with the factor -kappa/2
+//    (kappa (G/24) over -(G/12)), which sits in the constants of its users;
+//  - m - Lambda (m - m_eq) is expanded in the few sums it depends on:
+//    e* and eps* in f_0, the axis sum, the diagonal sum and rho|v|^2; q_x* =
+//    (s_q - 2) (f_1 - f_3) + (1 - 2 s_q) (diagonal x flux) - F_x, where the
+//    velocity's and the forcing's shares of F_x add up to -1;
+//  - the inverse transform takes its factors 1/36, 1/6 and 1/4 in fused
+//    multiply-adds.  a0 = rho/9 keeps its residual step (the node's mass).
+struct Sums64 {
+    double Fx, Fy, tr, qd, qxy;   // F; Q_xx + Q_yy, Q_xx - Q_yy, Q_xy without their constant factors
+};
+__device__ __forceinline__ Sums64 stencil64(const Phys<double>& P, double p0, double h0, double p1, double h1, double p2,
+                                            double h2, double p3, double h3, double p4, double h4, double p5, double h5,
+                                            double p6, double h6, double p7, double h7, double p8, double h8) {
+    const double c = P.cF * p0;
+    const double g0 = fma(c, p0, h0), g1 = fma(c, p1, h1), g2 = fma(c, p2, h2), g3 = fma(c, p3, h3);
+    const double g4 = fma(c, p4, h4), g5 = fma(c, p5, h5), g6 = fma(c, p6, h6), g7 = fma(c, p7, h7), g8 = fma(c, p8, h8);
+    const double a57 = g5 - g7, a86 = g8 - g6;
+    const double s13 = g1 + g3, s24 = g2 + g4, s57 = g5 + g7, s68 = g6 + g8;
+    Sums64 S;
+    S.Fx = fma(4.0, g1 - g3, a57 + a86);
+    S.Fy = fma(4.0, g2 - g4, a57 - a86);
+    S.tr = fma(2.0, s13 + s24, fma(-12.0, g0, s57 + s68));   // half of its sum
+    S.qd = s13 - s24;                                        // a quarter
+    S.qxy = s57 - s68;
+    return S;
+}
+
+template <bool VISC>
+__device__ __forceinline__ void collide64(const Phys<double>& P, const double (&f)[9], const Sums64& S, double (&out)[9]) {
+    const double ax = f[1] + f[3], ay = f[2] + f[4], b57 = f[5] + f[7], b68 = f[6] + f[8];
+    const double Sa = ax + ay, Sd = b57 + b68, rt = f[0] + Sa + Sd;
+    const double rho = P.rho_ref + rt, inv = Fast<double>::rcp(rho);
+    const double d13 = f[1] - f[3], d24 = f[2] - f[4], a57 = f[5] - f[7], a86 = f[8] - f[6];
+    const double Dx = a57 + a86, Dy = a57 - a86, jx = d13 + Dx, jy = d24 + Dy;
+    const double rux = fma(0.5, S.Fx, jx), ruy = fma(0.5, S.Fy, jy);   // rho v = j + F/2
+    const double ux = rux * inv, uy = ruy * inv;
+    const double P2 = ruy * uy, ru2 = fma(rux, ux, P2), D2 = fma(rux, ux, -P2);
+    const double V2 = uy * S.Fy, vF = fma(ux, S.Fx, V2), D1 = fma(ux, S.Fx, -V2), C1 = fma(ux, S.Fy, uy * S.Fx);
+    const double ms1 = fma(P.k1q, S.tr, fma(P.h6s1, vF, fma(P.k1r, ru2, fma(P.k1[0], f[0], fma(P.k1[1], Sa, P.k1[2] * Sd)))));
+    const double ms2 = fma(P.k2q, S.tr, fma(P.nh6s2, vF, fma(P.k2r, ru2, fma(P.k2[0], f[0], fma(P.k2[1], Sa, Sd)))));
+    double ns7 = P.ns[7], ns8 = P.ns[8], h2s7 = P.h2s7, hs8 = P.hs[8], k7q = P.k7q, k8q = P.k8q;
+    if (VISC && P.var_visc) {   // shear rates from the density-dependent viscosity (Section 4.2)
+        const double w = fmin(fmax((rho - P.visc_rho_g) * P.visc_inv_drho, 0.0), 1.0);
+        const double sn = Fast<double>::rcp(fma(3.0, fma(w, P.dnu, P.nu_g), 0.5));
+        ns7 = ns8 = -sn;
+        hs8 = fma(-0.5, sn, 1.0);
+        h2s7 = 2.0 - sn;
+        k8q = ns8 * (-0.5 * P.kappa);
+        k7q = 4.0 * k8q;
+    }
+    const double m7 = ax - ay, m8 = b57 - b68;
+    const double ms7 = fma(k7q, S.qd, fma(h2s7, D1, fma(ns7, m7 - D2, m7)));
+    const double ms8 = fma(k8q, S.qxy, fma(hs8, C1, fma(ns8, fma(-rux, uy, m8), m8)));
+    const double ms3 = jx + S.Fx, ms5 = jy + S.Fy;
+    const double ms4 = fma(P.k4[0], d13, fma(P.k4[1], Dx, -S.Fx)), ms6 = fma(P.k6[0], d24, fma(P.k6[1], Dy, -S.Fy));
+
+    constexpr double c9 = 1.0 / 9.0, c36 = 1.0 / 36.0, c6 = 1.0 / 6.0;
+    const double q9 = rt * c9, a0 = fma(fma(q9, -9.0, rt), c9, q9);
+    out[0] = fma(4.0 * c36, ms2, fma(-4.0 * c36, ms1, a0));
+    const double bax = fma(-2.0 * c36, ms2, fma(-c36, ms1, a0)), bdg = fma(c36, ms2, fma(2.0 * c36, ms1, a0));
+    const double X = ms3 - ms4, Y = ms5 - ms6, DX = fma(0.5, ms4, ms3), DY = fma(0.5, ms6, ms5);
+    const double e1 = fma(0.25, ms7, bax), e2 = fma(-0.25, ms7, bax);
+    const double e5 = fma(0.25, ms8, bdg), e6 = fma(-0.25, ms8, bdg), sm = DX + DY, df = DX - DY;
+    out[1] = fma(c6, X, e1);
+    out[3] = fma(-c6, X, e1);
+    out[2] = fma(c6, Y, e2);
+    out[4] = fma(-c6, Y, e2);
+    out[5] = fma(c6, sm, e5);
+    out[7] = fma(-c6, sm, e5);
+    out[8] = fma(c6, df, e6);
+    out[6] = fma(-c6, df, e6);
+}
+
+// collide_rows for FP64: the 3 x 3 window of psi and of hF psi^2 slides down
+// the column.
+template <typename Gm, int PATH, bool GHOST, typename RP>
+__device__ __forceinline__ bool collide_rows(const double* sf, const double* sp, const Phys<double>& P, const RP&,
+                                             double* __restrict__ dst, long long plane, int pitch, int x0, int y0,
+                                             int nx, int ny, bool border, bool interact_rt, int tx, int ty) {
+    const bool interact = PATH != kGeneral || interact_rt;
+    const int ly0 = ty * Gm::ROWS;
+    const double* s0 = sp + (ly0 + 1) * Gm::WP + (tx + 1);   // psi of node (tx, ly0)
+    const double hF = P.hF;
+    auto h_of = [&](const double* s, double p) {
+        if constexpr (Gm::kKeepSquares) return s[Gm::WP * Gm::HP];
+        else return (hF * p) * p;
+    };
+    double wm[3] = {0, 0, 0}, w0[3] = {0, 0, 0}, hm[3] = {0, 0, 0}, h0[3] = {0, 0, 0};
+    if (interact) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            wm[k] = s0[k - 1 - Gm::WP];
+            w0[k] = s0[k - 1];
+            hm[k] = h_of(s0 + k - 1 - Gm::WP, wm[k]);
+            h0[k] = h_of(s0 + k - 1, w0[k]);
+        }
+    }
+    bool bad = false;
+    double* o = dst + static_cast<long long>(y0 + ly0 + GY) * pitch + (x0 + tx + Gm::GX);
+#pragma unroll
+    for (int r = 0; r < Gm::ROWS; ++r, o += pitch) {
+        const int ly = ly0 + r, x = x0 + tx, y = y0 + ly;
+        double wp[3] = {0, 0, 0}, hp[3] = {0, 0, 0};
+        if (interact) {
+            const double* sr = s0 + (r + 1) * Gm::WP;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                wp[k] = sr[k - 1];
+                hp[k] = h_of(sr + k - 1, wp[k]);
+            }
+        }
+        if (PATH == kFast || (x < nx && y < ny)) {
+            const double* q = sf + (ly + GY) * Gm::WB + (tx + Gm::HX);
+            double f[9], out[9];
+#pragma unroll
+            for (int a = 0; a < 9; ++a) f[a] = q[a * Gm::PB - cy(a) * Gm::WB - cx(a)];
+            Sums64 S = {0.0, 0.0, 0.0, 0.0, 0.0};
+            if (interact)
+                S = stencil64(P, w0[1], h0[1], w0[2], h0[2], wp[1], hp[1], w0[0], h0[0], wm[1], hm[1], wp[2], hp[2],
+                              wp[0], hp[0], wm[0], hm[0], wm[2], hm[2]);
+            collide64<(PATH >= kVisc)>(P, f, S, out);
+            if (!(out[0] == out[0])) bad = true;
+#pragma unroll
+            for (int a = 0; a < 9; ++a) o[a * plane] = out[a];
+            if (GHOST && border) ghost_images(o, plane, pitch, x, y, nx, ny, out);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            wm[k] = w0[k]; w0[k] = wp[k];
+            hm[k] = h0[k]; h0[k] = hp[k];
+        }
     }
     return bad;
 }
@@ -474,12 +603,15 @@ __device__ __forceinline__ bool collide_rows(const T* sf, const T* sp, const Phy
 // The tile's psi ring: with the law fixed at compile time (fixed), or read
 // at run time.
 template <typename Gm, bool MERGE = (Gm::ROWS > 1), typename T>
-__device__ __forceinline__ void ring_dispatch(bool fixed, int eos, const T* sf, T* sp, const EosRegs<T>& E, T rho_ref,
-                                              int tid, int tx, int ty) {
-    if (fixed && eos == LBM_EOS_CS) psi_ring<Gm, LBM_EOS_CS, MERGE>(sf, sp, E, rho_ref, tid, tx, ty);
-    else if (fixed && eos == LBM_EOS_VDW) psi_ring<Gm, LBM_EOS_VDW, MERGE>(sf, sp, E, rho_ref, tid, tx, ty);
-    else if (fixed && eos == LBM_EOS_PR) psi_ring<Gm, LBM_EOS_PR, MERGE>(sf, sp, E, rho_ref, tid, tx, ty);
-    else psi_ring<Gm, 0, MERGE>(sf, sp, E, rho_ref, tid, tx, ty);
+__device__ __forceinline__ void ring_dispatch(bool fixed, const Phys<T>& P, const T* sf, T* sp, const EosRegs<T>& E,
+                                              T rho_ref, int tid, int tx, int ty) {
+    T hF = T(0);
+    if constexpr (Gm::kKeepSquares) hF = P.hF;
+    const int eos = P.eos;
+    if (fixed && eos == LBM_EOS_CS) psi_ring<Gm, LBM_EOS_CS, MERGE>(sf, sp, E, rho_ref, hF, tid, tx, ty);
+    else if (fixed && eos == LBM_EOS_VDW) psi_ring<Gm, LBM_EOS_VDW, MERGE>(sf, sp, E, rho_ref, hF, tid, tx, ty);
+    else if (fixed && eos == LBM_EOS_PR) psi_ring<Gm, LBM_EOS_PR, MERGE>(sf, sp, E, rho_ref, hF, tid, tx, ty);
+    else psi_ring<Gm, 0, MERGE>(sf, sp, E, rho_ref, hF, tid, tx, ty);
 }
 
 // The tile's collision and store on the path chosen for it; true when a
@@ -606,7 +738,6 @@ __device__ __forceinline__ void step_body(const Inst* __restrict__ insts, int nt
         // the fast path: every node of the tile inside the lattice, G != 0,
         // fixed shear rates
         const bool fast = interact && !P.var_visc && x0 + BX <= nx && y0 + BY <= ny;
-        const int eos = P.eos;
 
         bool ok = mbar_wait_bounded(&bar[b], ph, timeout_ns);
         if (k == 0 && (P.flags & LBM_FLAG_TEST_FORCE_TIMEOUT)) {
@@ -615,7 +746,7 @@ __device__ __forceinline__ void step_body(const Inst* __restrict__ insts, int nt
         }
 
         // ---- rho and psi of the tile and its ring (Eq. 10) ---------------
-        if (interact && ok) ring_dispatch<Gm>(fast, eos, sf, sp, E, rho_ref, tid, tx, ty);
+        if (interact && ok) ring_dispatch<Gm>(fast, P, sf, sp, E, rho_ref, tid, tx, ty);
         if (!__syncthreads_and(ok)) {
             if (tid == 0) {
                 atomicOr(status, ST_TIMEOUT);
@@ -834,7 +965,7 @@ __device__ __forceinline__ void run_body(const Inst* __restrict__ insts, unsigne
             ok = ok && mbar_wait_bounded(&bar, phase, 2000000ull);
         }
         first = false;
-        if (interact && ok) ring_dispatch<Gm>(fast, P.eos, sf, sp, E, rho_ref, tid, tx, ty);
+        if (interact && ok) ring_dispatch<Gm>(fast, P, sf, sp, E, rho_ref, tid, tx, ty);
         if (!__syncthreads_and(ok)) {
             if (tid == 0) {
                 atomicOr(status, ST_TIMEOUT);
@@ -868,7 +999,7 @@ __device__ __forceinline__ void run_body(const Inst* __restrict__ insts, unsigne
 template <typename T, bool ONE> using ArgsOf = typename std::conditional<ONE, StepArgs<T>, BatchArgs<T>>::type;
 
 template <typename T, int BX, int BY, int NT, int NBUF, bool ONE>
-__global__ void __launch_bounds__(NT) k_step(const Inst* __restrict__ insts, int ntiles, int parity,
+__global__ void __launch_bounds__(NT, 2) k_step(const Inst* __restrict__ insts, int ntiles, int parity,
                                              unsigned long long timeout_ns,
                                              const __grid_constant__ ArgsOf<T, ONE> args) {
     step_body<T, BX, BY, NT, NBUF, ONE>(insts, ntiles, parity, timeout_ns, args);
