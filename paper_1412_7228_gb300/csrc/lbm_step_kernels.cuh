@@ -326,9 +326,9 @@ __device__ __forceinline__ void psi_ring(const T* sf, T* sp, const EosRegs<T>& E
         sp[j * Gm::WP + i] = psi;
         if constexpr (Gm::kKeepSquares) sp[Gm::WP * Gm::HP + j * Gm::WP + i] = (hF * psi) * psi;
     };
-    // rows ty, ty + TY, ... (unrolled where a thread owns several rows and in
-    // the cluster kernel; the one-step kernels' one-row shapes run under a
-    // tighter register bound); the two right-hand ring columns go to the
+    // rows ty, ty + TY, ... (unrolled where a thread owns several rows, in
+    // CTAs of four warps and in the cluster kernel; the other one-row shapes
+    // run under a tighter register bound); the two right-hand ring columns go to the
     // threads the last row pass leaves idle when there are enough, so that no
     // warp evaluates more ring nodes than the busiest row pass gives it
     constexpr int K = (Gm::HP + Gm::TY - 1) / Gm::TY;
@@ -602,7 +602,7 @@ __device__ __forceinline__ bool collide_rows(const double* sf, const double* sp,
 
 // The tile's psi ring: with the law fixed at compile time (fixed), or read
 // at run time.
-template <typename Gm, bool MERGE = (Gm::ROWS > 1), typename T>
+template <typename Gm, bool MERGE = (Gm::ROWS > 1 || Gm::NT <= 128), typename T>
 __device__ __forceinline__ void ring_dispatch(bool fixed, const Phys<T>& P, const T* sf, T* sp, const EosRegs<T>& E,
                                               T rho_ref, int tid, int tx, int ty) {
     T hF = T(0);
