@@ -39,8 +39,45 @@ template <typename T> __device__ __forceinline__ long long at(const Inst* I, int
 // that no digit of a small difference is lost) to FP32 once and multiplies
 // by the weights in FP32 (within 1.5 ulp of the correctly rounded value, and
 // two FP64 operations per node instead of seven: GB300's FP64 pipe would
-// otherwise bound the initialisation).  Rows [y0, y1) of the field; rho,
-// ux and uy index the whole field.
+// otherwise bound the initialisation).  With a velocity the nine
+// values share the products of r, u and v: 33 FP64 instructions instead of
+// about 80 (FP32 lattice, 1531 x 1117 in bands: 38.8 -> 22.7 us a band).
+template <typename T, bool REST, typename R>
+__device__ __forceinline__ void equilibrium(double rr, R rho, R ux, R uy, T (&f)[9]) {
+    const double d = static_cast<double>(rho) - rr;
+    constexpr double t0 = 4.0 / 9.0, t1 = 1.0 / 9.0, t5 = 1.0 / 36.0;
+    if constexpr (REST) {
+        T t[3];
+        if constexpr (sizeof(T) == 4) {
+            const float df = static_cast<float>(d);
+            t[0] = __fmul_rn(4.0f / 9.0f, df);
+            t[1] = __fmul_rn(1.0f / 9.0f, df);
+            t[2] = __fmul_rn(1.0f / 36.0f, df);
+        } else {
+            t[0] = t0 * d;
+            t[1] = t1 * d;
+            t[2] = t5 * d;
+        }
+#pragma unroll
+        for (int a = 0; a < 9; ++a) f[a] = t[a == 0 ? 0 : (a < 5 ? 1 : 2)];
+    } else {
+        // t_a [(r - rr) + r (3 e.v + 4.5 (e.v)^2 - 1.5 v^2)], v = (u, v)
+        const double r = rho, u = ux, v = uy, ru = r * u, rv = r * v, uu = ru * u, vv = rv * v, uv = ru * v;
+        const double s = uu + vv, B = fma(-1.5, s, d), X = fma(4.5, uu, B), Y = fma(4.5, vv, B);
+        const double D = fma(4.5, s, B), P = fma(9.0, uv, D), M = fma(-9.0, uv, D), sp = ru + rv, sm = ru - rv;
+        f[0] = static_cast<T>(t0 * B);
+        f[1] = static_cast<T>(t1 * fma(3.0, ru, X));
+        f[3] = static_cast<T>(t1 * fma(-3.0, ru, X));
+        f[2] = static_cast<T>(t1 * fma(3.0, rv, Y));
+        f[4] = static_cast<T>(t1 * fma(-3.0, rv, Y));
+        f[5] = static_cast<T>(t5 * fma(3.0, sp, P));
+        f[7] = static_cast<T>(t5 * fma(-3.0, sp, P));
+        f[8] = static_cast<T>(t5 * fma(3.0, sm, M));
+        f[6] = static_cast<T>(t5 * fma(-3.0, sm, M));
+    }
+}
+
+// Rows [y0, y1) of the field; rho, ux and uy index the whole field.
 template <typename T, bool REST, typename R>
 __global__ void k_init(const Inst* __restrict__ I, const R* __restrict__ rho, const R* __restrict__ ux,
                        const R* __restrict__ uy, int parity, int y0, int y1) {
@@ -50,30 +87,14 @@ __global__ void k_init(const Inst* __restrict__ I, const R* __restrict__ rho, co
     for (int y = y0 + static_cast<int>(blockIdx.y); y < y1; y += gridDim.y)
         for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < nx; x += gridDim.x * blockDim.x) {
             const long long i = static_cast<long long>(y) * nx + x;
-            const double r = rho[i], u = !REST && ux ? double(ux[i]) : 0.0, v = !REST && uy ? double(uy[i]) : 0.0;
-            const double u2 = u * u + v * v;
-            // at rest: the three weights' products
-            const double d = r - rr;
-            T rest[3];
-            if constexpr (sizeof(T) == 4) {
-                const float df = static_cast<float>(d);
-                rest[0] = __fmul_rn(4.0f / 9.0f, df);
-                rest[1] = __fmul_rn(1.0f / 9.0f, df);
-                rest[2] = __fmul_rn(1.0f / 36.0f, df);
-            } else {
-                rest[0] = tw(0) * d;
-                rest[1] = tw(1) * d;
-                rest[2] = tw(5) * d;
-            }
+            T f[9];
+            equilibrium<T, REST>(rr, rho[i], !REST && ux ? ux[i] : R(0), !REST && uy ? uy[i] : R(0), f);
 #pragma unroll
             for (int a = 0; a < 9; ++a) {
-                const double eu = cx(a) * u + cy(a) * v;
-                // textbook second-order equilibrium, minus t_a rho_ref
-                const double dev = REST ? 0.0 : tw(a) * ((r - rr) + r * (3.0 * eu + 4.5 * eu * eu - 1.5 * u2));
                 int xs = x - cx(a), ys = y - cy(a);
                 xs = xs < 0 ? xs + nx : (xs >= nx ? xs - nx : xs);
                 ys = ys < 0 ? ys + ny : (ys >= ny ? ys - ny : ys);
-                p[at<T>(I, a, xs, ys)] = REST ? rest[a == 0 ? 0 : (a < 5 ? 1 : 2)] : static_cast<T>(dev);
+                p[at<T>(I, a, xs, ys)] = f[a];
             }
         }
 }
@@ -157,6 +178,15 @@ template <typename T> __device__ __forceinline__ void node_pops(const Inst* I, c
     for (int a = 0; a < 9; ++a) v[a] = p[at<T>(I, a, x - cx(a), y - cy(a))];
 }
 
+// A float as a double, by moving its bits: the conversion instruction holds
+// the FP64 pipe as long as an addition.  Denormals become zero.
+__device__ __forceinline__ double widen(float v) {
+    const unsigned u = __float_as_uint(v), sign = u & 0x80000000u;
+    const bool tiny = (u & 0x7f800000u) == 0;
+    return __hiloint2double(static_cast<int>(tiny ? sign : sign | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
+                            static_cast<int>(tiny ? 0u : u << 29));
+}
+
 // Sum of N floats in FP64 accuracy with three FP64 additions: the sum as an
 // unevaluated triple hi + lo + lo2 (Knuth's TwoSum gives the exact error of
 // each addition; the errors' own sum is kept the same way), within 2^-69 of
@@ -183,7 +213,7 @@ template <int N> __device__ __forceinline__ double sum_f32(const float (&v)[N], 
         for (int k = 0; k < N; ++k) r += static_cast<double>(v[k]);
         return r + plus;
     }
-    return (static_cast<double>(hi) + plus) + (static_cast<double>(lo) + static_cast<double>(lo2));
+    return (widen(hi) + plus) + (widen(lo) + widen(lo2));
 }
 
 // rho of a node from its nine populations.
@@ -214,16 +244,15 @@ __device__ __forceinline__ void node_j(const double (&v)[9], double& jx, double&
 
 // Tiles of the kernels that need the force (velocity fields, statistics):
 // psi of the tile and its 1-node ring (periodic) goes to shared memory once,
-// so a node costs 1.25 densities and square roots instead of nine, and about
-// 100 FP64 instructions instead of 700 (the FP64 pipe is the bound: 16
-// clocks of an SM per warp instruction).  32 x 16 nodes: two per thread, a
-// ring of 612 nodes in 20 warp passes for 16 of the tile's own.
-// FP32 statistics of 1024^2: 1113 -> 250 us per call, of 256^2: 149 -> 35;
-// the two velocity components of 1531 x 1117: 2 x 1709 -> 396 us, rho and
-// psi with them.
+// so a node costs 1.25 densities and psi instead of nine, and about 65 FP64
+// instructions instead of 700 (the FP64 pipe is the bound: 19 clocks of an
+// SM per warp instruction).  32 x 16 nodes: two per thread, a ring of 612
+// nodes in 20 warp passes for 16 of the tile's own.  FP32 statistics of
+// 1024^2: 1113 -> 180 us per call, of 256^2: 149 -> 30; the two velocity
+// components of 1531 x 1117: 2 x 1709 -> 277 us, rho and psi with them.
 constexpr int kFlowX = 32, kFlowY = 16, kFlowW = kFlowX + 2, kFlowH = kFlowY + 2;
 struct FlowTile {
-    double psi[kFlowH][kFlowW], rho[kFlowH][kFlowW];
+    double psi[kFlowH][kFlowW], h[kFlowH][kFlowW], rho[kFlowH][kFlowW];   // h: hF psi^2, as in the step kernels
 };
 
 // rho, velocity (rho u = sum f e + F/2, F of Eq. 9) and psi of the nodes
@@ -235,7 +264,7 @@ __device__ __forceinline__ void flow_tile(const Inst* I, const T* p, int x0, int
     const int nx = I->nx, ny = I->ny, interact = P.interact;
     const int tid = threadIdx.x;
     if (interact) {
-        const LawFp64 radicand(P, true);
+        const LawFp64 law(P, true);
         const int w = min(kFlowX, nx - x0) + 2, h = min(kFlowY, y1 - y0) + 2;
         for (int e = tid; e < kFlowW * kFlowH; e += kThreads) {
             const int j = e / kFlowW, i = e - j * kFlowW;
@@ -244,12 +273,14 @@ __device__ __forceinline__ void flow_tile(const Inst* I, const T* p, int x0, int
             x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
             y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
             const double r = node_rho<T>(I, p, x, y);
+            const double ps = law.psi(r);
             S.rho[j][i] = r;
-            S.psi[j][i] = sqrt(radicand(r));
+            S.psi[j][i] = ps;
+            S.h[j][i] = (P.hF * ps) * ps;
         }
         __syncthreads();
     }
-    const double negGw = -P.G * (1.0 / 12.0), hA = 0.5 * P.A, omA = 1.0 - P.A;
+    const double cF = P.cF;
     const int i = tid % kFlowX + 1, x = x0 + i - 1;
     for (int j = tid / kFlowX + 1; j <= kFlowY; j += kThreads / kFlowX) {
         const int y = y0 + j - 1;
@@ -260,19 +291,17 @@ __device__ __forceinline__ void flow_tile(const Inst* I, const T* p, int x0, int
         double jx, jy, ps = 0.0;
         node_j(v, jx, jy);
         if (interact) {
-            // Eq. 9 with the weights 12 w_a (4 on the axes, 1 on the diagonals)
-            const double p1 = S.psi[j][i + 1], p2 = S.psi[j + 1][i], p3 = S.psi[j][i - 1], p4 = S.psi[j - 1][i];
-            const double p5 = S.psi[j + 1][i + 1], p6 = S.psi[j + 1][i - 1], p7 = S.psi[j - 1][i - 1],
-                         p8 = S.psi[j - 1][i + 1];
+            // Eq. 9 with the weights 12 w_a (4 on the axes, 1 on the
+            // diagonals) over g_a = -(G/12) [(1-A) psi psi_a + (A/2) psi_a^2]
             ps = S.psi[j][i];
-            const double a57 = p5 - p7, a86 = p8 - p6, b57 = p5 * p5 - p7 * p7, b86 = p8 * p8 - p6 * p6;
-            const double gx1 = 4.0 * (p1 - p3) + (a57 + a86), gy1 = 4.0 * (p2 - p4) + (a57 - a86);
-            const double gx2 = 4.0 * (p1 * p1 - p3 * p3) + (b57 + b86), gy2 = 4.0 * (p2 * p2 - p4 * p4) + (b57 - b86);
-            const double c = omA * ps;
-            jx += 0.5 * (negGw * (c * gx1 + hA * gx2));
-            jy += 0.5 * (negGw * (c * gy1 + hA * gy2));
+            const double c = cF * ps;
+            auto g = [&](int dj, int di) { return fma(c, S.psi[j + dj][i + di], S.h[j + dj][i + di]); };
+            const double a57 = g(1, 1) - g(-1, -1), a86 = g(-1, 1) - g(1, -1);
+            jx = fma(0.5, fma(4.0, g(0, 1) - g(0, -1), a57 + a86), jx);
+            jy = fma(0.5, fma(4.0, g(1, 0) - g(-1, 0), a57 - a86), jy);
         }
-        use(x, y, r, jx / r, jy / r, ps);
+        const double inv = Fast<double>::rcp(r);
+        use(x, y, r, quotient(jx, inv, r), quotient(jy, inv, r), ps);
     }
     if (interact) __syncthreads();   // before the next tile's psi
 }
@@ -286,12 +315,12 @@ __global__ void k_field(const Inst* __restrict__ I, int parity, int y0, int y1, 
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *status = *I->status;
     const int nx = I->nx;
     const T* p = popk<T>(I, parity);
-    const LawFp64 radicand(I->pd, true);
+    const LawFp64 law(I->pd, true);
     for (int y = y0 + static_cast<int>(blockIdx.y); y < y1; y += gridDim.y)
         for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < nx; x += gridDim.x * blockDim.x) {
             const double r = node_rho<T>(I, p, x, y);
             double v = r;
-            if constexpr (FIELD == 3) v = I->pd.interact ? sqrt(radicand(r)) : 0.0;
+            if constexpr (FIELD == 3) v = I->pd.interact ? law.psi(r) : 0.0;
             out[static_cast<long long>(y) * nx + x] = static_cast<O>(v);
         }
 }
@@ -323,17 +352,17 @@ __global__ void __launch_bounds__(kThreads) k_flow(const Inst* __restrict__ I, i
 // Sums for Laplace's law (LaplaceSums); p = p_EOS(rho) (equal to
 // rho/3 + G psi^2/2, Eq. 10).  The last block puts the totals and the
 // instance's status into *out, which is mapped host memory: the call needs no
-// second launch and no copy.  About 33 FP64 instructions per node (nine
+// second launch and no copy.  About 22 FP64 instructions per node (nine
 // additions in FP64, the square root and the divisions by the lattice's size
-// are gone).  Per call, FP32: 256^2 88 -> 24 us, 1024^2 236 -> 85 us.
+// are gone).  Per call, FP32: 256^2 88 -> 21 us, 1024^2 236 -> 79 us.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_measure(const Inst* __restrict__ I, int parity, Discs D, int rpt,
                                                        double* __restrict__ partials, unsigned* ticket,
                                                        Reduced* out) {
-    __shared__ double dy2[kTileRows * kMaxRpt];
+    __shared__ AxisTable A;
     const T* p = popk<T>(I, parity);
     LaplaceSums L;
-    laplace_tiles(L, LawFp64(I->pd, false), D, I->nx, I->ny, rpt, dy2,
+    laplace_tiles(L, LawFp64(I->pd, false), D, I->nx, I->ny, rpt, A,
                   [&](int x, int y) { return node_rho<T>(I, p, x, y); });
     double total;
     if (grid_sum8(L.v, -1, 0.0, partials, ticket, &total)) {

@@ -5,8 +5,9 @@
 //
 // GB300's FP64 pipe (two thread operations per clock and SM) bounds all of
 // these, so the code around the sums spends as few FP64 instructions as it
-// can: an FP64 instruction of one warp holds the pipe for 16 clocks however
-// many of its lanes carry data.
+// can: an FP64 instruction of one warp holds the pipe for 16 to 19 clocks
+// however many of its lanes carry data, and conversions to and from FP64 do
+// as well.
 #pragma once
 
 #include <cmath>
@@ -147,27 +148,46 @@ __device__ __forceinline__ double axis2(int v, double c, int n, double inv_n) {
     return d * d;
 }
 
+// num / den rounded like the division up to the last bit's ties: a reciprocal
+// refined to its rounding, then one residual step.  Seven FP64 instructions;
+// the general division's special cases (overflowing or denormal quotients)
+// are not needed for den in (0, 1].
+__device__ __forceinline__ double quotient(double num, double inv_den, double den) {
+    const double q = num * inv_den;
+    return fma(fma(-q, den, num), inv_den, q);
+}
+
 // The pressure law with its constants folded, p = rho [K R T h(rho) - K a rho]
-// (h = num / q^3 for Carnahan-Starling), and Eq. 10's radicand
-// (2/G)(p - rho/3) in the same form: 18 and 19 FP64 instructions instead of
-// 22 and 25.
+// (h = num / q^3 for Carnahan-Starling), and psi = W / sqrt(W D) with Eq.
+// 10's radicand (2/G)(p - rho/3) = W / D: 16 and 17 FP64 instructions.
 struct LawFp64 {
     int eos;
-    double b, c1, c2, c3;   // p: K R T, K a (K a alpha), 0; radicand: those and 1/3, times 2/G
-    __device__ __forceinline__ LawFp64(const Phys<double>& P, bool radicand) {
-        const double s = radicand ? P.two_over_G : 1.0;
+    double b, c1, c2, c3;   // p: K R T, K a (K a alpha), 0; psi: those and 1/3, times 2/G
+    __device__ __forceinline__ LawFp64(const Phys<double>& P, bool psi) {
+        const double s = psi ? P.two_over_G : 1.0;
         eos = P.eos;
         b = P.eos == LBM_EOS_CS ? P.b4 : P.b;
         c1 = s * (P.K * P.RT);
         c2 = s * (P.K * (P.eos == LBM_EOS_PR ? P.aalpha : P.a));
-        c3 = radicand ? s * (1.0 / 3.0) : 0.0;
+        c3 = psi ? s * (1.0 / 3.0) : 0.0;
     }
-    __device__ __forceinline__ double operator()(double rho) const {
+    __device__ __forceinline__ double pressure(double rho) const {
         const double n = b * rho, q = 1.0 - n;
-        if (eos == LBM_EOS_CS) return rho * (c1 * fma(n, fma(n, q, 1.0), 1.0) / (q * q * q) - fma(c2, rho, c3));
-        if (eos == LBM_EOS_VDW) return rho * (c1 / q - fma(c2, rho, c3));
-        return rho * (c1 / q - fma(c2, rho / fma(n, 2.0 - n, 1.0), c3));
+        if (eos == LBM_EOS_CS) return rho * (c1 * div(fma(n, fma(n, q, 1.0), 1.0), q * q * q) - c2 * rho);
+        if (eos == LBM_EOS_VDW) return rho * (div(c1, q) - c2 * rho);
+        return rho * (div(c1, q) - div(c2 * rho, fma(n, 2.0 - n, 1.0)));
     }
+    __device__ __forceinline__ double psi(double rho) const {
+        const double n = b * rho, q = 1.0 - n;
+        if (eos == LBM_EOS_CS) {
+            const double q3 = q * q * q;
+            return psi_fold_fp64(rho * fma(-fma(c2, rho, c3), q3, c1 * fma(n, fma(n, q, 1.0), 1.0)), q3);
+        }
+        if (eos == LBM_EOS_VDW) return psi_fold_fp64(rho * fma(-fma(c2, rho, c3), q, c1), q);
+        const double e = fma(n, 2.0 - n, 1.0);
+        return psi_fold_fp64(rho * fma(-fma(c2, rho, c3 * e), q, c1 * e), q * e);
+    }
+    static __device__ __forceinline__ double div(double num, double den) { return quotient(num, Fast<double>::rcp(den), den); }
 };
 
 // Laplace sums of one thread: {sum rho, sum p_in, sum rho_in, n_in,
@@ -182,7 +202,7 @@ struct LaplaceSums {
         const bool in = b <= D.in2, out = b >= D.out2;
         if (in == out) rest += in ? -r : r;
         if (!in && !out) return;
-        const double p = p_eos(r);
+        const double p = p_eos.pressure(r);
         if (in) {
             v[1] += p;
             v[2] += r;
@@ -207,29 +227,44 @@ constexpr int kTileX = 64, kTileRows = kRedThreads / kTileX, kMaxRpt = 8;
 inline long long tile_count(int nx, int ny, int rpt) {
     return static_cast<long long>((nx + kTileX - 1) / kTileX) * ((ny + rpt * kTileRows - 1) / (rpt * kTileRows));
 }
-// Rows per thread: as many as leave two tiles per SM.  The distance along x
-// and the block's reduction are then paid once for them.
+// Rows per thread: the cheapest of 1 .. kMaxRpt in FP64 instructions of the
+// busiest SM, about 23 per node and 13 per thread and tile (its distances and
+// its block's reduction).
 inline int tile_rpt(int nx, int ny) {
-    int rpt = 1;
-    while (rpt < kMaxRpt && tile_count(nx, ny, 2 * rpt) >= kReduceBlocks) rpt *= 2;
-    return rpt;
+    int best = 1;
+    long long least = 0;
+    for (int rpt = 1; rpt <= kMaxRpt; rpt *= 2) {
+        const long long cost = (tile_count(nx, ny, rpt) + 151) / 152 * (23 * rpt + 13);
+        if (rpt == 1 || cost < least) {
+            least = cost;
+            best = rpt;
+        }
+    }
+    return best;
 }
 // The sums over the tiles of this block; rho_at(x, y) gives a node's density.
-// dy2 (kTileRows * kMaxRpt doubles of shared memory): the squared distances
-// along y of a tile's rows, formed once per tile.
+// A tile's squared distances along x and y are formed once, in shared memory.
+struct AxisTable {
+    double x[kTileX], y[kTileRows * kMaxRpt];
+};
 template <typename F>
 __device__ __forceinline__ void laplace_tiles(LaplaceSums& L, const LawFp64& p_eos, const Discs& D, int nx, int ny,
-                                              int rpt, double* dy2, F rho_at) {
-    const int rows = kTileRows * rpt, tx = threadIdx.x % kTileX, ty = threadIdx.x / kTileX;
+                                              int rpt, AxisTable& A, F rho_at) {
+    const int rows = kTileRows * rpt, t = threadIdx.x, tx = t % kTileX, ty = t / kTileX;
     const int tiles_x = (nx + kTileX - 1) / kTileX, tiles = tiles_x * ((ny + rows - 1) / rows);
-    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
-        const int row = t / tiles_x, x = (t - row * tiles_x) * kTileX + tx, y0 = row * rows;
-        __syncthreads();   // the tile before is done with dy2
-        if (static_cast<int>(threadIdx.x) < rows) dy2[threadIdx.x] = axis2(y0 + threadIdx.x, D.cy, ny, D.inv_ny);
+    for (int k = blockIdx.x; k < tiles; k += gridDim.x) {
+        const int row = k / tiles_x, x0 = (k - row * tiles_x) * kTileX, x = x0 + tx, y0 = row * rows;
+        __syncthreads();   // the tile before is done with the table
+        if (t < kTileX + rows) {
+            const bool along_x = t < kTileX;
+            const double d = axis2(along_x ? x0 + t : y0 + t - kTileX, along_x ? D.cx : D.cy, along_x ? nx : ny,
+                                   along_x ? D.inv_nx : D.inv_ny);
+            (along_x ? A.x[t] : A.y[t - kTileX]) = d;
+        }
         __syncthreads();
         if (x >= nx) continue;
-        const double dx2 = axis2(x, D.cx, nx, D.inv_nx);
-        for (int k = ty; k < rows && y0 + k < ny; k += kTileRows) L.add(p_eos, D, rho_at(x, y0 + k), dx2 + dy2[k]);
+        const double dx2 = A.x[tx];
+        for (int j = ty; j < rows && y0 + j < ny; j += kTileRows) L.add(p_eos, D, rho_at(x, y0 + j), dx2 + A.y[j]);
     }
     L.close();
 }

@@ -50,14 +50,14 @@ std::mutex g_mu;
 double* g_ptr[kMaxDevices] = {};
 
 // The Laplace sums of a field (LaplaceSums) in one launch, bound by the FP64
-// pipe (22 instructions per node; 4096^2: 1970 -> 846 us per call, of which
+// pipe (20 instructions per node; 4096^2: 1970 -> 725 us per call, of which
 // the former second launch was 168).
 __global__ void __launch_bounds__(kRedThreads)
     k_field_sums(const double* __restrict__ rho, int nx, int ny, Phys<double> P, Discs D, int rpt,
                  double* __restrict__ partials, unsigned* ticket, double* __restrict__ out) {
-    __shared__ double dy2[kTileRows * kMaxRpt];
+    __shared__ AxisTable A;
     LaplaceSums L;
-    laplace_tiles(L, LawFp64(P, false), D, nx, ny, rpt, dy2,
+    laplace_tiles(L, LawFp64(P, false), D, nx, ny, rpt, A,
                   [&](int x, int y) { return rho[static_cast<long long>(y) * nx + x]; });
     double total;
     if (grid_sum8(L.v, -1, 0.0, partials, ticket, &total)) out[threadIdx.x] = total;

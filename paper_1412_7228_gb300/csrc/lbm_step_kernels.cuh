@@ -221,21 +221,7 @@ template <int EOSK, typename T> __device__ __forceinline__ T radicand_step(const
 //   Peng-Robinson      D = d e, e = 1 + 2 b rho - (b rho)^2,
 //                      W = rho [kR e - (kAa rho + k3 e) d];
 // with kR = (2/G) K R T, kA = (2/G) K a, kAa = (2/G) K a alpha(T),
-// k3 = (2/G)/3.  Then psi = W / sqrt(W D); 1 / sqrt(x) comes from the hardware
-// estimate y refined by one third-order step (Householder's iteration):
-// with d = 1 - x y^2, y + y d (1/2 + 3/8 d) leaves an error of 5/16 d^3, far
-// below the last place from an estimate good to 2^-20; three FP64
-// instructions fewer than two second-order steps.  A negative radicand gives
-// NaN (as the square root does), psi(W = 0) = 0.
-__device__ __forceinline__ double psi_fold_fp64(double W, double D) {
-    const double x = W * D;
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double d = fma(-(x * y), y, 1.0);
-    const double r = fma(y * d, fma(d, 0.375, 0.5), y);
-    return W == 0.0 ? 0.0 : W * r;
-}
-
+// k3 = (2/G)/3.  Then psi = W / sqrt(W D) (psi_fold_fp64).
 template <int EOSK>
 __device__ __forceinline__ double psi_fp64(const EosRegs<double>& E, double kR, double kA, double kAa, double k3,
                                            double rho) {
