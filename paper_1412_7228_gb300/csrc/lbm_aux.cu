@@ -306,13 +306,32 @@ __device__ __forceinline__ void flow_tile(const Inst* I, const T* p, int x0, int
     if (interact) __syncthreads();   // before the next tile's psi
 }
 
+// The block's writes are done: the last block tells the host (Notice).
+__device__ __forceinline__ void notify(const Notice& to) {
+    if (!to.ticket) return;
+    __threadfence_system();
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    if (atomicAdd(to.ticket, 1u) != gridDim.x * gridDim.y - 1) return;
+    *to.ticket = 0;
+    __threadfence_system();
+    *static_cast<volatile unsigned*>(&to.to->call) = to.call;
+}
+// The same after a reduction, whose last block's first warp has written the
+// results.
+__device__ __forceinline__ void notify_reduced(const Notice& to) {
+    __threadfence_system();
+    __syncwarp(0xffu);
+    if (threadIdx.x == 0) *static_cast<volatile unsigned*>(&to.to->call) = to.call;
+}
+
 // rho or psi of the nodes, one field per launch (FIELD 0 rho, 3 psi): the
 // density read-back keeps the registers of a plain gather.  Rows [y0, y1) of
 // the field, at their place in out (row-major nx x ny).
 template <typename T, int FIELD, typename O>
 __global__ void k_field(const Inst* __restrict__ I, int parity, int y0, int y1, O* __restrict__ out,
-                        int* status) {
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *status = *I->status;
+                        Notice to) {
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) to.to->status = *I->status;
     const int nx = I->nx;
     const T* p = popk<T>(I, parity);
     const LawFp64 law(I->pd, true);
@@ -323,6 +342,7 @@ __global__ void k_field(const Inst* __restrict__ I, int parity, int y0, int y1, 
             if constexpr (FIELD == 3) v = I->pd.interact ? law.psi(r) : 0.0;
             out[static_cast<long long>(y) * nx + x] = static_cast<O>(v);
         }
+    notify(to);
 }
 
 // The velocity components and, where asked for, rho and psi of rows [y0, y1)
@@ -330,9 +350,9 @@ __global__ void k_field(const Inst* __restrict__ I, int parity, int y0, int y1, 
 template <typename T, typename O>
 __global__ void __launch_bounds__(kThreads) k_flow(const Inst* __restrict__ I, int parity, int y0, int y1,
                                                    O* __restrict__ rho, O* __restrict__ ux, O* __restrict__ uy,
-                                                   O* __restrict__ psi, int* status) {
+                                                   O* __restrict__ psi, Notice to) {
     __shared__ FlowTile S;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *status = *I->status;
+    if (blockIdx.x == 0 && threadIdx.x == 0) to.to->status = *I->status;
     const int nx = I->nx, tiles_x = (nx + kFlowX - 1) / kFlowX, tiles = tiles_x * ((y1 - y0 + kFlowY - 1) / kFlowY);
     const T* p = popk<T>(I, parity);
     for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
@@ -346,35 +366,36 @@ __global__ void __launch_bounds__(kThreads) k_flow(const Inst* __restrict__ I, i
                          if (psi) psi[i] = static_cast<O>(ps);
                      });
     }
+    notify(to);
 }
 
 // ---- FP64 reductions (lbm_reduce.cuh) -------------------------------------
 // Sums for Laplace's law (LaplaceSums); p = p_EOS(rho) (equal to
 // rho/3 + G psi^2/2, Eq. 10).  The last block puts the totals and the
-// instance's status into *out, which is mapped host memory: the call needs no
-// second launch and no copy.  About 22 FP64 instructions per node (nine
+// instance's status into mapped host memory and says so there: the call needs
+// no second launch, no copy and no wait for the stream.  About 22 FP64 instructions per node (nine
 // additions in FP64, the square root and the divisions by the lattice's size
 // are gone).  Per call, FP32: 256^2 88 -> 21 us, 1024^2 236 -> 79 us.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_measure(const Inst* __restrict__ I, int parity, Discs D, int rpt,
-                                                       double* __restrict__ partials, unsigned* ticket,
-                                                       Reduced* out) {
+                                                       double* __restrict__ partials, Notice to) {
     __shared__ AxisTable A;
     const T* p = popk<T>(I, parity);
     LaplaceSums L;
     laplace_tiles(L, LawFp64(I->pd, false), D, I->nx, I->ny, rpt, A,
                   [&](int x, int y) { return node_rho<T>(I, p, x, y); });
     double total;
-    if (grid_sum8(L.v, -1, 0.0, partials, ticket, &total)) {
-        out->v[threadIdx.x] = total;
-        if (threadIdx.x == 0) out->status = *I->status;
+    if (grid_sum8(L.v, -1, 0.0, partials, to.ticket, &total)) {
+        to.to->v[threadIdx.x] = total;
+        if (threadIdx.x == 0) to.to->status = *I->status;
+        notify_reduced(to);
     }
 }
 
 // {mass, sum rho u_x, sum rho u_y, sum rho |u|^2 / 2, max |u|, 0, 0, 0}
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_stats(const Inst* __restrict__ I, int parity, double* __restrict__ partials,
-                                                     unsigned* ticket, Reduced* out) {
+                                                     Notice to) {
     __shared__ FlowTile S;
     const int nx = I->nx, ny = I->ny;
     const int tiles_x = (nx + kFlowX - 1) / kFlowX, tiles = tiles_x * ((ny + kFlowY - 1) / kFlowY);
@@ -393,9 +414,10 @@ __global__ void __launch_bounds__(kThreads) k_stats(const Inst* __restrict__ I, 
                      });
     }
     double total;
-    if (grid_sum8(v, 4, most, partials, ticket, &total)) {
-        out->v[threadIdx.x] = threadIdx.x == 4 ? sqrt(total) : total;
-        if (threadIdx.x == 0) out->status = *I->status;
+    if (grid_sum8(v, 4, most, partials, to.ticket, &total)) {
+        to.to->v[threadIdx.x] = threadIdx.x == 4 ? sqrt(total) : total;
+        if (threadIdx.x == 0) to.to->status = *I->status;
+        notify_reduced(to);
     }
 }
 
@@ -570,10 +592,10 @@ cudaError_t aux_gather_plane(const Inst& h, const Inst* d, int parity, int a, do
 }
 
 template <typename O>
-cudaError_t field_t(const Inst& h, const Inst* d, int parity, int field, int y0, int y1, O* out, int* status,
-                    cudaStream_t st) {
+cudaError_t field_t(const Inst& h, const Inst* d, int parity, int field, int y0, int y1, O* out,
+                    const Notice& to, cudaStream_t st) {
     const dim3 g = grid_2d(h.nx, y1 - y0);
-    auto go = [&](auto k) { k<<<g, kThreads, 0, st>>>(d, parity, y0, y1, out, status); };
+    auto go = [&](auto k) { k<<<g, kThreads, 0, st>>>(d, parity, y0, y1, out, to); };
     const bool f32 = h.prec == LBM_FP32;
     if (field == 0) f32 ? go(k_field<float, 0, O>) : go(k_field<double, 0, O>);
     else f32 ? go(k_field<float, 3, O>) : go(k_field<double, 3, O>);
@@ -581,10 +603,10 @@ cudaError_t field_t(const Inst& h, const Inst* d, int parity, int field, int y0,
 }
 
 cudaError_t aux_field(const Inst& h, const Inst* d, int parity, int field, int y0, int y1, void* out, bool f32out,
-                      int* status, cudaStream_t st) {
+                      const Notice& to, cudaStream_t st) {
     if (field != 0 && field != 3) return cudaErrorInvalidValue;
-    if (f32out) return field_t(h, d, parity, field, y0, y1, static_cast<float*>(out), status, st);
-    return field_t(h, d, parity, field, y0, y1, static_cast<double*>(out), status, st);
+    if (f32out) return field_t(h, d, parity, field, y0, y1, static_cast<float*>(out), to, st);
+    return field_t(h, d, parity, field, y0, y1, static_cast<double*>(out), to, st);
 }
 
 // Blocks of the flow and reduction kernels: one per tile up to what the
@@ -596,12 +618,12 @@ int flow_grid(int nx, int rows) {
 }
 
 cudaError_t aux_flow(const Inst& h, const Inst* d, int parity, int y0, int y1, void* const out[4], bool f32out,
-                     int* status, cudaStream_t st) {
+                     const Notice& to, cudaStream_t st) {
     const int g = flow_grid(h.nx, y1 - y0);
     auto go = [&](auto k, auto* zero) {
         using O = typename std::remove_pointer<decltype(zero)>::type;
         k<<<g, kThreads, 0, st>>>(d, parity, y0, y1, static_cast<O*>(out[0]), static_cast<O*>(out[1]),
-                                  static_cast<O*>(out[2]), static_cast<O*>(out[3]), status);
+                                  static_cast<O*>(out[2]), static_cast<O*>(out[3]), to);
     };
     const bool f32 = h.prec == LBM_FP32;
     float* zf = nullptr;
@@ -612,23 +634,22 @@ cudaError_t aux_flow(const Inst& h, const Inst* d, int parity, int y0, int y1, v
 }
 
 cudaError_t aux_measure(const Inst& h, const Inst* d, int parity, double cxc, double cyc, double r_in,
-                        double r_out, double* partials, int rows, unsigned* ticket, Reduced* out,
-                        cudaStream_t st) {
+                        double r_out, double* partials, int rows, const Notice& to, cudaStream_t st) {
     if (rows > kResident) rows = kResident;
     const Discs D = make_discs(h.nx, h.ny, cxc, cyc, r_in, r_out);
     const int rpt = tile_rpt(h.nx, h.ny);
     const long long tiles = tile_count(h.nx, h.ny, rpt);
     const int g = static_cast<int>(tiles < rows ? tiles : rows);
-    if (h.prec == LBM_FP32) k_measure<float><<<g, kThreads, 0, st>>>(d, parity, D, rpt, partials, ticket, out);
-    else k_measure<double><<<g, kThreads, 0, st>>>(d, parity, D, rpt, partials, ticket, out);
+    if (h.prec == LBM_FP32) k_measure<float><<<g, kThreads, 0, st>>>(d, parity, D, rpt, partials, to);
+    else k_measure<double><<<g, kThreads, 0, st>>>(d, parity, D, rpt, partials, to);
     return cudaGetLastError();
 }
 
-cudaError_t aux_stats(const Inst& h, const Inst* d, int parity, double* partials, int rows, unsigned* ticket,
-                      Reduced* out, cudaStream_t st) {
+cudaError_t aux_stats(const Inst& h, const Inst* d, int parity, double* partials, int rows, const Notice& to,
+                      cudaStream_t st) {
     const int tiles = flow_grid(h.nx, h.ny), g = tiles < rows ? tiles : rows;
-    if (h.prec == LBM_FP32) k_stats<float><<<g, kThreads, 0, st>>>(d, parity, partials, ticket, out);
-    else k_stats<double><<<g, kThreads, 0, st>>>(d, parity, partials, ticket, out);
+    if (h.prec == LBM_FP32) k_stats<float><<<g, kThreads, 0, st>>>(d, parity, partials, to);
+    else k_stats<double><<<g, kThreads, 0, st>>>(d, parity, partials, to);
     return cudaGetLastError();
 }
 

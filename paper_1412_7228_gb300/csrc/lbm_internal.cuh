@@ -351,6 +351,26 @@ cudaError_t run_launch(int prec, int k, const Inst* d_insts, const void* args, b
 bool cluster_supported(int prec, int nx, int ny);
 cudaError_t cluster_run(const Inst& host, int parity, int nsteps, cudaStream_t st);
 
+// What a call reads back besides its arrays: the sums of a reduction and the
+// instance's status word, written by the device into pinned host memory
+// mapped for it, and the number of the call whose results these are, written
+// last.
+constexpr int kReduceSlots = 8;
+struct Reduced {
+    double v[kReduceSlots];
+    int status;
+    unsigned call;
+};
+// How a kernel gives its results: its last block (by `ticket`, a device word
+// that is zero between launches) writes to->call = call once every block's
+// writes are visible to the host.  ticket NULL: the status word only (the host
+// waits for the stream).
+struct Notice {
+    Reduced* to;
+    unsigned* ticket;
+    unsigned call;
+};
+
 // Auxiliary kernels (lbm_aux.cu); `host` is the host copy of the descriptor.
 // Fields of nx*ny doubles, or floats with f32 (each widened to FP64 exactly).
 cudaError_t aux_init(const Inst& host, const Inst* d_inst, const void* rho, const void* ux, const void* uy, bool f32,
@@ -363,31 +383,22 @@ cudaError_t aux_gather_plane(const Inst& host, const Inst* d_inst, int parity, i
                              cudaStream_t st);
 // field: 0 rho, 3 psi; rows [y0, y1), written at their place in out
 // (row-major, nx per row)
-// f32out: floats, each the FP64 value rounded to nearest; *status (mapped host
-// memory): the instance's status word
+// f32out: floats, each the FP64 value rounded to nearest; `to`: where the
+// instance's status word goes and how the host is told
 cudaError_t aux_field(const Inst& host, const Inst* d_inst, int parity, int field, int y0, int y1, void* out,
-                      bool f32out, int* status, cudaStream_t st);
+                      bool f32out, const Notice& to, cudaStream_t st);
 // rho, ux, uy, psi into out[0..3] (any may be NULL) in one pass; rows and types as above
 cudaError_t aux_flow(const Inst& host, const Inst* d_inst, int parity, int y0, int y1, void* const out[4], bool f32out,
-                     int* status, cudaStream_t st);
+                     const Notice& to, cudaStream_t st);
 // out: 4 device words (see lbm_fp64_math_check); default stream.
 cudaError_t aux_math_check(long long n, double lo, double hi, unsigned long long* out);
 // FP64 FMA throughput of the current device (see lbm_fp64_fma_rate).
 cudaError_t aux_fp64_fma_rate(int iters, cudaStream_t st, double* flops_per_s, double* seconds);
 constexpr int kReduceBlocks = 304;   // rows of partial sums that every context has; larger lattices use their field scratch
-constexpr int kReduceSlots = 8;
-// What a reduction returns: its sums and the instance's status word, written
-// by the device (into host memory mapped for it).
-struct Reduced {
-    double v[kReduceSlots];
-    int status;
-};
-// partials: device doubles for the partial sums of `rows` blocks
-// (kReduceSlots each); ticket: a device word that is zero between launches
+// partials: device doubles for the partial sums of `rows` blocks (kReduceSlots each)
 cudaError_t aux_measure(const Inst& host, const Inst* d_inst, int parity, double cx, double cy,
-                        double r_in, double r_out, double* partials, int rows, unsigned* ticket, Reduced* out,
-                        cudaStream_t st);
-cudaError_t aux_stats(const Inst& host, const Inst* d_inst, int parity, double* partials, int rows, unsigned* ticket,
-                      Reduced* out, cudaStream_t st);
+                        double r_in, double r_out, double* partials, int rows, const Notice& to, cudaStream_t st);
+cudaError_t aux_stats(const Inst& host, const Inst* d_inst, int parity, double* partials, int rows, const Notice& to,
+                      cudaStream_t st);
 
 }  // namespace lbm

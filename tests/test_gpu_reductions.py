@@ -147,3 +147,53 @@ def test_field_sums_of_a_device_field(P, nx, ny):
             for k, v, s in (("rho_in", rho, i), ("p_in", p, i), ("rho_out", rho, o), ("p_out", p, o)):
                 if s.any():
                     assert abs(m[k] - v[s].mean()) <= 1e-12, k
+
+
+@pytest.mark.parametrize("nx,ny", [(5, 3), (181, 180), (700, 150), (2900, 3000)])
+def test_reads_into_every_kind_of_memory(P, nx, ny):
+    """Pinned arrays are written by the kernels, small pageable ones come
+    through the context's stage, larger ones and those read in bands by
+    copies: the same values in each, and nothing beside them."""
+    import torch
+    lat, _, _ = _lattice(P, nx, ny, P.LBM_FP32, "cs")
+    for dtype in (np.float32, np.float64):
+        tdt = torch.float32 if dtype == np.float32 else torch.float64
+        want = lat.read_fields(dtype=dtype)
+        pinned = torch.full((6 * nx * ny + 6,), -7.0, dtype=tdt).pin_memory().numpy()
+        plain = np.full(6 * nx * ny + 6, -7.0, dtype=dtype)
+        for mem in (pinned, plain):
+            out = {k: mem[1 + j * (nx * ny + 1):1 + j * (nx * ny + 1) + nx * ny].reshape(ny, nx)
+                   for j, k in enumerate(("rho", "ux", "uy", "psi"))}
+            for which in (("rho",), ("rho", "psi"), ("rho", "ux", "uy", "psi")):
+                mem[:] = -7.0
+                got = lat.read_fields(which=which, out=out, dtype=dtype)
+                for k in which:
+                    assert np.array_equal(got[k], want[k]), k
+                assert (mem == -7.0).sum() == mem.size - len(which) * nx * ny
+        mixed = {"rho": pinned[:nx * ny].reshape(ny, nx), "ux": np.empty((ny, nx), dtype=dtype)}
+        got = lat.read_fields(which=("rho", "ux"), out=mixed, dtype=dtype)
+        assert np.array_equal(got["rho"], want["rho"]) and np.array_equal(got["ux"], want["ux"])
+    lat.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(30, 20), (1100, 1000)])
+def test_a_refused_field_leaves_one_lattice_as_it_was(P, nx, ny):
+    """The equilibrium of a context of one lattice is written beside its
+    current state before the check is known."""
+    lat, eos, A = _lattice(P, nx, ny, P.LBM_FP32, "cs")
+    lat.step(2)
+    before = lat.read_populations()
+    bad = np.full((ny, nx), 0.2)
+    bad[ny - 1, nx - 1] = -1.0
+    for args in ((bad,), (np.full((ny, nx), 0.2), np.full((ny, nx), np.inf), np.zeros((ny, nx)))):
+        with pytest.raises(P.LbmError) as ei:
+            lat.init_density(*args)
+        assert ei.value.code == P.lbm.LBM_EINVAL
+        assert np.array_equal(lat.read_populations(), before) and lat.status(0) == 0
+    lat.step(3)
+    after = lat.read_populations()
+    fresh, _, _ = _lattice(P, nx, ny, P.LBM_FP32, "cs")
+    fresh.step(5)
+    assert np.array_equal(fresh.read_populations(), after)
+    lat.close()
+    fresh.close()
