@@ -1242,9 +1242,8 @@ int lbm_batch_create(lbm_ctx** out, int n, const int* nx, const int* ny, int pre
         c->owns = true;
         c->buf_bytes = c->L.total;
     }
-    void* red = nullptr;
-    if (cudaHostAlloc(&red, 256 + kStageBytes, cudaHostAllocMapped) != cudaSuccess) {
-        cudaGetLastError();
+    void* const red = lbm::pinned_get(256 + kStageBytes);
+    if (!red) {
         lbm_destroy(c);
         return LBM_ENOMEM;
     }
@@ -1295,7 +1294,7 @@ int lbm_create(lbm_ctx** out, int nx, int ny, int precision, void* dev_buf, size
 void lbm_destroy(lbm_ctx* c) {
     if (!c) return;
     cudaSetDevice(c->device);
-    if (c->stream || c->buf) cudaStreamSynchronize(c->stream);
+    if (c->stream || c->buf) cudaStreamSynchronize(c->stream);   // also: nothing writes the pinned block any more
     drop_graphs(c);
     if (c->copy_stream) {
         cudaStreamSynchronize(c->copy_stream);
@@ -1303,7 +1302,7 @@ void lbm_destroy(lbm_ctx* c) {
     }
     for (auto& e : c->band_done)
         if (e) cudaEventDestroy(e);
-    if (c->h_red) cudaFreeHost(c->h_red);
+    lbm::pinned_put(c->h_red, 256 + kStageBytes);
     if (c->owns && c->buf) cudaFree(c->buf);
     delete c;
 }

@@ -29,6 +29,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -631,16 +632,17 @@ double uniform01(uint64_t& s) { return (splitmix(s) >> 11) * (1.0 / 900719925474
 
 struct lbm_mlp {
     int max_n = 0;
-    void *dev = nullptr, *host = nullptr;   // the device and the pinned memory that the buffers are in
+    void* dev = nullptr;     // the device memory that the buffers are in
     cudaStream_t st = nullptr;
     Norm norm{};
     float *P = nullptr, *M = nullptr, *V = nullptr, *X = nullptr, *Y = nullptr, *partials = nullptr,
-          *grad = nullptr, *io = nullptr;
-    // training: the sample orders, bias corrections and losses of a launch's
+          *grad = nullptr, *sum = nullptr, *io = nullptr;   // sum: the loss of a single gradient
+    // training (from the first call of it on): the sample orders, bias corrections and losses of a launch's
     // epochs, twice, so that the host prepares a launch while another runs
     int *order[2] = {}, *h_order[2] = {};
     float2 *corr[2] = {}, *h_corr[2] = {};
     float *loss[2] = {}, *h_loss[2] = {};
+    void *stage = nullptr, *h_stage = nullptr;   // device and pinned memory that these are in
     cudaEvent_t done[2] = {};
     float* h_io = nullptr;   // pinned and mapped: NI + NO floats of up to io_n samples, read and written by the kernels
     int io_n = 0;
@@ -660,6 +662,45 @@ constexpr int kIoMax = 1 << 16;       // samples of the pinned buffer at most
 constexpr int kClusterMax = 768;
 
 bool valid(lbm_mlp* m) { return m && m->P; }
+size_t io_bytes(const lbm_mlp* m) { return sizeof(float) * (NI + NO) * static_cast<size_t>(m->io_n); }
+
+// A block of memory cut into buffers, each a multiple of 16 bytes so that all
+// are aligned alike (with at == NULL: their sizes only).
+struct Cut {
+    char* at;
+    size_t used;
+    void* take(size_t bytes) {
+        void* p = at ? at + used : nullptr;
+        used += (bytes + 15) / 16 * 16;
+        return p;
+    }
+};
+
+// The buffers of training, made by its first call and kept.
+int ensure_stage(lbm_mlp* m) {
+    if (m->cap) return LBM_OK;
+    const size_t cap = std::max(m->max_n, kOrderMin);
+    auto cut = [&](Cut c, float2* (&corr)[2], int* (&order)[2], float* (&loss)[2]) {
+        for (int k = 0; k < 2; ++k) {
+            corr[k] = static_cast<float2*>(c.take(cap * sizeof(float2)));
+            order[k] = static_cast<int*>(c.take(cap * sizeof(int)));
+            loss[k] = static_cast<float*>(c.take(cap * sizeof(float)));
+        }
+        return c.used;
+    };
+    const size_t bytes = cut({nullptr, 0}, m->corr, m->order, m->loss);
+    bool ok = (m->stage || cudaMalloc(&m->stage, bytes) == cudaSuccess) &&
+              (m->h_stage || cudaMallocHost(&m->h_stage, bytes) == cudaSuccess);
+    for (auto& e : m->done) ok = ok && (e || cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess);
+    if (!ok) {
+        cudaGetLastError();
+        return LBM_ENOMEM;
+    }
+    cut({static_cast<char*>(m->stage), 0}, m->corr, m->order, m->loss);
+    cut({static_cast<char*>(m->h_stage), 0}, m->h_corr, m->h_order, m->h_loss);
+    m->cap = static_cast<int>(cap);
+    return LBM_OK;
+}
 
 // Standardised samples to the device; from pinned memory (n <= io_n) without
 // waiting, since every call waits for its stream before it returns.
@@ -690,12 +731,12 @@ float2 next_corr(lbm_mlp* m, float b1, float b2) {
 }
 
 // The launch of the training cluster.
-void train_config(lbm_mlp* m, cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr) {
+void train_config(cudaStream_t st, cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr) {
     cfg = {};
     cfg.gridDim = dim3(kC);
     cfg.blockDim = dim3(kT);
     cfg.dynamicSmemBytes = sizeof(TrainSmem);
-    cfg.stream = m->st;
+    cfg.stream = st;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = kC;
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
@@ -703,11 +744,43 @@ void train_config(lbm_mlp* m, cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr
     cfg.numAttrs = 1;
 }
 
+// The kernels' attributes on the current device, set by the first network
+// made on it, and whether it can hold the training cluster.
+bool prepare_kernels(bool* cluster) {
+    constexpr int kDevices = 64;
+    static std::mutex mu;
+    static int known[kDevices];   // 1: attributes set, no cluster; 2: cluster too
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lock(mu);
+    int k = dev >= 0 && dev < kDevices ? known[dev] : 0;
+    if (!k) {
+        auto room = [](auto fn, size_t bytes) {
+            return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes)) ==
+                   cudaSuccess;
+        };
+        if (!room(k_train, sizeof(TrainSmem)) || !room(k_grad, sizeof(GradSmem)) || !room(k_predict, sizeof(GradSmem)) ||
+            !room(k_invert<1>, sizeof(GradSmem)) || !room(k_invert<2>, sizeof(GradSmem)) ||
+            !room(k_invert<3>, sizeof(GradSmem)) ||
+            cudaFuncSetAttribute(k_train, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+            return false;
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr;
+        int n = 0;
+        train_config(nullptr, cfg, attr);
+        k = cudaOccupancyMaxActiveClusters(&n, &k_train, &cfg) == cudaSuccess && n > 0 ? 2 : 1;
+        if (k == 1) cudaGetLastError();
+        if (dev >= 0 && dev < kDevices) known[dev] = k;
+    }
+    *cluster = k == 2;
+    return true;
+}
+
 // Epochs in the cluster, enqueued.
 cudaError_t launch_train(lbm_mlp* m, const TrainArgs& a) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
-    train_config(m, cfg, attr);
+    train_config(m->st, cfg, attr);
     return cudaLaunchKernelEx(&cfg, &k_train, a);
 }
 
@@ -735,72 +808,33 @@ int lbm_mlp_create(lbm_mlp** out, int max_samples, unsigned long long seed, void
     lbm_mlp* m = new lbm_mlp();
     m->max_n = max_samples;
     m->st = static_cast<cudaStream_t>(stream);
-    const size_t max_rows = std::min((max_samples + kS - 1) / kS, kRows), cap = std::max(max_samples, kOrderMin);
-    const size_t rows = static_cast<size_t>(max_samples);
-    m->cap = static_cast<int>(cap);
+    const size_t max_rows = std::min((max_samples + kS - 1) / kS, kRows), rows = static_cast<size_t>(max_samples);
     m->io_n = std::min(max_samples, kIoMax);
-    // one block of device memory and one of pinned memory, cut into the
-    // buffers (each a multiple of 16 bytes, so that all are aligned alike)
-    struct Cut {
-        char* at;
-        size_t used;
-        void* take(size_t bytes) {
-            void* p = at ? at + used : nullptr;
-            used += (bytes + 15) / 16 * 16;
-            return p;
-        }
-    };
-    auto stage = [&](Cut& c, float2*& corr, int*& order, float*& loss) {
-        corr = static_cast<float2*>(c.take(cap * sizeof(float2)));
-        order = static_cast<int*>(c.take(cap * sizeof(int)));
-        loss = static_cast<float*>(c.take(cap * sizeof(float)));
-    };
-    auto cut_device = [&](Cut c) {
+    auto cut = [&](Cut c) {
         auto floats = [&](size_t n) { return static_cast<float*>(c.take(n * sizeof(float))); };
         m->P = floats(NP);
         m->M = floats(NP);
         m->V = floats(NP);
         m->grad = floats(NP);
+        m->sum = floats(1);
         m->X = floats(NI * rows);
         m->Y = floats(NO * rows);
         m->io = floats(NO * rows);
         m->partials = floats(NPL * max_rows);
-        for (int k = 0; k < 2; ++k) stage(c, m->corr[k], m->order[k], m->loss[k]);
         return c.used;
     };
-    auto cut_host = [&](Cut c) {
-        m->h_io = static_cast<float*>(c.take(sizeof(float) * (NI + NO) * m->io_n));
-        for (int k = 0; k < 2; ++k) stage(c, m->h_corr[k], m->h_order[k], m->h_loss[k]);
-        return c.used;
-    };
-    bool ok = cudaMalloc(&m->dev, cut_device({nullptr, 0})) == cudaSuccess &&
-              cudaHostAlloc(&m->host, cut_host({nullptr, 0}), cudaHostAllocMapped) == cudaSuccess;
-    for (int k = 0; k < 2 && ok; ++k) ok = cudaEventCreateWithFlags(&m->done[k], cudaEventDisableTiming) == cudaSuccess;
-    if (ok) {
-        cut_device({static_cast<char*>(m->dev), 0});
-        cut_host({static_cast<char*>(m->host), 0});
-    }
+    const bool ok = cudaMalloc(&m->dev, cut({nullptr, 0})) == cudaSuccess &&
+                    (m->h_io = static_cast<float*>(lbm::pinned_get(io_bytes(m)))) != nullptr;
+    cut({ok ? static_cast<char*>(m->dev) : nullptr, 0});
     if (!ok) {
         cudaGetLastError();
         lbm_mlp_destroy(m);
         return LBM_ENOMEM;
     }
-    auto room = [](auto fn, size_t bytes) {
-        return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes)) == cudaSuccess;
-    };
-    if (!room(k_train, sizeof(TrainSmem)) || !room(k_grad, sizeof(GradSmem)) || !room(k_predict, sizeof(GradSmem)) ||
-        !room(k_invert<1>, sizeof(GradSmem)) || !room(k_invert<2>, sizeof(GradSmem)) ||
-        !room(k_invert<3>, sizeof(GradSmem)) ||
-        cudaFuncSetAttribute(k_train, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    if (!prepare_kernels(&m->cluster)) {
         lbm_mlp_destroy(m);
         return LBM_ECUDA;
     }
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr;
-    int clusters = 0;
-    train_config(m, cfg, attr);
-    m->cluster = cudaOccupancyMaxActiveClusters(&clusters, &k_train, &cfg) == cudaSuccess && clusters > 0;
-    if (!m->cluster) cudaGetLastError();
     // Glorot-uniform weights from a seeded splitmix64 stream, zero biases
     std::vector<float> p(NP, 0.0f);
     uint64_t s = seed;
@@ -824,9 +858,11 @@ int lbm_mlp_create(lbm_mlp** out, int max_samples, unsigned long long seed, void
 
 void lbm_mlp_destroy(lbm_mlp* m) {
     if (!m) return;
-    if (m->P) cudaStreamSynchronize(m->st);
+    if (m->P) cudaStreamSynchronize(m->st);   // also: nothing uses the pinned memory any more
     if (m->dev) cudaFree(m->dev);
-    if (m->host) cudaFreeHost(m->host);
+    if (m->stage) cudaFree(m->stage);
+    if (m->h_stage) cudaFreeHost(m->h_stage);
+    lbm::pinned_put(m->h_io, io_bytes(m));
     for (cudaEvent_t e : m->done)
         if (e) cudaEventDestroy(e);
     delete m;
@@ -869,8 +905,8 @@ int lbm_mlp_loss_grad(lbm_mlp* m, const float* X, const float* Y, int n, float* 
     if (!valid(m) || !X || !Y || n < 1 || n > m->max_n) return LBM_EINVAL;
     int rc = standardise_upload(m, X, Y, n);
     if (rc) return rc;
-    if (grad_pass(m, nullptr, 0, n, false, 0, 0, 0, 0, make_float2(1, 1), m->loss[0]) != cudaSuccess) return LBM_ECUDA;
-    if (loss && cudaMemcpyAsync(loss, m->loss[0], sizeof(float), cudaMemcpyDeviceToHost, m->st) != cudaSuccess)
+    if (grad_pass(m, nullptr, 0, n, false, 0, 0, 0, 0, make_float2(1, 1), m->sum) != cudaSuccess) return LBM_ECUDA;
+    if (loss && cudaMemcpyAsync(loss, m->sum, sizeof(float), cudaMemcpyDeviceToHost, m->st) != cudaSuccess)
         return LBM_ECUDA;
     if (grad && cudaMemcpyAsync(grad, m->grad, NP * sizeof(float), cudaMemcpyDeviceToHost, m->st) != cudaSuccess)
         return LBM_ECUDA;
@@ -882,7 +918,7 @@ int lbm_mlp_adam_step(lbm_mlp* m, const float* X, const float* Y, int n, float l
     if (!valid(m) || !X || !Y || n < 1 || n > m->max_n || !(lr > 0)) return LBM_EINVAL;
     int rc = standardise_upload(m, X, Y, n);
     if (rc) return rc;
-    if (grad_pass(m, nullptr, 0, n, true, lr, beta1, beta2, eps, next_corr(m, beta1, beta2), m->loss[0]) != cudaSuccess)
+    if (grad_pass(m, nullptr, 0, n, true, lr, beta1, beta2, eps, next_corr(m, beta1, beta2), m->sum) != cudaSuccess)
         return LBM_ECUDA;
     return cudaStreamSynchronize(m->st) == cudaSuccess ? LBM_OK : LBM_ECUDA;
 }
@@ -890,7 +926,8 @@ int lbm_mlp_adam_step(lbm_mlp* m, const float* X, const float* Y, int n, float l
 int lbm_mlp_train(lbm_mlp* m, const float* X, const float* Y, int n, int epochs, int batch, float lr,
                   unsigned long long seed, float* loss_per_epoch) {
     if (!valid(m) || !X || !Y || n < 1 || n > m->max_n || epochs < 1 || batch < 1 || !(lr > 0)) return LBM_EINVAL;
-    int rc = standardise_upload(m, X, Y, n);
+    int rc = ensure_stage(m);
+    if (!rc) rc = standardise_upload(m, X, Y, n);
     if (rc) return rc;
     std::vector<int> order(n);
     for (int i = 0; i < n; ++i) order[i] = i;
