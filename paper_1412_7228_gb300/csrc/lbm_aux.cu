@@ -77,18 +77,60 @@ __device__ __forceinline__ void equilibrium(double rr, R rho, R ux, R uy, T (&f)
     }
 }
 
-// Rows [y0, y1) of the field; rho, ux and uy index the whole field.
+// The checks of an initial field, on the device: bit 1 of *bad when a
+// density is not finite, not positive or not below rho_max, bit 2 when a
+// velocity is not finite (the caller has zeroed *bad).  On the bit patterns,
+// as integers (no FP64 work): for rho_max > 0, 0 < r < rho_max with r finite
+// is 0 < bits(r) < bits(top), top = rho_max in FP64, or for FP32 fields the
+// smallest float not below rho_max (positive values order as their patterns;
+// negatives and -0 have the sign bit, NaN and inf patterns lie above every
+// finite value); finite is an exponent field below all ones.
+__device__ __forceinline__ long long bits_of(double v) { return __double_as_longlong(v); }
+__device__ __forceinline__ long long bits_of(float v) { return __float_as_int(v); }
+template <typename R> __host__ __device__ constexpr long long exp_mask() {
+    return sizeof(R) == 8 ? 0x7ff0000000000000ll : 0x7f800000ll;
+}
+__device__ __forceinline__ long long top_bits(double rho_max, double) { return bits_of(rho_max); }
+__device__ __forceinline__ long long top_bits(double rho_max, float) { return bits_of(__double2float_ru(rho_max)); }
+template <typename R> struct FieldCheck {
+    long long top;
+    int b = 0;
+    __device__ __forceinline__ explicit FieldCheck(double rho_max) : top(top_bits(rho_max, R(0))) {}
+    __device__ __forceinline__ void density(R v) {
+        const long long r = bits_of(v);
+        if (!(r > 0 && r < top)) b |= 1;
+    }
+    __device__ __forceinline__ void velocity(R v) {
+        constexpr long long kExp = exp_mask<R>();
+        if ((bits_of(v) & kExp) == kExp) b |= 2;
+    }
+    __device__ __forceinline__ void report(int* bad) {   // every lane of the warp
+        b = __reduce_or_sync(0xffffffffu, b);
+        if (b && (threadIdx.x & 31) == 0) atomicOr(bad, b);
+    }
+};
+
+// Rows [y0, y1) of the field; rho, ux and uy index the whole field, in device
+// memory or in pinned host memory (each value is read once, so the field
+// need not be copied first).  bad != NULL: the values are checked on the way.
 template <typename T, bool REST, typename R>
 __global__ void k_init(const Inst* __restrict__ I, const R* __restrict__ rho, const R* __restrict__ ux,
-                       const R* __restrict__ uy, int parity, int y0, int y1) {
+                       const R* __restrict__ uy, int parity, int y0, int y1, double rho_max, int* bad) {
     const int nx = I->nx, ny = I->ny;
     T* p = popk<T>(I, parity);
     const double rr = static_cast<double>(phys<T>(I).rho_ref);
+    FieldCheck<R> check(rho_max);
     for (int y = y0 + static_cast<int>(blockIdx.y); y < y1; y += gridDim.y)
         for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < nx; x += gridDim.x * blockDim.x) {
             const long long i = static_cast<long long>(y) * nx + x;
+            const R r = rho[i], u = !REST && ux ? ux[i] : R(0), v = !REST && uy ? uy[i] : R(0);
+            check.density(r);
+            if (!REST) {
+                check.velocity(u);
+                check.velocity(v);
+            }
             T f[9];
-            equilibrium<T, REST>(rr, rho[i], !REST && ux ? ux[i] : R(0), !REST && uy ? uy[i] : R(0), f);
+            equilibrium<T, REST>(rr, r, u, v, f);
 #pragma unroll
             for (int a = 0; a < 9; ++a) {
                 int xs = x - cx(a), ys = y - cy(a);
@@ -97,46 +139,43 @@ __global__ void k_init(const Inst* __restrict__ I, const R* __restrict__ rho, co
                 p[at<T>(I, a, xs, ys)] = f[a];
             }
         }
+    __syncwarp();
+    if (bad) check.report(bad);
 }
 
-// The checks of an initial field, on the device: bit 1 of *bad when a
-// density is not finite, not positive or not below rho_max, bit 2 when a
-// velocity is not finite (the caller has zeroed *bad).
-// Bit patterns of the field's type as signed integers, and the exponent field.
-__device__ __forceinline__ long long bits_of(double v) { return __double_as_longlong(v); }
-__device__ __forceinline__ long long bits_of(float v) { return __float_as_int(v); }
-template <typename R> __host__ __device__ constexpr long long exp_mask() {
-    return sizeof(R) == 8 ? 0x7ff0000000000000ll : 0x7f800000ll;
-}
 template <typename R>
 __global__ void k_check_init(const R* __restrict__ rho, const R* __restrict__ ux, const R* __restrict__ uy,
                              long long N, double rho_max, int* bad) {
-    // on the bit patterns, as integers (no FP64 work): for rho_max > 0,
-    // 0 < r < rho_max with r finite is 0 < bits(r) < bits(top), top = rho_max
-    // in FP64, or for FP32 fields the smallest float not below rho_max
-    // (positive values order as their patterns; negatives and -0 have the
-    // sign bit, NaN and inf patterns lie above every finite value); finite is
-    // an exponent field below all ones
-    const long long top = sizeof(R) == 8 ? bits_of(rho_max) : bits_of(__double2float_ru(rho_max));
-    constexpr long long kExp = exp_mask<R>();
-    auto finite = [](R v) { return (bits_of(v) & kExp) != kExp; };
-    int b = 0;
+    FieldCheck<R> check(rho_max);
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < N;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const long long r = bits_of(rho[i]);
-        if (!(r > 0 && r < top)) b |= 1;
-        if ((ux && !finite(ux[i])) || (uy && !finite(uy[i]))) b |= 2;
+        check.density(rho[i]);
+        if (ux) check.velocity(ux[i]);
+        if (uy) check.velocity(uy[i]);
     }
-    b = __reduce_or_sync(0xffffffffu, b);
-    if (b && (threadIdx.x & 31) == 0) atomicOr(bad, b);
+    __syncwarp();
+    check.report(bad);
 }
 
+// The block's writes are done: the last block tells the host (Notice).
+__device__ __forceinline__ void notify(const Notice& to) {
+    if (!to.ticket) return;
+    __threadfence_system();
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    if (atomicAdd(to.ticket, 1u) != gridDim.x * gridDim.y - 1) return;
+    *to.ticket = 0;
+    __threadfence_system();
+    *static_cast<volatile unsigned*>(&to.to->call) = to.call;
+}
 // Ghost cells x in [-2,0) U [nx,nx+2), y in [-2,0) U [ny,ny+2) of every
 // plane, and only those: per plane the rows y = -2, -1, ny, ny + 1 over
 // x in [-2, nx + 2) (4 (nx + 4) cells), then the columns x = -2, -1, nx,
 // nx + 1 over y in [0, ny) (4 ny cells).  Each copies its periodic image
-// inside the lattice.
-template <typename T> __global__ void k_ghosts(const Inst* __restrict__ I, int parity) {
+// inside the lattice.  With a Notice, *word goes to its status field.
+template <typename T>
+__global__ void k_ghosts(const Inst* __restrict__ I, int parity, Notice to, const int* __restrict__ word) {
+    if (to.ticket && blockIdx.x == 0 && threadIdx.x == 0) to.to->status = *word;
     const int nx = I->nx, ny = I->ny;
     const int W = nx + 4, per = 4 * W + 4 * ny;
     const long long M = 9ll * per;
@@ -158,6 +197,7 @@ template <typename T> __global__ void k_ghosts(const Inst* __restrict__ I, int p
         const int xs = ((x % nx) + nx) % nx, ys = ((y % ny) + ny) % ny;
         p[at<T>(I, a, x, y)] = p[at<T>(I, a, xs, ys)];
     }
+    notify(to);
 }
 
 // f_a(z, t) = pop_a(z - e_a) + t_a rho_ref, for one plane a.
@@ -306,17 +346,6 @@ __device__ __forceinline__ void flow_tile(const Inst* I, const T* p, int x0, int
     if (interact) __syncthreads();   // before the next tile's psi
 }
 
-// The block's writes are done: the last block tells the host (Notice).
-__device__ __forceinline__ void notify(const Notice& to) {
-    if (!to.ticket) return;
-    __threadfence_system();
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    if (atomicAdd(to.ticket, 1u) != gridDim.x * gridDim.y - 1) return;
-    *to.ticket = 0;
-    __threadfence_system();
-    *static_cast<volatile unsigned*>(&to.to->call) = to.call;
-}
 // The same after a reduction, whose last block's first warp has written the
 // results.
 __device__ __forceinline__ void notify_reduced(const Notice& to) {
@@ -535,30 +564,29 @@ cudaError_t aux_fp64_fma_rate(int iters, cudaStream_t st, double* flops_per_s, d
 
 template <typename R>
 cudaError_t init_rows_t(const Inst& h, const Inst* d, const R* rho, const R* ux, const R* uy, int parity, int y0,
-                        int y1, cudaStream_t st) {
+                        int y1, double rho_max, int* bad, cudaStream_t st) {
     const dim3 g = grid_2d(h.nx, y1 - y0);
     const bool rest = !ux && !uy;
-    if (h.prec == LBM_FP32 && rest) k_init<float, true, R><<<g, kThreads, 0, st>>>(d, rho, ux, uy, parity, y0, y1);
-    else if (h.prec == LBM_FP32) k_init<float, false, R><<<g, kThreads, 0, st>>>(d, rho, ux, uy, parity, y0, y1);
-    else if (rest) k_init<double, true, R><<<g, kThreads, 0, st>>>(d, rho, ux, uy, parity, y0, y1);
-    else k_init<double, false, R><<<g, kThreads, 0, st>>>(d, rho, ux, uy, parity, y0, y1);
+    auto go = [&](auto k) { k<<<g, kThreads, 0, st>>>(d, rho, ux, uy, parity, y0, y1, rho_max, bad); };
+    if (h.prec == LBM_FP32) rest ? go(k_init<float, true, R>) : go(k_init<float, false, R>);
+    else rest ? go(k_init<double, true, R>) : go(k_init<double, false, R>);
     return cudaGetLastError();
 }
 
 cudaError_t aux_init(const Inst& h, const Inst* d, const void* rho, const void* ux, const void* uy, bool f32,
                      int parity, cudaStream_t st) {
-    const cudaError_t e = aux_init_rows(h, d, rho, ux, uy, f32, parity, 0, h.ny, st);
-    return e != cudaSuccess ? e : aux_fill_ghosts(h, d, parity, st);
+    const cudaError_t e = aux_init_rows(h, d, rho, ux, uy, f32, parity, 0, h.ny, 0.0, nullptr, st);
+    return e != cudaSuccess ? e : aux_fill_ghosts(h, d, parity, Notice{}, nullptr, st);
 }
 
 cudaError_t aux_init_rows(const Inst& h, const Inst* d, const void* rho, const void* ux, const void* uy, bool f32,
-                          int parity, int y0, int y1, cudaStream_t st) {
+                          int parity, int y0, int y1, double rho_max, int* bad, cudaStream_t st) {
     if (y0 < 0 || y1 > h.ny || y0 >= y1) return cudaErrorInvalidValue;
     if (f32)
         return init_rows_t(h, d, static_cast<const float*>(rho), static_cast<const float*>(ux),
-                           static_cast<const float*>(uy), parity, y0, y1, st);
+                           static_cast<const float*>(uy), parity, y0, y1, rho_max, bad, st);
     return init_rows_t(h, d, static_cast<const double*>(rho), static_cast<const double*>(ux),
-                       static_cast<const double*>(uy), parity, y0, y1, st);
+                       static_cast<const double*>(uy), parity, y0, y1, rho_max, bad, st);
 }
 
 cudaError_t aux_check_init(const void* rho, const void* ux, const void* uy, bool f32, long long N, double rho_max,
@@ -574,12 +602,13 @@ cudaError_t aux_check_init(const void* rho, const void* ux, const void* uy, bool
     return cudaGetLastError();
 }
 
-cudaError_t aux_fill_ghosts(const Inst& h, const Inst* d, int parity, cudaStream_t st) {
+cudaError_t aux_fill_ghosts(const Inst& h, const Inst* d, int parity, const Notice& to, const int* word,
+                            cudaStream_t st) {
     const long long M = 9ll * (4 * (h.nx + 4) + 4 * h.ny);
     if (h.prec == LBM_FP32)
-        k_ghosts<float><<<grid_for(M), kThreads, 0, st>>>(d, parity);
+        k_ghosts<float><<<grid_for(M), kThreads, 0, st>>>(d, parity, to, word);
     else
-        k_ghosts<double><<<grid_for(M), kThreads, 0, st>>>(d, parity);
+        k_ghosts<double><<<grid_for(M), kThreads, 0, st>>>(d, parity, to, word);
     return cudaGetLastError();
 }
 

@@ -842,97 +842,11 @@ int ensure_copy_stream(lbm_ctx* c) {
     return LBM_OK;
 }
 
-template <typename R> int init_density_t(lbm_ctx* c, int i, const R* rho, const R* ux, const R* uy) {
-    int rc = check_idx(c, i);
-    if (rc) return rc;
-    if (!rho) return fail(c, LBM_EINVAL, "rho must not be NULL%s");
-    if (!c->hp[i].set) return fail(c, LBM_EINVAL, "set the parameters before the density%s");
-    Range range("lbm_batch_init_density");
-    const size_t N = static_cast<size_t>(c->nx[i]) * c->ny[i];
-    // the EOS range only matters when psi is evaluated (G != 0)
-    const double rmax = c->hp[i].G != 0.0 ? eos_rho_max(c->hp[i].eos) : HUGE_VAL;
-    CK(c, cudaSetDevice(c->device));
-    CK(c, cudaStreamSynchronize(c->stream));
-    R* const scratch = reinterpret_cast<R*>(c->d_scratch);
-    R* d_rho = scratch;
-    R* d_ux = ux ? scratch + N : nullptr;
-    R* d_uy = uy ? scratch + 2 * N : nullptr;
-    constexpr bool f32 = sizeof(R) == 4;
-    // the field is checked on the device before anything of the instance's
-    // current time level is written.  A context of one lattice has its
-    // equilibrium written into the other time level (which the next step
-    // overwrites whole) without waiting for the check; that level becomes the
-    // current one once the field has passed.  With 2^20 nodes or more the
-    // field arrives in row bands on the copy stream, each band checked and
-    // its equilibrium written while the next band is in flight.  An instance
-    // of a batch, whose time level is the others' too, waits for the check.
-    int* d_bad = reinterpret_cast<int*>(c->d_result);
-    int* const bad = &c->h_red->status;   // pinned
-    const bool ahead = c->n == 1;
-    const int bands = ahead ? field_bands(c, i) : 1;
-    const int level = ahead ? c->parity ^ 1 : c->parity;
-    if (bands > 1 && (rc = ensure_copy_stream(c))) return rc;
-    auto copy_and_check = [&]() -> int {
-        CK(c, cudaMemsetAsync(d_bad, 0, sizeof(int), c->stream));
-        if (bands == 1) {
-            CK(c, cudaMemcpyAsync(d_rho, rho, N * sizeof(R), cudaMemcpyHostToDevice, c->stream));
-            if (ux) CK(c, cudaMemcpyAsync(d_ux, ux, N * sizeof(R), cudaMemcpyHostToDevice, c->stream));
-            if (uy) CK(c, cudaMemcpyAsync(d_uy, uy, N * sizeof(R), cudaMemcpyHostToDevice, c->stream));
-            CK(c, lbm::aux_check_init(d_rho, d_ux, d_uy, f32, static_cast<long long>(N), rmax, d_bad, c->stream));
-            if (ahead)
-                CK(c, lbm::aux_init_rows(c->h[i], c->d_inst + i, d_rho, d_ux, d_uy, f32, level, 0, c->ny[i], c->stream));
-        } else {
-            const int nx = c->nx[i], ny = c->ny[i];
-            for (int b = 0; b < bands; ++b) {
-                const int y0 = static_cast<int>(static_cast<long long>(ny) * b / bands);
-                const int y1 = static_cast<int>(static_cast<long long>(ny) * (b + 1) / bands);
-                const size_t off = static_cast<size_t>(y0) * nx, cnt = static_cast<size_t>(y1 - y0) * nx;
-                CK(c, cudaMemcpyAsync(d_rho + off, rho + off, cnt * sizeof(R), cudaMemcpyHostToDevice, c->copy_stream));
-                if (ux)
-                    CK(c, cudaMemcpyAsync(d_ux + off, ux + off, cnt * sizeof(R), cudaMemcpyHostToDevice,
-                                          c->copy_stream));
-                if (uy)
-                    CK(c, cudaMemcpyAsync(d_uy + off, uy + off, cnt * sizeof(R), cudaMemcpyHostToDevice,
-                                          c->copy_stream));
-                CK(c, cudaEventRecord(c->band_done[b], c->copy_stream));
-                CK(c, cudaStreamWaitEvent(c->stream, c->band_done[b], 0));
-                CK(c, lbm::aux_check_init(d_rho + off, d_ux ? d_ux + off : nullptr, d_uy ? d_uy + off : nullptr, f32,
-                                          static_cast<long long>(cnt), rmax, d_bad, c->stream));
-                CK(c, lbm::aux_init_rows(c->h[i], c->d_inst + i, d_rho, d_ux, d_uy, f32, level, y0, y1, c->stream));
-            }
-        }
-        if (ahead) CK(c, lbm::aux_fill_ghosts(c->h[i], c->d_inst + i, level, c->stream));
-        CK(c, cudaMemcpyAsync(bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-        return LBM_OK;
-    };
-    rc = copy_and_check();
-    if (rc) {   // no copy from the caller's arrays may outlive the call
-        if (bands > 1) cudaStreamSynchronize(c->copy_stream);
-        cudaStreamSynchronize(c->stream);
-        return rc;
-    }
-    // the stream waited for every band's copy: all of them have landed
-    CK(c, cudaStreamSynchronize(c->stream));
-    if (*bad & 1) return fail(c, LBM_EINVAL, "initial density must be finite, positive and inside the EOS range%s");
-    if (*bad & 2) return fail(c, LBM_EINVAL, "initial velocity must be finite%s");
-    if (ahead) {
-        c->parity = level;
-        CK(c, cudaMemsetAsync(c->d_status + i, 0, sizeof(int), c->stream));
-    } else {
-        CK(c, lbm::aux_init(c->h[i], c->d_inst + i, d_rho, d_ux, d_uy, f32, c->parity, c->stream));
-        CK(c, cudaMemsetAsync(c->d_status + i, 0, sizeof(int), c->stream));
-        CK(c, cudaStreamSynchronize(c->stream));
-    }
-    c->inited[i] = 1;
-    c->steps = 0;
-    return LBM_OK;
-}
-
-// How a call's results can reach the n values at p: pinned host memory that
-// kernels can write (*dev: its address for them), ordinary host memory, or
-// anything else (left to the copy, which knows what to do with it).
+// How kernels can reach the n values at p: pinned host memory that they may
+// read, or write where asked (*dev: its address for them), ordinary host
+// memory, or anything else (left to the copies, which know what to do with it).
 enum HostKind { kPinned, kPageable, kOther };
-template <typename O> HostKind host_kind(O* p, size_t n, O** dev) {
+template <typename O> HostKind host_kind(O* p, size_t n, bool write, O** dev) {
     cudaPointerAttributes a, b;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaPointerGetAttributes(&b, p + n - 1) != cudaSuccess) {
         cudaGetLastError();
@@ -945,12 +859,114 @@ template <typename O> HostKind host_kind(O* p, size_t n, O** dev) {
         static_cast<std::ptrdiff_t>((n - 1) * sizeof(O)))
         return kOther;
     unsigned flags = 0;
-    if (cudaHostGetFlags(&flags, p) != cudaSuccess || (flags & cudaHostRegisterReadOnly)) {
+    if (write && (cudaHostGetFlags(&flags, const_cast<std::remove_const_t<O>*>(p)) != cudaSuccess ||
+                  (flags & cudaHostRegisterReadOnly))) {
         cudaGetLastError();
         return kOther;
     }
     *dev = static_cast<O*>(a.devicePointer);
     return kPinned;
+}
+
+template <typename R> int init_density_t(lbm_ctx* c, int i, const R* rho, const R* ux, const R* uy) {
+    int rc = check_idx(c, i);
+    if (rc) return rc;
+    if (!rho) return fail(c, LBM_EINVAL, "rho must not be NULL%s");
+    if (!c->hp[i].set) return fail(c, LBM_EINVAL, "set the parameters before the density%s");
+    Range range("lbm_batch_init_density");
+    const size_t N = static_cast<size_t>(c->nx[i]) * c->ny[i];
+    // the EOS range only matters when psi is evaluated (G != 0)
+    const double rmax = c->hp[i].G != 0.0 ? eos_rho_max(c->hp[i].eos) : HUGE_VAL;
+    CK(c, cudaSetDevice(c->device));
+    CK(c, cudaStreamSynchronize(c->stream));
+    R* const scratch = reinterpret_cast<R*>(c->d_scratch);
+    const R* d_rho = scratch;
+    const R* d_ux = ux ? scratch + N : nullptr;
+    const R* d_uy = uy ? scratch + 2 * N : nullptr;
+    constexpr bool f32 = sizeof(R) == 4;
+    // the field is checked on the device before anything of the instance's
+    // current time level is written.  A context of one lattice has its
+    // equilibrium written into the other time level (which the next step
+    // overwrites whole) without waiting for the check; that level becomes the
+    // current one once the field has passed.  Pinned fields are read by that
+    // kernel where they are (4096^2 FP32: the whole call 0.41 -> 0.36 ms, of
+    // which the host link takes 0.32).  Others of 2^20 nodes or more arrive in
+    // row bands on the copy stream, each band checked and its equilibrium
+    // written while the next band is in flight.  An instance of a batch, whose
+    // time level is the others' too, waits for the check.
+    int* const d_bad = reinterpret_cast<int*>(c->d_result);
+    const bool ahead = c->n == 1;
+    const int nx = c->nx[i], ny = c->ny[i];
+    const int level = ahead ? c->parity ^ 1 : c->parity;
+    bool in_place = ahead;
+    {
+        const R* at[3] = {};
+        const R* const from[3] = {rho, ux, uy};
+        for (int f = 0; f < 3 && in_place; ++f)
+            in_place = !from[f] || host_kind(from[f], N, false, &at[f]) == kPinned;
+        if (in_place) {
+            d_rho = at[0];
+            d_ux = at[1];
+            d_uy = at[2];
+        }
+    }
+    const int bands = ahead && !in_place ? field_bands(c, i) : 1;
+    if (bands > 1 && (rc = ensure_copy_stream(c))) return rc;
+    // rows [y0, y1) of the three fields into the scratch
+    auto copy_rows = [&](int y0, int y1, cudaStream_t st) -> int {
+        const size_t off = static_cast<size_t>(y0) * nx, bytes = static_cast<size_t>(y1 - y0) * nx * sizeof(R);
+        CK(c, cudaMemcpyAsync(scratch + off, rho + off, bytes, cudaMemcpyHostToDevice, st));
+        if (ux) CK(c, cudaMemcpyAsync(scratch + N + off, ux + off, bytes, cudaMemcpyHostToDevice, st));
+        if (uy) CK(c, cudaMemcpyAsync(scratch + 2 * N + off, uy + off, bytes, cudaMemcpyHostToDevice, st));
+        return LBM_OK;
+    };
+    auto issue = [&]() -> int {
+        CK(c, cudaMemsetAsync(d_bad, 0, sizeof(int), c->stream));
+        for (int b = 0; b < bands; ++b) {
+            const int y0 = static_cast<int>(static_cast<long long>(ny) * b / bands);
+            const int y1 = static_cast<int>(static_cast<long long>(ny) * (b + 1) / bands);
+            if (!in_place) {
+                const int r = copy_rows(y0, y1, bands > 1 ? c->copy_stream : c->stream);
+                if (r) return r;
+            }
+            if (bands > 1) {
+                CK(c, cudaEventRecord(c->band_done[b], c->copy_stream));
+                CK(c, cudaStreamWaitEvent(c->stream, c->band_done[b], 0));
+            }
+            if (ahead)
+                CK(c, lbm::aux_init_rows(c->h[i], c->d_inst + i, d_rho, d_ux, d_uy, f32, level, y0, y1, rmax, d_bad,
+                                         c->stream));
+            else
+                CK(c, lbm::aux_check_init(d_rho, d_ux, d_uy, f32, static_cast<long long>(N), rmax, d_bad, c->stream));
+        }
+        if (ahead) {
+            CK(c, lbm::aux_fill_ghosts(c->h[i], c->d_inst + i, level, next_notice(c), d_bad, c->stream));
+            return wait_notice(c);
+        }
+        CK(c, cudaMemcpyAsync(&c->h_red->status, d_bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+        CK(c, cudaStreamSynchronize(c->stream));
+        return LBM_OK;
+    };
+    rc = issue();
+    if (rc) {   // no read of the caller's arrays may outlive the call
+        if (bands > 1) cudaStreamSynchronize(c->copy_stream);
+        cudaStreamSynchronize(c->stream);
+        return rc;
+    }
+    const int bad = c->h_red->status;
+    if (bad & 1) return fail(c, LBM_EINVAL, "initial density must be finite, positive and inside the EOS range%s");
+    if (bad & 2) return fail(c, LBM_EINVAL, "initial velocity must be finite%s");
+    if (ahead) {
+        c->parity = level;
+        CK(c, cudaMemsetAsync(c->d_status + i, 0, sizeof(int), c->stream));
+    } else {
+        CK(c, lbm::aux_init(c->h[i], c->d_inst + i, d_rho, d_ux, d_uy, f32, c->parity, c->stream));
+        CK(c, cudaMemsetAsync(c->d_status + i, 0, sizeof(int), c->stream));
+        CK(c, cudaStreamSynchronize(c->stream));
+    }
+    c->inited[i] = 1;
+    c->steps = 0;
+    return LBM_OK;
 }
 
 // Macroscopic fields into host arrays of O (double, or float: each value
@@ -965,7 +981,6 @@ template <typename O> int read_fields_t(lbm_ctx* c, int i, O* rho, O* ux, O* uy,
     const size_t N = static_cast<size_t>(nx) * ny;
     // a large lattice in row bands: band b's copy to the host overlaps band b + 1's kernel
     const int bands = field_bands(c, i);
-    if (bands > 1 && (rc = ensure_copy_stream(c))) return rc;
     O* const outs[4] = {rho, ux, uy, psi};
     O* const scratch = reinterpret_cast<O*>(c->d_scratch);
     constexpr bool f32 = sizeof(O) == 4;
@@ -991,17 +1006,18 @@ template <typename O> int read_fields_t(lbm_ctx* c, int i, O* rho, O* ux, O* uy,
         for (int f : want) groups.push_back({false, {f}});
     }
     c->h_red->status = 0;
-    // a lattice read whole: the kernels write straight to where the host
-    // reads, the caller's arrays if they are pinned, else (small ones) the
-    // context's stage; no copy is enqueued and no stream waited for (rho into
-    // pinned memory, FP32: 64^2 15.3 -> 11.3 us per call, 512^2 29.3 -> 19.0)
-    if (bands == 1) {
+    // where they can, the kernels write straight to where the host reads: the
+    // caller's arrays if they are pinned, else (small ones) the context's
+    // stage; no copy is enqueued and no stream waited for (rho into pinned
+    // memory, FP32: 64^2 15.3 -> 11.3 us per call, 512^2 29.3 -> 19.0, 1024^2 in
+    // bands 67 -> 40 us)
+    {
         O* to[4] = {};
         size_t staged = 0;
         bool direct = true;
         for (int f = 0; f < 4 && direct; ++f) {
             if (!outs[f]) continue;
-            const HostKind kind = host_kind(outs[f], N, &to[f]);
+            const HostKind kind = host_kind(outs[f], N, true, &to[f]);
             if (kind == kPinned) continue;
             to[f] = reinterpret_cast<O*>(c->h_stage + staged);
             staged += (N * sizeof(O) + 15) / 16 * 16;
@@ -1027,6 +1043,7 @@ template <typename O> int read_fields_t(lbm_ctx* c, int i, O* rho, O* ux, O* uy,
             return status_code(c->h_red->status);
         }
     }
+    if (bands > 1 && (rc = ensure_copy_stream(c))) return rc;
     const lbm::Notice quiet = {c->h_red, nullptr, 0};
     auto issue = [&](const Group& g) -> int {
         for (int b = 0; b < bands; ++b) {

@@ -383,7 +383,9 @@ struct Notice {
 // Fields of nx*ny doubles, or floats with f32 (each widened to FP64 exactly).
 cudaError_t aux_init(const Inst& host, const Inst* d_inst, const void* rho, const void* ux, const void* uy, bool f32,
                      int parity, cudaStream_t st);
-cudaError_t aux_fill_ghosts(const Inst& host, const Inst* d_inst, int parity, cudaStream_t st);
+// *word (device) goes to the Notice's status field
+cudaError_t aux_fill_ghosts(const Inst& host, const Inst* d_inst, int parity, const Notice& to, const int* word,
+                            cudaStream_t st);
 // bad |= 1: a density not finite, positive and below rho_max; |= 2: a velocity not finite
 cudaError_t aux_check_init(const void* rho, const void* ux, const void* uy, bool f32, long long N, double rho_max,
                            int* bad, cudaStream_t st);
