@@ -11,7 +11,7 @@
 namespace lbm {
 namespace {
 
-constexpr int kThreads = kRedThreads;
+constexpr int kThreads = 256;
 
 // Lattice weights t_a of the D2Q9 equilibrium (4/9, 1/9, 1/36).
 __device__ __forceinline__ double tw(int a) { return a == 0 ? 4.0 / 9.0 : (a < 5 ? 1.0 / 9.0 : 1.0 / 36.0); }
@@ -288,25 +288,30 @@ __device__ __forceinline__ void node_j(const double (&v)[9], double& jx, double&
 // instructions instead of 700 (the FP64 pipe is the bound: 19 clocks of an
 // SM per warp instruction).  32 x 16 nodes: two per thread, a ring of 612
 // nodes in 20 warp passes for 16 of the tile's own.  FP32 statistics of
-// 1024^2: 1113 -> 180 us per call, of 256^2: 149 -> 30; the two velocity
+// 1024^2: 1113 -> 177 us per call, of 256^2: 149 -> 27; the two velocity
 // components of 1531 x 1117: 2 x 1709 -> 277 us, rho and psi with them.
-constexpr int kFlowX = 32, kFlowY = 16, kFlowW = kFlowX + 2, kFlowH = kFlowY + 2;
-struct FlowTile {
-    double psi[kFlowH][kFlowW], h[kFlowH][kFlowW], rho[kFlowH][kFlowW];   // h: hF psi^2, as in the step kernels
+// Lattices that leave SMs idle (up to 128^2) take 32 x 4 tiles of 128 threads,
+// whose larger ring costs less than the longer chain (statistics of 64^2: 20.8
+// us on the device with 32 x 16 tiles, 11.8 with 32 x 4).
+constexpr int kFlowX = 32, kFlowW = kFlowX + 2;
+template <int NT> struct FlowTile {
+    static constexpr int Y = NT == 128 ? 4 : 16, H = Y + 2;
+    double psi[H][kFlowW], h[H][kFlowW], rho[H][kFlowW];   // h: hF psi^2, as in the step kernels
 };
 
 // rho, velocity (rho u = sum f e + F/2, F of Eq. 9) and psi of the nodes
 // of tile (x0, y0), rows below y1, given to use(x, y, rho, ux, uy, psi) by
-// the thread that owns each; every thread of the block (kThreads) calls it.
-template <typename T, typename Use>
-__device__ __forceinline__ void flow_tile(const Inst* I, const T* p, int x0, int y0, int y1, FlowTile& S, Use use) {
+// the thread that owns each; every thread of the block (NT) calls it.
+template <int NT, typename T, typename Use>
+__device__ __forceinline__ void flow_tile(const Inst* I, const T* p, int x0, int y0, int y1, FlowTile<NT>& S, Use use) {
+    constexpr int kFlowY = FlowTile<NT>::Y, kFlowH = FlowTile<NT>::H;
     const Phys<double>& P = I->pd;
     const int nx = I->nx, ny = I->ny, interact = P.interact;
     const int tid = threadIdx.x;
     if (interact) {
         const LawFp64 law(P, true);
         const int w = min(kFlowX, nx - x0) + 2, h = min(kFlowY, y1 - y0) + 2;
-        for (int e = tid; e < kFlowW * kFlowH; e += kThreads) {
+        for (int e = tid; e < kFlowW * kFlowH; e += NT) {
             const int j = e / kFlowW, i = e - j * kFlowW;
             if (i >= w || j >= h) continue;
             int x = x0 + i - 1, y = y0 + j - 1;
@@ -322,7 +327,7 @@ __device__ __forceinline__ void flow_tile(const Inst* I, const T* p, int x0, int
     }
     const double cF = P.cF;
     const int i = tid % kFlowX + 1, x = x0 + i - 1;
-    for (int j = tid / kFlowX + 1; j <= kFlowY; j += kThreads / kFlowX) {
+    for (int j = tid / kFlowX + 1; j <= kFlowY; j += NT / kFlowX) {
         const int y = y0 + j - 1;
         if (x >= nx || y >= y1) continue;
         T v[9];
@@ -344,14 +349,6 @@ __device__ __forceinline__ void flow_tile(const Inst* I, const T* p, int x0, int
         use(x, y, r, quotient(jx, inv, r), quotient(jy, inv, r), ps);
     }
     if (interact) __syncthreads();   // before the next tile's psi
-}
-
-// The same after a reduction, whose last block's first warp has written the
-// results.
-__device__ __forceinline__ void notify_reduced(const Notice& to) {
-    __threadfence_system();
-    __syncwarp(0xffu);
-    if (threadIdx.x == 0) *static_cast<volatile unsigned*>(&to.to->call) = to.call;
 }
 
 // rho or psi of the nodes, one field per launch (FIELD 0 rho, 3 psi): the
@@ -376,17 +373,18 @@ __global__ void k_field(const Inst* __restrict__ I, int parity, int y0, int y1, 
 
 // The velocity components and, where asked for, rho and psi of rows [y0, y1)
 // in one pass (any output may be NULL).
-template <typename T, typename O>
-__global__ void __launch_bounds__(kThreads) k_flow(const Inst* __restrict__ I, int parity, int y0, int y1,
+template <int NT, typename T, typename O>
+__global__ void __launch_bounds__(NT) k_flow(const Inst* __restrict__ I, int parity, int y0, int y1,
                                                    O* __restrict__ rho, O* __restrict__ ux, O* __restrict__ uy,
                                                    O* __restrict__ psi, Notice to) {
-    __shared__ FlowTile S;
+    __shared__ FlowTile<NT> S;
+    constexpr int kFlowY = FlowTile<NT>::Y;
     if (blockIdx.x == 0 && threadIdx.x == 0) to.to->status = *I->status;
     const int nx = I->nx, tiles_x = (nx + kFlowX - 1) / kFlowX, tiles = tiles_x * ((y1 - y0 + kFlowY - 1) / kFlowY);
     const T* p = popk<T>(I, parity);
     for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
         const int ty = t / tiles_x;
-        flow_tile<T>(I, p, (t - ty * tiles_x) * kFlowX, y0 + ty * kFlowY, y1, S,
+        flow_tile<NT, T>(I, p, (t - ty * tiles_x) * kFlowX, y0 + ty * kFlowY, y1, S,
                      [&](int x, int y, double r, double u, double w, double ps) {
                          const long long i = static_cast<long long>(y) * nx + x;
                          if (rho) rho[i] = static_cast<O>(r);
@@ -398,15 +396,25 @@ __global__ void __launch_bounds__(kThreads) k_flow(const Inst* __restrict__ I, i
     notify(to);
 }
 
+// The results of a reduction and the status word, by threads 0..7 of the
+// last block.  Each is one word, which the host has set to kNoResult before
+// and watches for itself, so none waits for another to be visible (a fence to
+// the host's memory takes a microsecond).
+__device__ __forceinline__ void give(const Notice& to, double total, const Inst* I) {
+    volatile Reduced* const r = to.to;
+    r->v[threadIdx.x] = total;
+    if (threadIdx.x == 0) r->word = static_cast<unsigned>(*I->status);
+}
+
 // ---- FP64 reductions (lbm_reduce.cuh) -------------------------------------
 // Sums for Laplace's law (LaplaceSums); p = p_EOS(rho) (equal to
 // rho/3 + G psi^2/2, Eq. 10).  The last block puts the totals and the
-// instance's status into mapped host memory and says so there: the call needs
-// no second launch, no copy and no wait for the stream.  About 22 FP64 instructions per node (nine
+// instance's status into mapped host memory: the call needs no second launch,
+// no copy and no wait for the stream.  About 22 FP64 instructions per node (nine
 // additions in FP64, the square root and the divisions by the lattice's size
-// are gone).  Per call, FP32: 256^2 88 -> 21 us, 1024^2 236 -> 79 us.
+// are gone).  Per call, FP32: 256^2 88 -> 18 us, 1024^2 236 -> 72 us.
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_measure(const Inst* __restrict__ I, int parity, Discs D, int rpt,
+__global__ void __launch_bounds__(kLapThreads) k_measure(const Inst* __restrict__ I, int parity, Discs D, int rpt,
                                                        double* __restrict__ partials, Notice to) {
     __shared__ AxisTable A;
     const T* p = popk<T>(I, parity);
@@ -414,25 +422,22 @@ __global__ void __launch_bounds__(kThreads) k_measure(const Inst* __restrict__ I
     laplace_tiles(L, LawFp64(I->pd, false), D, I->nx, I->ny, rpt, A,
                   [&](int x, int y) { return node_rho<T>(I, p, x, y); });
     double total;
-    if (grid_sum8(L.v, -1, 0.0, partials, to.ticket, &total)) {
-        to.to->v[threadIdx.x] = total;
-        if (threadIdx.x == 0) to.to->status = *I->status;
-        notify_reduced(to);
-    }
+    if (grid_sum8<kLapThreads>(L.v, -1, 0.0, partials, to.ticket, &total)) give(to, total, I);
 }
 
 // {mass, sum rho u_x, sum rho u_y, sum rho |u|^2 / 2, max |u|, 0, 0, 0}
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k_stats(const Inst* __restrict__ I, int parity, double* __restrict__ partials,
+template <int NT, typename T>
+__global__ void __launch_bounds__(NT) k_stats(const Inst* __restrict__ I, int parity, double* __restrict__ partials,
                                                      Notice to) {
-    __shared__ FlowTile S;
+    __shared__ FlowTile<NT> S;
+    constexpr int kFlowY = FlowTile<NT>::Y;
     const int nx = I->nx, ny = I->ny;
     const int tiles_x = (nx + kFlowX - 1) / kFlowX, tiles = tiles_x * ((ny + kFlowY - 1) / kFlowY);
     const T* p = popk<T>(I, parity);
     double v[8] = {0, 0, 0, 0, 0, 0, 0, 0}, most = 0.0;   // most: max |u|^2 (the root is monotone)
     for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
         const int ty = t / tiles_x;
-        flow_tile<T>(I, p, (t - ty * tiles_x) * kFlowX, ty * kFlowY, ny, S,
+        flow_tile<NT, T>(I, p, (t - ty * tiles_x) * kFlowX, ty * kFlowY, ny, S,
                      [&](int, int, double r, double u, double w, double) {
                          const double u2 = u * u + w * w;
                          v[0] += r;
@@ -443,11 +448,7 @@ __global__ void __launch_bounds__(kThreads) k_stats(const Inst* __restrict__ I, 
                      });
     }
     double total;
-    if (grid_sum8(v, 4, most, partials, to.ticket, &total)) {
-        to.to->v[threadIdx.x] = threadIdx.x == 4 ? sqrt(total) : total;
-        if (threadIdx.x == 0) to.to->status = *I->status;
-        notify_reduced(to);
-    }
+    if (grid_sum8<NT>(v, 4, most, partials, to.ticket, &total)) give(to, threadIdx.x == 4 ? sqrt(total) : total, I);
 }
 
 int grid_for(long long n) {
@@ -641,25 +642,32 @@ cudaError_t aux_field(const Inst& h, const Inst* d, int parity, int field, int y
 // Blocks of the flow and reduction kernels: one per tile up to what the
 // device holds at once (eight blocks of 256 threads on each of 152 SMs).
 constexpr int kResident = 8 * 152;
-int flow_grid(int nx, int rows) {
-    const long long tiles = static_cast<long long>((nx + kFlowX - 1) / kFlowX) * ((rows + kFlowY - 1) / kFlowY);
+template <int NT> int flow_grid(int nx, int rows) {
+    constexpr int Y = FlowTile<NT>::Y;
+    const long long tiles = static_cast<long long>((nx + kFlowX - 1) / kFlowX) * ((rows + Y - 1) / Y);
     return static_cast<int>(tiles < kResident ? tiles : kResident);
 }
+// whether the small tiles all find an SM of their own
+bool flow_small(int nx, int rows) { return flow_grid<128>(nx, rows) <= kReduceBlocks / 2; }
 
+template <int NT, typename O>
+cudaError_t flow_t(const Inst& h, const Inst* d, int parity, int y0, int y1, void* const out[4], const Notice& to,
+                   cudaStream_t st) {
+    auto go = [&](auto k) {
+        k<<<flow_grid<NT>(h.nx, y1 - y0), NT, 0, st>>>(d, parity, y0, y1, static_cast<O*>(out[0]), static_cast<O*>(out[1]),
+                                                       static_cast<O*>(out[2]), static_cast<O*>(out[3]), to);
+    };
+    if (h.prec == LBM_FP32) go(k_flow<NT, float, O>);
+    else go(k_flow<NT, double, O>);
+    return cudaGetLastError();
+}
 cudaError_t aux_flow(const Inst& h, const Inst* d, int parity, int y0, int y1, void* const out[4], bool f32out,
                      const Notice& to, cudaStream_t st) {
-    const int g = flow_grid(h.nx, y1 - y0);
-    auto go = [&](auto k, auto* zero) {
-        using O = typename std::remove_pointer<decltype(zero)>::type;
-        k<<<g, kThreads, 0, st>>>(d, parity, y0, y1, static_cast<O*>(out[0]), static_cast<O*>(out[1]),
-                                  static_cast<O*>(out[2]), static_cast<O*>(out[3]), to);
-    };
-    const bool f32 = h.prec == LBM_FP32;
-    float* zf = nullptr;
-    double* zd = nullptr;
-    if (f32out) f32 ? go(k_flow<float, float>, zf) : go(k_flow<double, float>, zf);
-    else f32 ? go(k_flow<float, double>, zd) : go(k_flow<double, double>, zd);
-    return cudaGetLastError();
+    if (flow_small(h.nx, y1 - y0))
+        return f32out ? flow_t<128, float>(h, d, parity, y0, y1, out, to, st)
+                      : flow_t<128, double>(h, d, parity, y0, y1, out, to, st);
+    return f32out ? flow_t<256, float>(h, d, parity, y0, y1, out, to, st)
+                  : flow_t<256, double>(h, d, parity, y0, y1, out, to, st);
 }
 
 cudaError_t aux_measure(const Inst& h, const Inst* d, int parity, double cxc, double cyc, double r_in,
@@ -669,16 +677,18 @@ cudaError_t aux_measure(const Inst& h, const Inst* d, int parity, double cxc, do
     const int rpt = tile_rpt(h.nx, h.ny);
     const long long tiles = tile_count(h.nx, h.ny, rpt);
     const int g = static_cast<int>(tiles < rows ? tiles : rows);
-    if (h.prec == LBM_FP32) k_measure<float><<<g, kThreads, 0, st>>>(d, parity, D, rpt, partials, to);
-    else k_measure<double><<<g, kThreads, 0, st>>>(d, parity, D, rpt, partials, to);
+    if (h.prec == LBM_FP32) k_measure<float><<<g, kLapThreads, 0, st>>>(d, parity, D, rpt, partials, to);
+    else k_measure<double><<<g, kLapThreads, 0, st>>>(d, parity, D, rpt, partials, to);
     return cudaGetLastError();
 }
 
 cudaError_t aux_stats(const Inst& h, const Inst* d, int parity, double* partials, int rows, const Notice& to,
                       cudaStream_t st) {
-    const int tiles = flow_grid(h.nx, h.ny), g = tiles < rows ? tiles : rows;
-    if (h.prec == LBM_FP32) k_stats<float><<<g, kThreads, 0, st>>>(d, parity, partials, to);
-    else k_stats<double><<<g, kThreads, 0, st>>>(d, parity, partials, to);
+    const bool small = flow_small(h.nx, h.ny);
+    const int tiles = small ? flow_grid<128>(h.nx, h.ny) : flow_grid<256>(h.nx, h.ny), g = tiles < rows ? tiles : rows;
+    auto go = [&](auto k, int threads) { k<<<g, threads, 0, st>>>(d, parity, partials, to); };
+    if (h.prec == LBM_FP32) small ? go(k_stats<128, float>, 128) : go(k_stats<256, float>, 256);
+    else small ? go(k_stats<128, double>, 128) : go(k_stats<256, double>, 256);
     return cudaGetLastError();
 }
 

@@ -3,6 +3,7 @@
 // read-back, checkpoints, the tile/schedule autotuner and the host-side EOS
 // helpers (critical point, Maxwell coexistence, Laplace fit).
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstddef>
 #include <cstdio>
@@ -707,8 +708,7 @@ int status_of(lbm_ctx* c, int i, int* code) {
 // some microseconds before the end of the stream's work is known, and asks
 // the stream only now and then (so that an error ends the wait).
 lbm::Notice next_notice(lbm_ctx* c) { return {c->h_red, c->d_ticket, ++c->call}; }
-int wait_notice(lbm_ctx* c) {
-    auto here = [&] { return __atomic_load_n(&c->h_red->call, __ATOMIC_ACQUIRE) == c->call; };
+template <typename Here> int wait_for(lbm_ctx* c, Here here) {
     for (unsigned it = 1;; ++it) {
         if (here()) return LBM_OK;
         if (it & 2047u) continue;
@@ -717,6 +717,31 @@ int wait_notice(lbm_ctx* c) {
         if (e != cudaSuccess) return cuda_fail(c, e, "waiting for the results");
         return here() ? LBM_OK : fail(c, LBM_ECUDA, "the stream ended without the results%s");
     }
+}
+int wait_notice(lbm_ctx* c) {
+    return wait_for(c, [&] { return __atomic_load_n(&c->h_red->call, __ATOMIC_ACQUIRE) == c->call; });
+}
+
+// A reduction: its words are made empty, and waited for one by one.
+lbm::Notice next_reduction(lbm_ctx* c) {
+    for (double& v : c->h_red->v) std::memcpy(&v, &lbm::kNoResult, sizeof v);
+    c->h_red->word = lbm::kNoResult;
+    std::atomic_thread_fence(std::memory_order_seq_cst);
+    return {c->h_red, c->d_ticket, 0};
+}
+int wait_reduction(lbm_ctx* c, double (&v)[lbm::kReduceSlots]) {
+    unsigned long long w[lbm::kReduceSlots + 1];
+    const unsigned long long* const from = reinterpret_cast<const unsigned long long*>(c->h_red);
+    static_assert(offsetof(lbm::Reduced, word) == sizeof v, "the status word follows the sums");
+    const int rc = wait_for(c, [&] {
+        for (int k = lbm::kReduceSlots; k >= 0; --k)
+            if ((w[k] = __atomic_load_n(from + k, __ATOMIC_ACQUIRE)) == lbm::kNoResult) return false;
+        return true;
+    });
+    if (rc) return rc;
+    std::memcpy(v, w, sizeof v);
+    c->h_red->status = static_cast<int>(w[lbm::kReduceSlots]);
+    return LBM_OK;
 }
 
 // Where a reduction's blocks put their partial sums, and how many rows fit:
@@ -1493,9 +1518,9 @@ int lbm_batch_measure(lbm_ctx* c, int i, double cxc, double cyc, double r_in, do
     Range range("lbm_batch_measure");
     CK(c, cudaSetDevice(c->device));
     CK(c, lbm::aux_measure(c->h[i], c->d_inst + i, c->parity, cxc, cyc, r_in, r_out, partial_rows(c).first,
-                           partial_rows(c).second, next_notice(c), c->stream));
-    if ((rc = wait_notice(c))) return rc;
-    const double* s = c->h_red->v;
+                           partial_rows(c).second, next_reduction(c), c->stream));
+    double s[lbm::kReduceSlots];
+    if ((rc = wait_reduction(c, s))) return rc;
     const double N = static_cast<double>(c->nx[i]) * c->ny[i];
     const double p_in = s[3] > 0 ? s[1] / s[3] : NAN, rho_in = s[3] > 0 ? s[2] / s[3] : NAN;
     const double p_out = s[6] > 0 ? s[4] / s[6] : NAN, rho_out = s[6] > 0 ? s[5] / s[6] : NAN;
@@ -1526,9 +1551,10 @@ int lbm_batch_stats(lbm_ctx* c, int i, double* out5) {
     Range range("lbm_batch_stats");
     CK(c, cudaSetDevice(c->device));
     CK(c, lbm::aux_stats(c->h[i], c->d_inst + i, c->parity, partial_rows(c).first, partial_rows(c).second,
-                         next_notice(c), c->stream));
-    if ((rc = wait_notice(c))) return rc;
-    std::memcpy(out5, c->h_red->v, 5 * sizeof(double));
+                         next_reduction(c), c->stream));
+    double s[lbm::kReduceSlots];
+    if ((rc = wait_reduction(c, s))) return rc;
+    std::memcpy(out5, s, 5 * sizeof(double));
     return status_code(c->h_red->status);
 }
 

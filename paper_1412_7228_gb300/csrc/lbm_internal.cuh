@@ -359,16 +359,20 @@ constexpr size_t kPinnedBlock = (size_t(1) << 16) + 256;
 void* pinned_get(size_t bytes);
 void pinned_put(void* p, size_t bytes);
 
-// What a call reads back besides its arrays: the sums of a reduction and the
-// instance's status word, written by the device into pinned host memory
-// mapped for it, and the number of the call whose results these are, written
-// last.
+// What a call reads back besides its arrays, written by the device into
+// pinned host memory mapped for it: the sums of a reduction with its status
+// word, each of which the host watches; or the instance's status word and the
+// number of the call whose results these are, written last.
 constexpr int kReduceSlots = 8;
 struct Reduced {
     double v[kReduceSlots];
+    unsigned long long word;   // a reduction's status word
     int status;
     unsigned call;
 };
+// What a reduction's words hold before their results arrive: a NaN with a
+// payload that no arithmetic gives.
+constexpr unsigned long long kNoResult = 0x7ff4d1c5a3b29687ull;
 // How a kernel gives its results: its last block (by `ticket`, a device word
 // that is zero between launches) writes to->call = call once every block's
 // writes are visible to the host.  ticket NULL: the status word only (the host

@@ -17,7 +17,6 @@
 namespace lbm {
 namespace {
 
-constexpr int kRedThreads = 256;   // threads per block of every reduction kernel
 
 // Sums of eight values over a warp.  A shuffle tree per value costs 8 x 5
 // FP64 additions per warp; here each exchange halves the values a lane
@@ -54,11 +53,12 @@ __device__ __forceinline__ double warp_sum8(const double (&v)[8]) {
 // this thread when max_slot >= 0 (its own v entry is ignored).
 //
 // The former second launch (one warp adding 304 rows one after another)
-// took 45 us by itself; here the last block's 32 groups of 8 threads take
-// the rows in turn.
+// took 45 us by itself; here the last block's groups of 8 threads take the
+// rows in turn.
+template <int NT>
 __device__ __forceinline__ bool grid_sum8(const double (&v)[8], int max_slot, double vmax, double* partials,
                                           unsigned* ticket, double* total) {
-    constexpr int kWarps = kRedThreads / 32, kGroups = kRedThreads / 8;
+    constexpr int kWarps = NT / 32, kGroups = NT / 8;
     __shared__ double red[kWarps][8];
     __shared__ unsigned s_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -159,7 +159,8 @@ __device__ __forceinline__ double quotient(double num, double inv_den, double de
 
 // The pressure law with its constants folded, p = rho [K R T h(rho) - K a rho]
 // (h = num / q^3 for Carnahan-Starling), and psi = W / sqrt(W D) with Eq.
-// 10's radicand (2/G)(p - rho/3) = W / D: 16 and 17 FP64 instructions.
+// 10's radicand (2/G)(p - rho/3) = W / D: 16 (with the sum) and 17 FP64
+// instructions.
 struct LawFp64 {
     int eos;
     double b, c1, c2, c3;   // p: K R T, K a (K a alpha), 0; psi: those and 1/3, times 2/G
@@ -171,11 +172,12 @@ struct LawFp64 {
         c2 = s * (P.K * (P.eos == LBM_EOS_PR ? P.aalpha : P.a));
         c3 = psi ? s * (1.0 / 3.0) : 0.0;
     }
-    __device__ __forceinline__ double pressure(double rho) const {
+    // p / rho
+    __device__ __forceinline__ double pressure_over_rho(double rho) const {
         const double n = b * rho, q = 1.0 - n;
-        if (eos == LBM_EOS_CS) return rho * (c1 * div(fma(n, fma(n, q, 1.0), 1.0), q * q * q) - c2 * rho);
-        if (eos == LBM_EOS_VDW) return rho * (div(c1, q) - c2 * rho);
-        return rho * (div(c1, q) - div(c2 * rho, fma(n, 2.0 - n, 1.0)));
+        if (eos == LBM_EOS_CS) return c1 * div(fma(n, fma(n, q, 1.0), 1.0), q * q * q) - c2 * rho;
+        if (eos == LBM_EOS_VDW) return div(c1, q) - c2 * rho;
+        return div(c1, q) - div(c2 * rho, fma(n, 2.0 - n, 1.0));
     }
     __device__ __forceinline__ double psi(double rho) const {
         const double n = b * rho, q = 1.0 - n;
@@ -202,14 +204,14 @@ struct LaplaceSums {
         const bool in = b <= D.in2, out = b >= D.out2;
         if (in == out) rest += in ? -r : r;
         if (!in && !out) return;
-        const double p = p_eos.pressure(r);
+        const double p = p_eos.pressure_over_rho(r);   // its product with rho goes into the sum
         if (in) {
-            v[1] += p;
+            v[1] = fma(r, p, v[1]);
             v[2] += r;
             ++n_in;
         }
         if (out) {
-            v[4] += p;
+            v[4] = fma(r, p, v[4]);
             v[5] += r;
             ++n_out;
         }
@@ -222,8 +224,11 @@ struct LaplaceSums {
 };
 
 // Tiles of the Laplace sums: kTileX columns by kTileRows * rpt rows, a
-// thread taking rpt nodes of one column.
-constexpr int kTileX = 64, kTileRows = kRedThreads / kTileX, kMaxRpt = 8;
+// thread taking rpt nodes of one column.  Blocks of four warps, one per SM
+// quarter: the FP64 pipe takes 64 clocks per warp instruction of a quarter, so
+// more warps on an SM only lengthen a small lattice's chain (64^2: 256
+// threads per block 11.0 us on the device, 128 threads 8.3).
+constexpr int kLapThreads = 128, kTileX = 64, kTileRows = kLapThreads / kTileX, kMaxRpt = 16;
 inline long long tile_count(int nx, int ny, int rpt) {
     return static_cast<long long>((nx + kTileX - 1) / kTileX) * ((ny + rpt * kTileRows - 1) / (rpt * kTileRows));
 }
@@ -243,7 +248,8 @@ inline int tile_rpt(int nx, int ny) {
     return best;
 }
 // The sums over the tiles of this block; rho_at(x, y) gives a node's density.
-// A tile's squared distances along x and y are formed once, in shared memory.
+// A tile's squared distances along x and y are formed once, in shared memory,
+// while the first densities arrive.
 struct AxisTable {
     double x[kTileX], y[kTileRows * kMaxRpt];
 };
@@ -254,17 +260,19 @@ __device__ __forceinline__ void laplace_tiles(LaplaceSums& L, const LawFp64& p_e
     const int tiles_x = (nx + kTileX - 1) / kTileX, tiles = tiles_x * ((ny + rows - 1) / rows);
     for (int k = blockIdx.x; k < tiles; k += gridDim.x) {
         const int row = k / tiles_x, x0 = (k - row * tiles_x) * kTileX, x = x0 + tx, y0 = row * rows;
-        __syncthreads();   // the tile before is done with the table
-        if (t < kTileX + rows) {
-            const bool along_x = t < kTileX;
-            const double d = axis2(along_x ? x0 + t : y0 + t - kTileX, along_x ? D.cx : D.cy, along_x ? nx : ny,
+        const double first = x < nx && y0 + ty < ny ? rho_at(x, y0 + ty) : 0.0;
+        if (k != static_cast<int>(blockIdx.x)) __syncthreads();   // the tile before is done with the table
+        for (int e = t; e < kTileX + rows; e += kLapThreads) {
+            const bool along_x = e < kTileX;
+            const double d = axis2(along_x ? x0 + e : y0 + e - kTileX, along_x ? D.cx : D.cy, along_x ? nx : ny,
                                    along_x ? D.inv_nx : D.inv_ny);
-            (along_x ? A.x[t] : A.y[t - kTileX]) = d;
+            (along_x ? A.x[e] : A.y[e - kTileX]) = d;
         }
         __syncthreads();
         if (x >= nx) continue;
         const double dx2 = A.x[tx];
-        for (int j = ty; j < rows && y0 + j < ny; j += kTileRows) L.add(p_eos, D, rho_at(x, y0 + j), dx2 + A.y[j]);
+        for (int j = ty; j < rows && y0 + j < ny; j += kTileRows)
+            L.add(p_eos, D, j == ty ? first : rho_at(x, y0 + j), dx2 + A.y[j]);
     }
     L.close();
 }

@@ -50,9 +50,9 @@ std::mutex g_mu;
 double* g_ptr[kMaxDevices] = {};
 
 // The Laplace sums of a field (LaplaceSums) in one launch, bound by the FP64
-// pipe (20 instructions per node; 4096^2: 1970 -> 725 us per call, of which
+// pipe (19 instructions per node; 4096^2: 1970 -> 689 us per call, of which
 // the former second launch was 168).
-__global__ void __launch_bounds__(kRedThreads)
+__global__ void __launch_bounds__(kLapThreads)
     k_field_sums(const double* __restrict__ rho, int nx, int ny, Phys<double> P, Discs D, int rpt,
                  double* __restrict__ partials, unsigned* ticket, double* __restrict__ out) {
     __shared__ AxisTable A;
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(kRedThreads)
     laplace_tiles(L, LawFp64(P, false), D, nx, ny, rpt, A,
                   [&](int x, int y) { return rho[static_cast<long long>(y) * nx + x]; });
     double total;
-    if (grid_sum8(L.v, -1, 0.0, partials, ticket, &total)) out[threadIdx.x] = total;
+    if (grid_sum8<kLapThreads>(L.v, -1, 0.0, partials, ticket, &total)) out[threadIdx.x] = total;
 }
 
 // Address of g_scratch on the current device, looked up once per device.
@@ -122,7 +122,7 @@ extern "C" int lbm_field_pressure_jump_static(const double* d_rho, int nx, int n
     if (cudaMemsetAsync(ticket, 0, sizeof *ticket, st) != cudaSuccess) return LBM_ECUDA;
     // cudaLaunchKernel returns this launch's own error (never an earlier one)
     void* args[] = {&d_rho, &nx, &ny, &P, &D, &rpt, &partials, &ticket, &totals};
-    if (cudaLaunchKernel(reinterpret_cast<const void*>(&k_field_sums), dim3(blocks), dim3(kRedThreads), args, 0, st) !=
+    if (cudaLaunchKernel(reinterpret_cast<const void*>(&k_field_sums), dim3(blocks), dim3(kLapThreads), args, 0, st) !=
         cudaSuccess)
         return LBM_ECUDA;
     double s[kSlots];
