@@ -1344,7 +1344,7 @@ void lbm_destroy(lbm_ctx* c) {
     }
     for (auto& e : c->band_done)
         if (e) cudaEventDestroy(e);
-    lbm::pinned_put(c->h_red, 256 + kStageBytes);
+    lbm::pinned_put(c->h_red);
     if (c->owns && c->buf) cudaFree(c->buf);
     delete c;
 }

@@ -351,13 +351,12 @@ cudaError_t run_launch(int prec, int k, const Inst* d_insts, const void* args, b
 bool cluster_supported(int prec, int nx, int ny);
 cudaError_t cluster_run(const Inst& host, int parity, int nsteps, cudaStream_t st);
 
-// Pinned host memory, mapped for every device (lbm_pinned.cu): blocks of
-// kPinnedBlock bytes come from a small pool, larger ones straight from the
-// driver.  NULL when there is none.  Give a block back with the size that was
-// asked for, once nothing uses it any more.
+// Pinned host memory, mapped for every device (lbm_pinned.cu): up to
+// kPinnedBlock bytes come from a small slab, more straight from the driver.
+// NULL when there is none.  Given back once nothing uses it any more.
 constexpr size_t kPinnedBlock = (size_t(1) << 16) + 256;
 void* pinned_get(size_t bytes);
-void pinned_put(void* p, size_t bytes);
+void pinned_put(void* p);
 
 // What a call reads back besides its arrays, written by the device into
 // pinned host memory mapped for it: the sums of a reduction with its status

@@ -1,8 +1,10 @@
 // lbm_pinned.cu -- pinned host memory, mapped for the devices, of the contexts
 // and networks.  Allocating and freeing it takes the driver about 100 and 180 us,
-// three times what making a small context takes otherwise, so blocks of
-// one size are kept for the next owner: at most kKept of them, given back at
-// exit.  A block's former owner has waited for its stream before it lets go.
+// three times what making a small context takes otherwise, so the first
+// owner allocates a slab of kBlocks blocks of one size, which serves up to
+// that many owners at a time and is given back at exit; further owners, and
+// larger requests, go to the driver.  A block's owner has waited for its
+// stream before it lets go.
 #include <mutex>
 
 #include "lbm_internal.cuh"
@@ -10,14 +12,41 @@
 namespace lbm {
 namespace {
 
-constexpr int kKept = 8;   // half a megabyte
+constexpr int kBlocks = 8;   // half a megabyte
 
 struct Pool {
     std::mutex mu;
-    void* block[kKept] = {};
-    int n = 0;
+    char* slab = nullptr;
+    bool used[kBlocks] = {};
     ~Pool() {
-        for (int k = 0; k < n; ++k) cudaFreeHost(block[k]);
+        if (slab) cudaFreeHost(slab);
+    }
+    // a free block of the slab, or NULL
+    void* take() {
+        std::lock_guard<std::mutex> lock(mu);
+        if (!slab) slab = static_cast<char*>(allocate(kBlocks * kPinnedBlock));
+        for (int k = 0; slab && k < kBlocks; ++k)
+            if (!used[k]) {
+                used[k] = true;
+                return slab + k * kPinnedBlock;
+            }
+        return nullptr;
+    }
+    // whether p was a block of the slab, now free again
+    bool put(void* p) {
+        std::lock_guard<std::mutex> lock(mu);
+        for (int k = 0; slab && k < kBlocks; ++k)
+            if (p == slab + k * kPinnedBlock) {
+                used[k] = false;
+                return true;
+            }
+        return false;
+    }
+    static void* allocate(size_t bytes) {
+        void* v = nullptr;
+        if (cudaHostAlloc(&v, bytes, cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess) return v;
+        cudaGetLastError();
+        return nullptr;
     }
 };
 Pool& pool() {
@@ -28,31 +57,13 @@ Pool& pool() {
 }  // namespace
 
 void* pinned_get(size_t bytes) {
-    if (bytes <= kPinnedBlock) {
-        Pool& p = pool();
-        std::lock_guard<std::mutex> lock(p.mu);
-        if (p.n > 0) return p.block[--p.n];
-    }
-    void* v = nullptr;
-    const size_t size = bytes <= kPinnedBlock ? kPinnedBlock : bytes;
-    if (cudaHostAlloc(&v, size, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    return v;
+    if (bytes <= kPinnedBlock)
+        if (void* p = pool().take()) return p;
+    return Pool::allocate(bytes);
 }
 
-void pinned_put(void* v, size_t bytes) {
-    if (!v) return;
-    if (bytes <= kPinnedBlock) {
-        Pool& p = pool();
-        std::lock_guard<std::mutex> lock(p.mu);
-        if (p.n < kKept) {
-            p.block[p.n++] = v;
-            return;
-        }
-    }
-    cudaFreeHost(v);
+void pinned_put(void* p) {
+    if (p && !pool().put(p)) cudaFreeHost(p);
 }
 
 }  // namespace lbm

@@ -524,6 +524,31 @@ __global__ void k_reduce_adam(const float* __restrict__ partials, int nparts, fl
     }
 }
 
+// Raw samples to standardised ones, by IEEE division (in place or not).
+__global__ void k_standardise(const float* x, const float* y, int n, Norm nm, float* X, float* Y) {
+    const long long nx = static_cast<long long>(n) * NI, all = static_cast<long long>(n) * (NI + NO);
+    for (long long i = blockIdx.x * static_cast<long long>(kT) + threadIdx.x; i < all;
+         i += static_cast<long long>(gridDim.x) * kT) {
+        if (i < nx) {
+            const int c = static_cast<int>(i % NI);
+            X[i] = (x[i] - nm.in_mean[c]) / nm.in_std[c];
+        } else {
+            const long long j = i - nx;
+            const int k = static_cast<int>(j % NO);
+            Y[j] = (y[j] - nm.out_mean[k]) / nm.out_std[k];
+        }
+    }
+}
+
+// New parameters, moments at zero.
+__global__ void k_set_params(const float* __restrict__ from, float* __restrict__ P, float* __restrict__ M,
+                             float* __restrict__ V) {
+    const int p = blockIdx.x * kT + threadIdx.x;
+    if (p >= NP) return;
+    P[p] = from[p];
+    M[p] = V[p] = 0.0f;
+}
+
 // ---- inference ---------------------------------------------------------------
 // Inference on raw inputs: standardise, forward, de-standardise; CTAs
 // striding over the passes.
@@ -637,14 +662,16 @@ struct lbm_mlp {
     Norm norm{};
     float *P = nullptr, *M = nullptr, *V = nullptr, *X = nullptr, *Y = nullptr, *partials = nullptr,
           *grad = nullptr, *sum = nullptr, *io = nullptr;   // sum: the loss of a single gradient
-    // training (from the first call of it on): the sample orders, bias corrections and losses of a launch's
-    // epochs, twice, so that the host prepares a launch while another runs
-    int *order[2] = {}, *h_order[2] = {};
-    float2 *corr[2] = {}, *h_corr[2] = {};
-    float *loss[2] = {}, *h_loss[2] = {};
-    void *stage = nullptr, *h_stage = nullptr;   // device and pinned memory that these are in
+    // training (from the first call of it on): the sample orders, bias
+    // corrections and losses of a launch's epochs, twice, so that the host
+    // prepares a launch while another runs; in pinned memory, where the
+    // kernels fetch them minibatches ahead of their use
+    int* order[2] = {};
+    float2* corr[2] = {};
+    float* loss[2] = {};
+    void* stage = nullptr;   // the memory these are in
     cudaEvent_t done[2] = {};
-    float* h_io = nullptr;   // pinned and mapped: NI + NO floats of up to io_n samples, read and written by the kernels
+    float* h_io = nullptr;   // pinned and mapped: NI + NO floats of up to io_n samples (or the parameters), for the kernels
     int io_n = 0;
     int cap = 0;             // samples (and minibatches) each of them holds
     int adam_t = 0;
@@ -662,7 +689,10 @@ constexpr int kIoMax = 1 << 16;       // samples of the pinned buffer at most
 constexpr int kClusterMax = 768;
 
 bool valid(lbm_mlp* m) { return m && m->P; }
-size_t io_bytes(const lbm_mlp* m) { return sizeof(float) * (NI + NO) * static_cast<size_t>(m->io_n); }
+// the samples, or the parameters
+size_t io_bytes(const lbm_mlp* m) {
+    return sizeof(float) * std::max<size_t>((NI + NO) * static_cast<size_t>(m->io_n), NP);
+}
 
 // A block of memory cut into buffers, each a multiple of 16 bytes so that all
 // are aligned alike (with at == NULL: their sizes only).
@@ -680,48 +710,44 @@ struct Cut {
 int ensure_stage(lbm_mlp* m) {
     if (m->cap) return LBM_OK;
     const size_t cap = std::max(m->max_n, kOrderMin);
-    auto cut = [&](Cut c, float2* (&corr)[2], int* (&order)[2], float* (&loss)[2]) {
+    auto cut = [&](Cut c) {
         for (int k = 0; k < 2; ++k) {
-            corr[k] = static_cast<float2*>(c.take(cap * sizeof(float2)));
-            order[k] = static_cast<int*>(c.take(cap * sizeof(int)));
-            loss[k] = static_cast<float*>(c.take(cap * sizeof(float)));
+            m->corr[k] = static_cast<float2*>(c.take(cap * sizeof(float2)));
+            m->order[k] = static_cast<int*>(c.take(cap * sizeof(int)));
+            m->loss[k] = static_cast<float*>(c.take(cap * sizeof(float)));
         }
         return c.used;
     };
-    const size_t bytes = cut({nullptr, 0}, m->corr, m->order, m->loss);
-    bool ok = (m->stage || cudaMalloc(&m->stage, bytes) == cudaSuccess) &&
-              (m->h_stage || cudaMallocHost(&m->h_stage, bytes) == cudaSuccess);
+    const size_t bytes = cut({nullptr, 0});
+    bool ok = m->stage || cudaHostAlloc(&m->stage, bytes, cudaHostAllocMapped) == cudaSuccess;
     for (auto& e : m->done) ok = ok && (e || cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess);
     if (!ok) {
         cudaGetLastError();
         return LBM_ENOMEM;
     }
-    cut({static_cast<char*>(m->stage), 0}, m->corr, m->order, m->loss);
-    cut({static_cast<char*>(m->h_stage), 0}, m->h_corr, m->h_order, m->h_loss);
+    cut({static_cast<char*>(m->stage), 0});
     m->cap = static_cast<int>(cap);
     return LBM_OK;
 }
 
-// Standardised samples to the device; from pinned memory (n <= io_n) without
-// waiting, since every call waits for its stream before it returns.
+// Standardised samples to m->X, m->Y, enqueued: from pinned memory, which
+// every call has done with before it returns, or in place from copies.
 int standardise_upload(lbm_mlp* m, const float* X, const float* Y, int n) {
-    std::vector<float> far;
-    float* xs = m->h_io;
-    if (n > m->io_n) {
-        far.resize(static_cast<size_t>(n) * (NI + NO));
-        xs = far.data();
-    }
-    float* const ys = xs + static_cast<size_t>(n) * NI;
-    for (int s = 0; s < n; ++s) {
-        for (int c = 0; c < NI; ++c) xs[s * NI + c] = (X[s * NI + c] - m->norm.in_mean[c]) / m->norm.in_std[c];
-        for (int k = 0; k < NO; ++k) ys[s * NO + k] = (Y[s * NO + k] - m->norm.out_mean[k]) / m->norm.out_std[k];
-    }
     const size_t bytes = static_cast<size_t>(n) * sizeof(float);
-    if (cudaMemcpyAsync(m->X, xs, NI * bytes, cudaMemcpyHostToDevice, m->st) != cudaSuccess ||
-        cudaMemcpyAsync(m->Y, ys, NO * bytes, cudaMemcpyHostToDevice, m->st) != cudaSuccess ||
-        (n > m->io_n && cudaStreamSynchronize(m->st) != cudaSuccess))
+    const float *x = m->X, *y = m->Y;
+    if (n <= m->io_n) {
+        std::memcpy(m->h_io, X, NI * bytes);
+        std::memcpy(m->h_io + static_cast<size_t>(n) * NI, Y, NO * bytes);
+        x = m->h_io;
+        y = m->h_io + static_cast<size_t>(n) * NI;
+    } else if (cudaMemcpyAsync(m->X, X, NI * bytes, cudaMemcpyHostToDevice, m->st) != cudaSuccess ||
+               cudaMemcpyAsync(m->Y, Y, NO * bytes, cudaMemcpyHostToDevice, m->st) != cudaSuccess ||
+               cudaStreamSynchronize(m->st) != cudaSuccess) {
         return LBM_ECUDA;
-    return LBM_OK;
+    }
+    const int blocks = std::min(n / 32 + 1, 8 * kRows);
+    k_standardise<<<blocks, kT, 0, m->st>>>(x, y, n, m->norm, m->X, m->Y);
+    return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ECUDA;
 }
 
 float2 next_corr(lbm_mlp* m, float b1, float b2) {
@@ -860,9 +886,8 @@ void lbm_mlp_destroy(lbm_mlp* m) {
     if (!m) return;
     if (m->P) cudaStreamSynchronize(m->st);   // also: nothing uses the pinned memory any more
     if (m->dev) cudaFree(m->dev);
-    if (m->stage) cudaFree(m->stage);
-    if (m->h_stage) cudaFreeHost(m->h_stage);
-    lbm::pinned_put(m->h_io, io_bytes(m));
+    if (m->stage) cudaFreeHost(m->stage);
+    lbm::pinned_put(m->h_io);
     for (cudaEvent_t e : m->done)
         if (e) cudaEventDestroy(e);
     delete m;
@@ -884,11 +909,9 @@ int lbm_mlp_set_normalization(lbm_mlp* m, const float in_mean[3], const float in
 
 int lbm_mlp_set_params(lbm_mlp* m, const float* params) {
     if (!valid(m) || !params) return LBM_EINVAL;
-    if (cudaMemcpyAsync(m->P, params, NP * sizeof(float), cudaMemcpyHostToDevice, m->st) != cudaSuccess ||
-        cudaMemsetAsync(m->M, 0, NP * sizeof(float), m->st) != cudaSuccess ||
-        cudaMemsetAsync(m->V, 0, NP * sizeof(float), m->st) != cudaSuccess ||
-        cudaStreamSynchronize(m->st) != cudaSuccess)
-        return LBM_ECUDA;
+    std::memcpy(m->h_io, params, NP * sizeof(float));
+    k_set_params<<<(NP + kT - 1) / kT, kT, 0, m->st>>>(m->h_io, m->P, m->M, m->V);
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(m->st) != cudaSuccess) return LBM_ECUDA;
     m->adam_t = 0;
     return LBM_OK;
 }
@@ -944,7 +967,7 @@ int lbm_mlp_train(lbm_mlp* m, const float* X, const float* Y, int n, int epochs,
         if (cudaEventSynchronize(m->done[k]) != cudaSuccess) return LBM_ECUDA;
         for (int e = 0; e < pending[k] && loss_per_epoch; ++e) {
             double acc = 0;
-            for (int b = 0; b < nb; ++b) acc += m->h_loss[k][e * nb + b];
+            for (int b = 0; b < nb; ++b) acc += m->loss[k][e * nb + b];
             loss_per_epoch[at[k] + e] = static_cast<float>(acc / nb);
         }
         pending[k] = 0;
@@ -960,30 +983,22 @@ int lbm_mlp_train(lbm_mlp* m, const float* X, const float* Y, int n, int epochs,
                     const int j = static_cast<int>(splitmix(s) % static_cast<uint64_t>(i + 1));
                     std::swap(order[i], order[j]);
                 }
-                std::memcpy(m->h_order[k] + static_cast<size_t>(e) * n, order.data(), n * sizeof(int));
-                for (int b = 0; b < nb; ++b) m->h_corr[k][e * nb + b] = next_corr(m, b1, b2);
+                std::memcpy(m->order[k] + static_cast<size_t>(e) * n, order.data(), n * sizeof(int));
+                for (int b = 0; b < nb; ++b) m->corr[k][e * nb + b] = next_corr(m, b1, b2);
             }
-            if (cudaMemcpyAsync(m->order[k], m->h_order[k], static_cast<size_t>(len) * n * sizeof(int),
-                                cudaMemcpyHostToDevice, m->st) != cudaSuccess)
-                return LBM_ECUDA;
             if (m->cluster && batch <= kClusterMax) {
-                if (cudaMemcpyAsync(m->corr[k], m->h_corr[k], static_cast<size_t>(len) * nb * sizeof(float2),
-                                    cudaMemcpyHostToDevice, m->st) != cudaSuccess)
-                    return LBM_ECUDA;
-                const TrainArgs a = {m->P, m->M, m->V, m->X, m->Y, m->order[k], m->corr[k], m->loss[k], n, batch, len, lr, b1, b2, eps};
+                const TrainArgs a = {m->P, m->M, m->V, m->X, m->Y, m->order[k], m->corr[k], m->loss[k], n,
+                                     batch, len, lr, b1, b2, eps};
                 if (launch_train(m, a) != cudaSuccess) return LBM_ECUDA;
             } else {
                 for (int q = 0; q < len * nb; ++q) {
                     const int first = (q % nb) * batch;
                     if (grad_pass(m, m->order[k] + static_cast<size_t>(q / nb) * n, first, std::min(batch, n - first),
-                                  true, lr, b1, b2, eps, m->h_corr[k][q], m->loss[k] + q) != cudaSuccess)
+                                  true, lr, b1, b2, eps, m->corr[k][q], m->loss[k] + q) != cudaSuccess)
                         return LBM_ECUDA;
                 }
             }
-            if (cudaMemcpyAsync(m->h_loss[k], m->loss[k], static_cast<size_t>(len) * nb * sizeof(float),
-                                cudaMemcpyDeviceToHost, m->st) != cudaSuccess ||
-                cudaEventRecord(m->done[k], m->st) != cudaSuccess)
-                return LBM_ECUDA;
+            if (cudaEventRecord(m->done[k], m->st) != cudaSuccess) return LBM_ECUDA;
             pending[k] = len;
             at[k] = e0;
         }
