@@ -102,11 +102,13 @@ Layout make_layout(int n, const int* nx, const int* ny, int prec) {
         for (int i = 0; i < n; ++i) s += static_cast<size_t>((nx[i] + t.bx - 1) / t.bx) * ((ny[i] + t.by - 1) / t.by);
         tiles = std::max(tiles, s);
     }
+    // An interleaved schedule's tile table and the multi-step launches' step
+    // counters (one per tile), of which a context uses one at a time.
     L.inst_off = off;
     off = align_up(off + n * sizeof(Inst), 256);
     L.tiles_off = off;
     L.tiles_cap = tiles;
-    off = align_up(off + tiles * sizeof(int4), 256);
+    off = align_up(off + tiles * sizeof(int2), 256);
     L.status_off = off;
     off = align_up(off + n * sizeof(int), 256);
     L.partials_off = off;
@@ -116,8 +118,8 @@ Layout make_layout(int n, const int* nx, const int* ny, int prec) {
     L.scratch_off = off;
     L.scratch_elems = 3 * maxN;
     off = align_up(off + L.scratch_elems * sizeof(double), 256);
-    L.run_off = off;   // multi-step launches: work counter, abort flag, then one step counter per tile
-    off = align_up(off + 16 + tiles * sizeof(int), 256);
+    L.run_off = off;   // multi-step launches: work counter, abort flag
+    off = align_up(off + 16, 256);
     L.total = off;
     return L;
 }
@@ -226,7 +228,7 @@ struct lbm_ctx {
     bool owns = false;
     cudaStream_t stream = nullptr;
     Inst* d_inst = nullptr;
-    int4* d_tiles = nullptr;
+    int2* d_tiles = nullptr;
     int ntiles = 0;                   // tiles of all instances
     std::vector<Maps> maps;
     // a batch (n > 1) is stepped by one launch per chunk of up to
@@ -383,7 +385,7 @@ const void* one_args(lbm_ctx* c) {
 template <typename T>
 int build_chunks(lbm_ctx* c, std::vector<lbm::BatchArgs<T>> (&out)[2], const std::vector<int>& order,
                  const std::vector<int>& tx, const std::vector<int>& cnt, const lbm::TileCfg& t,
-                 std::vector<int4>& table) {
+                 std::vector<int2>& table) {
     for (int c0 = 0; c0 < c->n; c0 += lbm::kBatchLaunchMax) {
         const int m = std::min(lbm::kBatchLaunchMax, c->n - c0);
         lbm::BatchArgs<T> a;
@@ -410,7 +412,7 @@ int build_chunks(lbm_ctx* c, std::vector<lbm::BatchArgs<T>> (&out)[2], const std
             for (int r = 0; r < most; ++r)
                 for (int k = 0; k < m; ++k)
                     if (r < cnt[a.inst[k]])
-                        table.push_back(make_int4(k, (r % a.tiles_x[k]) * t.bx, (r / a.tiles_x[k]) * t.by, 0));
+                        table.push_back(make_int2(k << 24 | (r % a.tiles_x[k]) * t.bx, (r / a.tiles_x[k]) * t.by));
         }
         for (int par = 0; par < 2; ++par) {
             for (int k = 0; k < m; ++k) a.tmap[k] = c->maps[a.inst[k]].tmap[par];
@@ -474,7 +476,7 @@ std::vector<std::vector<int>> plan_run_chunks(const std::vector<size_t>& bytes) 
 template <typename T>
 int build_run_chunks(lbm_ctx* c, std::vector<lbm::RunArgs<T>>& out, const std::vector<int>& tx,
                      const std::vector<int>& cnt) {
-    int* done = reinterpret_cast<int*>(c->d_run + 16);
+    int* done = reinterpret_cast<int*>(c->d_tiles);
     std::vector<size_t> bytes(c->n);
     for (int i = 0; i < c->n; ++i) bytes[i] = 2 * 9 * static_cast<size_t>(c->h[i].plane) * c->esz;
     int tile0 = 0;
@@ -538,12 +540,12 @@ int build_tiles(lbm_ctx* c) {
     std::vector<int> order(c->n);
     for (int i = 0; i < c->n; ++i) order[i] = i;
     if (c->sched == 2) std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cnt[a] > cnt[b]; });
-    std::vector<int4> table;   // schedule 1: every chunk's table, one after another
+    std::vector<int2> table;   // schedule 1: every chunk's table, one after another
     const int rc = c->prec == LBM_FP32 ? build_chunks(c, c->bargs_f, order, tx, cnt, t, table)
                                        : build_chunks(c, c->bargs_d, order, tx, cnt, t, table);
     if (rc) return rc;
     if (!table.empty()) {
-        CK(c, cudaMemcpyAsync(c->d_tiles, table.data(), table.size() * sizeof(int4), cudaMemcpyHostToDevice,
+        CK(c, cudaMemcpyAsync(c->d_tiles, table.data(), table.size() * sizeof(int2), cudaMemcpyHostToDevice,
                               c->stream));
         CK(c, cudaStreamSynchronize(c->stream));
     }
@@ -606,7 +608,9 @@ int apply_schedule(lbm_ctx* c, int cfg, int sched) {
     return build_tiles(c);
 }
 
-inline void fill_node(lbm::NodeConsts<float>&, const HostParams&) {}
+inline void fill_node(lbm::NodeConsts<float>& N, const HostParams& hp) {
+    for (int k = 0; k < 9; ++k) N.nhs[k] = -static_cast<float>(1.0 - 0.5 * hp.s[k]);
+}
 inline void fill_node(lbm::NodeConsts<double>& N, const HostParams& hp) {
     const double w = -hp.G / 12.0, kq = hp.G != 0.0 ? -0.5 * hp.kappa : 0.0;
     const double s1 = hp.s[1], s2 = hp.s[2], s4 = hp.s[4], s6 = hp.s[6];
@@ -668,10 +672,8 @@ template <typename T> void fill_phys(lbm::Phys<T>& P, const HostParams& hp) {
     P.two_over_G = hp.G != 0.0 ? T(2.0 / hp.G) : T(0);
     P.interact = hp.G != 0.0;
     for (int k = 0; k < 9; ++k) {
-        P.s[k] = T(hp.s[k]);
         P.hs[k] = T(1.0 - 0.5 * hp.s[k]);
-        P.ns[k] = -P.s[k];
-        P.nhs[k] = -P.hs[k];
+        P.ns[k] = -T(hp.s[k]);
     }
     P.h2s7 = T(2) * P.hs[7];
     P.h6s1 = T(6.0 * (1.0 - 0.5 * hp.s[1]));
@@ -1298,7 +1300,7 @@ int lbm_batch_create(lbm_ctx** out, int n, const int* nx, const int* ny, int pre
         return LBM_ECUDA;
     }
     c->d_inst = reinterpret_cast<Inst*>(c->buf + c->L.inst_off);
-    c->d_tiles = reinterpret_cast<int4*>(c->buf + c->L.tiles_off);
+    c->d_tiles = reinterpret_cast<int2*>(c->buf + c->L.tiles_off);
     c->d_status = reinterpret_cast<int*>(c->buf + c->L.status_off);
     c->d_partials = reinterpret_cast<double*>(c->buf + c->L.partials_off);
     c->d_result = reinterpret_cast<double*>(c->buf + c->L.result_off);

@@ -40,9 +40,14 @@ __host__ __device__ constexpr int cy(int a) {
 constexpr int ST_UNSTABLE = 1;
 constexpr int ST_TIMEOUT = 2;
 
-// Constants of the FP64 node (collide64 in lbm_step_kernels.cuh), formed once
-// on the host.
-template <typename T> struct NodeConsts {};
+// Constants of one precision's node only, formed once on the host: FP32
+// (collide in lbm_step_kernels.cuh) and FP64 (collide64).  Apart, they leave
+// Inst, and so the memory that a context asks for, as small as it was before
+// FP64 had its own.
+template <typename T> struct NodeConsts;
+template <> struct NodeConsts<float> {
+    float nhs[9];                // -(1 - s/2)
+};
 template <> struct NodeConsts<double> {
     double cF, hF;               // -(G/12) (1 - A), -(G/12) A/2
     double k1[3], k1r, k1q;      // e*: f_0, axis sum, diagonal sum; rho|v|^2; tr Q's sum
@@ -57,9 +62,8 @@ template <typename T> struct Phys : NodeConsts<T> {
     unsigned flags;     // LBM_FLAG_*
     T K, a, b, b4, RT, aalpha;   // EOS; b4 = b/4 (CS), aalpha = a alpha(T) (PR)
     T A, kappa, G, two_over_G;   // Eq. 9, Eq. 23, Eq. 10
-    T s[9];             // Lambda
-    T hs[9];            // 1 - s/2, the forcing weight of Eq. 5
-    T ns[9], nhs[9];    // -s, -hs
+    T hs[9];            // 1 - s/2, the forcing weight of Eq. 5 (s: Lambda)
+    T ns[9];            // -s
     T h2s7;             // 2 hs[7] (exact)
     T h6s1, nh6s2;      // 6 hs[1], -6 hs[2]: the forcing weights of S[1] = 6 v.F, S[2] = -6 v.F
     T c1, c2;           // C[1] = c1 tr Q, C[2] = c2 tr Q (Eq. 26)
@@ -106,7 +110,7 @@ template <typename T> struct StepArgs {   // CUtensorMap members give it their a
 // instance descriptors: 64 FP64 constant sets would not fit the 32 KB
 // argument space).  Slot k's tiles are first[k] .. first[k+1]-1, row-major
 // over tiles_x[k] columns; with a tile table (the interleaved schedule)
-// entry t gives (slot, x0, y0) instead.  A batch with more instances is
+// entry t gives (slot << 24 | x0, y0) instead.  A batch with more instances is
 // stepped by several launches.
 constexpr int kBatchLaunchMax = 64;
 struct SlotLattice {                     // the fields of Inst the step uses
@@ -121,7 +125,7 @@ template <> struct BatchPhys<float> {
 };
 template <typename T> struct BatchArgs {
     CUtensorMap tmap[kBatchLaunchMax];   // maps of the source time level of slot k
-    const int4* tiles;                   // tile table, or nullptr: tiles in slot order
+    const int2* tiles;                   // tile table, or nullptr: tiles in slot order
     int first[kBatchLaunchMax + 1];      // first tile of slot k; first[n] = tiles of the launch
     int tiles_x[kBatchLaunchMax];        // tile columns of slot k
     unsigned div_m[kBatchLaunchMax];     // division by tiles_x[k]: see tile_row()

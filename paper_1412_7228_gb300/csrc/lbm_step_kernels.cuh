@@ -661,10 +661,10 @@ __device__ __forceinline__ void step_body(const Inst* __restrict__ insts, int nt
             y0 = (tt / a.tiles_x) * BY;
         } else {
             if (a.tiles) {
-                const int4 tl = a.tiles[tt];
-                slot = tl.x;
-                x0 = tl.y;
-                y0 = tl.z;
+                const int2 tl = a.tiles[tt];
+                slot = tl.x >> 24;
+                x0 = tl.x & 0xffffff;
+                y0 = tl.y;
             } else {
                 int lo = 0, hi = a.n - 1;   // the last slot with first[slot] <= tt
                 while (lo < hi) {
