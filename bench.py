@@ -33,8 +33,8 @@ SEED = 14127228
 S_CFG = [1.0, 1.1, 1.1, 1.0, 1.1, 1.0, 1.1, 1.0, 1.0]
 A_CFG, KAPPA_CFG, TR_CFG, RHO0 = -0.85, 0.3, 0.7, 0.25
 # default tile configurations (indices into lbm_tile_config): the fastest at
-# 4096^2 when timed with lbm_autotune, 128 x 16 (FP32) and 64 x 16 (FP64)
-TILE_FP32, TILE_FP64 = 0, 5
+# 4096^2 when timed with lbm_autotune, 128 x 16 (FP32) and 32 x 32 (FP64)
+TILE_FP32, TILE_FP64 = 0, 6
 PEAK_FALLBACK_GBS = 6800.0
 
 

@@ -93,8 +93,8 @@ int lbm_eos_maxwell(const lbm_eos* eos, double* rho_g, double* rho_l, double* p0
 int lbm_laplace_fit(int n, const double* dp, const double* R, double* sigma, double* icpt,
                     double* r2);
 
-/* Self-check of the FP64 step's reciprocal, division and square root (two
- * Newton-Raphson, resp. Goldschmidt, steps from the hardware estimates)
+/* Self-check of the FP64 step's reciprocal, division and square root (one
+ * third-order, resp. two Goldschmidt, steps from the hardware estimates)
  * against IEEE-rounded 1/d, a/d and sqrt(d) on the current device: n values
  * of d spread evenly over [lo, hi], numerators a in [0.37, 0.87).  Writes
  * result[0..2] = the largest distances in units in the last place (rcp, div,
@@ -178,13 +178,14 @@ int lbm_batch_set_viscosity(lbm_ctx* ctx, int i, int enable, double nu_gas, doub
 
 /* Initial state f_a = M^-1 m_eq(rho, u) (Eq. 4) from host fields of nx*ny
  * doubles; ux, uy may be NULL (zero velocity).  Resets the step counter and
- * the instance's status.  The fields are copied to the device and checked
- * there first: a density that is not finite, positive and below the EOS's
+ * the instance's status.  The fields are checked on the device (copied there,
+ * or read in place where they lie in pinned memory): a density that is not finite, positive and below the EOS's
  * upper limit (4/b Carnahan-Starling, 1/b otherwise; any positive density
  * when G = 0) or a velocity that is not finite returns LBM_EINVAL and leaves
- * the instance as it was.  A context of one lattice of 2^20 nodes or more
- * takes the fields in row bands, each band checked and its populations
- * written while the next band is copied.  Synchronous. */
+ * the instance as it was.  A context of one lattice writes the populations
+ * into its other time level while it checks the fields, one of 2^20 nodes or
+ * more from pageable memory in row bands, each while the next is copied.
+ * Synchronous. */
 int lbm_init_density(lbm_ctx* ctx, const double* rho, const double* ux, const double* uy);
 int lbm_batch_init_density(lbm_ctx* ctx, int i, const double* rho, const double* ux,
                            const double* uy);
@@ -348,7 +349,8 @@ int lbm_mlp_adam_step(lbm_mlp* m, const float* X, const float* Y, int n, float l
                       float eps);
 /* Train for `epochs` passes over n samples in shuffled minibatches of
  * `batch` (seeded), Adam(lr, 0.9, 0.999, 1e-8); loss_per_epoch (nullable)
- * receives the mean minibatch loss of each epoch. */
+ * receives the mean minibatch loss of each epoch.  The first call allocates
+ * the buffers of the sample orders (LBM_ENOMEM when it cannot). */
 int lbm_mlp_train(lbm_mlp* m, const float* X, const float* Y, int n, int epochs, int batch, float lr,
                   unsigned long long seed, float* loss_per_epoch);
 /* Forward pass: n raw inputs -> n raw outputs (de-standardised). */
