@@ -235,19 +235,21 @@ template <> struct Fast<double> {
     }
 };
 
-// psi = sqrt(W / D) = W / sqrt(W D) for D > 0.  1 / sqrt(x) comes from the
+// psi = sqrt(W / D) = |W| / sqrt(W D): the positive root also beyond the law's
+// pole, where W and D are both negative.  1 / sqrt(x) comes from the
 // hardware estimate y refined by one third-order step (Householder's
 // iteration): with d = 1 - x y^2, y + y d (1/2 + 3/8 d) leaves an error of
 // 5/16 d^3, far below the last place from an estimate good to 2^-20; three
-// FP64 instructions fewer than two second-order steps.  A negative radicand
-// gives NaN (as the square root does), psi(W = 0) = 0.
+// FP64 instructions fewer than two second-order steps (the absolute value is
+// an operand's modifier).  A negative radicand gives NaN (as the square root
+// does), psi(W = 0) = 0.
 __device__ __forceinline__ double psi_fold_fp64(double W, double D) {
     const double x = W * D;
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double d = fma(-(x * y), y, 1.0);
     const double r = fma(y * d, fma(d, 0.375, 0.5), y);
-    return W == 0.0 ? 0.0 : W * r;
+    return W == 0.0 ? 0.0 : fabs(W) * r;
 }
 
 // ---- PTX helpers --------------------------------------------------------

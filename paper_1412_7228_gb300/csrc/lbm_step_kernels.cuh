@@ -221,7 +221,7 @@ template <int EOSK, typename T> __device__ __forceinline__ T radicand_step(const
 //   Peng-Robinson      D = d e, e = 1 + 2 b rho - (b rho)^2,
 //                      W = rho [kR e - (kAa rho + k3 e) d];
 // with kR = (2/G) K R T, kA = (2/G) K a, kAa = (2/G) K a alpha(T),
-// k3 = (2/G)/3.  Then psi = W / sqrt(W D) (psi_fold_fp64).
+// k3 = (2/G)/3.  Then psi = |W| / sqrt(W D) (psi_fold_fp64).
 template <int EOSK>
 __device__ __forceinline__ double psi_fp64(const EosRegs<double>& E, double kR, double kA, double kAa, double k3,
                                            double rho) {

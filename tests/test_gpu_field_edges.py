@@ -1,0 +1,70 @@
+"""Fields and statistics at the edges of their arguments: densities
+beyond the law's pole.
+
+Tolerances.  psi^2 is a difference of terms of the size of the pressure; with
+|1 - b rho| >= 0.09 and 2^-53 per operation over some 40 operations its
+relative error is below 40 x 2^-53 x 3 / 0.09 = 1.5e-13: 1e-12 covers it, and
+the velocity's share of it too.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+from test_gpu_reductions import _fields, _law, _pressure
+
+pytestmark = pytest.mark.gpu
+
+BEYOND = {"cs": ((0.05, 0.42), (1.2, 1.6)), "vdw": ((0.5, 7.0), (11.6, 14.0)), "pr": ((0.5, 7.0), (11.6, 14.0))}
+
+
+@pytest.fixture(scope="module")
+def P():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1412_7228_gb300 as P
+    P.lib()
+    return P
+
+
+def _across_the_pole(P, kind, prec, nx=45, ny=37):
+    """A lattice whose nodes lie on both sides of the law's pole: without the
+    interaction any positive density is a valid initial one."""
+    eos, A = _law(P, kind)
+    (a, b), (c, d) = BEYOND[kind]
+    rng = np.random.default_rng(5)
+    rho0 = np.where(rng.random((ny, nx)) < 0.5, rng.uniform(a, b, (ny, nx)), rng.uniform(c, d, (ny, nx)))
+    lat = P.Lattice(nx, ny, prec)
+    lat.set_params(eos, A, 0.2, G=0.0, s=[1.0] * 9, rho_ref=a)
+    lat.init_density(rho0)
+    lat.set_params(eos, A, 0.2, G=-1.0, s=[1.0] * 9, rho_ref=a)
+    return lat, eos, A, rho0
+
+
+@pytest.mark.parametrize("prec", [1, 2])
+@pytest.mark.parametrize("kind", ["cs", "vdw", "pr"])
+def test_psi_is_the_positive_root_on_both_sides_of_the_pole(P, kind, prec):
+    lat, eos, A, _ = _across_the_pole(P, kind, prec)
+    rho, ux, uy, psi = _fields(P, eos, A, lat.read_populations())
+    assert (-2.0 * (_pressure(P, eos, rho) - rho / 3.0) > 0.0).all() and (rho * eos.b / (4.0 if kind == "cs" else 1.0) > 1.0).any()
+    for which in (("psi",), ("rho", "ux", "uy", "psi")):
+        got = lat.read_fields(which=which)
+        assert (np.abs(got["psi"] - psi) <= 1e-12 * psi).all()
+    assert np.abs(got["ux"] - ux).max() <= 1e-12 * np.abs(ux).max()
+    assert np.abs(got["uy"] - uy).max() <= 1e-12 * np.abs(uy).max()
+    st = lat.stats()
+    assert abs(st["umax"] - np.sqrt((ux * ux + uy * uy).max())) <= 1e-12 * st["umax"]
+    lat.close()
+
+
+@pytest.mark.parametrize("kind", ["cs", "vdw", "pr"])
+def test_an_fp64_step_across_the_pole_is_the_oracle_s(P, kind):
+    lat, eos, A, rho0 = _across_the_pole(P, kind, P.LBM_FP64)
+    law = {P.LBM_EOS_CS: O.EOS_CS, P.LBM_EOS_VDW: O.EOS_VDW, P.LBM_EOS_PR: O.EOS_PR}[eos.kind]
+    op = O.Params(eos=law, a=eos.a, b=eos.b, R=eos.R, K=eos.K, T=eos.T, omega=eos.omega, Tc=eos.Tc, A=A, kappa=0.2,
+                  G=-1.0, s=[1.0] * 9)
+    f = O.init_equilibrium(rho0)
+    O.step(op, f, 1)
+    lat.step(1)
+    assert np.abs(lat.read_populations() - f).max() <= 1e-12 * np.abs(f).max()
+    lat.close()
