@@ -698,9 +698,12 @@ int status_code(int st) {
     return (st & lbm::ST_UNSTABLE) ? LBM_EUNSTABLE : ((st & lbm::ST_TIMEOUT) ? LBM_ETIMEOUT : LBM_OK);
 }
 
+// The status after all the work enqueued so far: the copy is the stream's own
+// (the legacy stream's copies do not wait for a non-blocking stream).
 int status_of(lbm_ctx* c, int i, int* code) {
     int st = 0;
-    CK(c, cudaMemcpy(&st, c->d_status + i, sizeof(int), cudaMemcpyDeviceToHost));
+    CK(c, cudaMemcpyAsync(&st, c->d_status + i, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    CK(c, cudaStreamSynchronize(c->stream));
     *code = status_code(st);
     return LBM_OK;
 }
@@ -1465,7 +1468,6 @@ int lbm_status(lbm_ctx* c, int i) {
     int rc = check_idx(c, i);
     if (rc) return rc;
     CK(c, cudaSetDevice(c->device));
-    CK(c, cudaStreamSynchronize(c->stream));
     int code = LBM_OK;
     rc = status_of(c, i, &code);
     return rc ? rc : code;
