@@ -17,6 +17,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "lbm_eos_host.h"
+#include "lbm_host_rules.h"
 #include "lbm_init.h"
 #include "lbm_internal.cuh"
 
@@ -874,7 +875,8 @@ int ensure_copy_stream(lbm_ctx* c) {
 
 // How kernels can reach the n values at p: pinned host memory that they may
 // read, or write where asked (*dev: its address for them), ordinary host
-// memory, or anything else (left to the copies, which know what to do with it).
+// memory, or anything else (left to the copies, which know what to do with it;
+// they also take an array at any address, the kernels only whole values).
 enum HostKind { kPinned, kPageable, kOther };
 template <typename O> HostKind host_kind(O* p, size_t n, bool write, O** dev) {
     cudaPointerAttributes a, b;
@@ -885,6 +887,7 @@ template <typename O> HostKind host_kind(O* p, size_t n, bool write, O** dev) {
     if (a.type == cudaMemoryTypeUnregistered && b.type == cudaMemoryTypeUnregistered) return kPageable;
     // pinned from the first value to the last, in one mapping, and not read-only
     if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer || !b.devicePointer) return kOther;
+    if (!lbm::in_place({reinterpret_cast<uintptr_t>(a.devicePointer), n * sizeof(O)}, sizeof(O))) return kOther;
     if (static_cast<char*>(b.devicePointer) - static_cast<char*>(a.devicePointer) !=
         static_cast<std::ptrdiff_t>((n - 1) * sizeof(O)))
         return kOther;

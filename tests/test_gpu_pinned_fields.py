@@ -77,3 +77,31 @@ def test_a_refused_pinned_field_leaves_the_lattice_as_it_was(P, nx, ny):
         assert ei.value.code == P.lbm.LBM_EINVAL
         assert np.array_equal(lat.read_populations(), before) and lat.status(0) == 0 and lat.steps_done == 3
     lat.close()
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("nx,ny", [(5, 3), (181, 180), (1100, 1000)])
+def test_pinned_arrays_at_any_address(P, nx, ny, dtype):
+    """A view of pinned bytes behind a header need not be aligned: such arrays
+    go through the copies, read and written."""
+    import torch
+    lat = _lattice(P, nx, ny, P.LBM_FP32)
+    rho, ux, uy = _inputs(nx, ny, dtype)
+    lat.init_density(rho, ux, uy)
+    want, state = lat.read_fields(dtype=dtype), lat.read_populations()
+    size = rho.nbytes
+    raw = torch.zeros(4 * (size + 3) + 8, dtype=torch.uint8).pin_memory().numpy()
+    views = [raw[k * (size + 3) + 1:k * (size + 3) + 1 + size].view(dtype).reshape(ny, nx) for k in range(4)]
+    assert not any(v.ctypes.data % rho.itemsize == 0 for v in views[:1] + views[2:3])
+    out = dict(zip(("rho", "ux", "uy", "psi"), views))
+    for which in (("rho",), ("rho", "psi"), ("rho", "ux", "uy", "psi")):
+        raw[:] = 0
+        got = lat.read_fields(which=which, out=out, dtype=dtype)
+        for k in which:
+            assert got[k] is out[k] and np.array_equal(got[k], want[k]), k
+    for v, a in zip(views, (rho, ux, uy)):
+        v[...] = a
+    lat.init_density(np.full((ny, nx), 0.25))
+    lat.init_density(*views[:3])
+    assert np.array_equal(lat.read_populations(), state)
+    lat.close()
