@@ -885,11 +885,12 @@ template <typename O> HostKind host_kind(O* p, size_t n, bool write, O** dev) {
         return kOther;
     }
     if (a.type == cudaMemoryTypeUnregistered && b.type == cudaMemoryTypeUnregistered) return kPageable;
-    // pinned from the first value to the last, in one mapping, and not read-only
-    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer || !b.devicePointer) return kOther;
-    if (!lbm::in_place({reinterpret_cast<uintptr_t>(a.devicePointer), n * sizeof(O)}, sizeof(O))) return kOther;
-    if (static_cast<char*>(b.devicePointer) - static_cast<char*>(a.devicePointer) !=
-        static_cast<std::ptrdiff_t>((n - 1) * sizeof(O)))
+    // pinned, in one mapped range, and not read-only
+    if (a.type != cudaMemoryTypeHost || !a.devicePointer) return kOther;
+    lbm::Span range = {};
+    if (!lbm::pointer_attribute(CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, a.devicePointer, &range.at) ||
+        !lbm::pointer_attribute(CU_POINTER_ATTRIBUTE_RANGE_SIZE, a.devicePointer, &range.bytes) ||
+        !lbm::in_place({reinterpret_cast<uintptr_t>(a.devicePointer), n * sizeof(O)}, sizeof(O), range))
         return kOther;
     unsigned flags = 0;
     if (write && (cudaHostGetFlags(&flags, const_cast<std::remove_const_t<O>*>(p)) != cudaSuccess ||

@@ -15,7 +15,12 @@ struct Span {
 
 // Whether kernels may access the array as values of `size` bytes where it
 // lies: at a multiple of the size (a kernel's access to any other address
-// faults).
-inline bool in_place(Span array, size_t size) { return array.at % size == 0; }
+// faults), and within one mapped range, the one that its first byte is in.
+// (The addresses of its two ends do not tell: with unified addressing they
+// are as far apart for two ranges with unmapped pages between them.)
+inline bool in_place(Span array, size_t size, Span range) {
+    return array.at % size == 0 && array.at >= range.at && array.at - range.at <= range.bytes &&
+           array.bytes <= range.bytes - (array.at - range.at);
+}
 
 }  // namespace lbm

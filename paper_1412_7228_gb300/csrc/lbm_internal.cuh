@@ -363,6 +363,9 @@ cudaError_t cluster_run(const Inst& host, int parity, int nsteps, cudaStream_t s
 constexpr size_t kPinnedBlock = (size_t(1) << 16) + 256;
 void* pinned_get(size_t bytes);
 void pinned_put(void* p);
+// An attribute of the memory at p, as the driver has it (out: of the
+// attribute's type); false when p is not known to it.
+bool pointer_attribute(CUpointer_attribute what, const void* p, void* out);
 
 // What a call reads back besides its arrays, written by the device into
 // pinned host memory mapped for it: the sums of a reduction with its status

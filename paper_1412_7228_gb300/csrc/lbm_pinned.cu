@@ -56,6 +56,19 @@ Pool& pool() {
 
 }  // namespace
 
+bool pointer_attribute(CUpointer_attribute what, const void* p, void* out) {
+    typedef CUresult (*Get)(void*, CUpointer_attribute, CUdeviceptr);
+    static const Get get = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const bool ok = cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &fn, 12000, cudaEnableDefault, &q) ==
+                            cudaSuccess &&
+                        q == cudaDriverEntryPointSuccess;
+        return ok ? reinterpret_cast<Get>(fn) : nullptr;
+    }();
+    return get && get(out, what, reinterpret_cast<CUdeviceptr>(p)) == CUDA_SUCCESS;
+}
+
 void* pinned_get(size_t bytes) {
     if (bytes <= kPinnedBlock)
         if (void* p = pool().take()) return p;

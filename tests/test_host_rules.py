@@ -26,6 +26,22 @@ def ask(tmp_path, body):
 def test_arrays_off_their_values_alignment_are_left_to_the_copies(tmp_path):
     got = ask(tmp_path, """
         for (size_t size : {4, 8})
-            for (uintptr_t off = 0; off < 17; ++off) printf("%d ", lbm::in_place({0x7f0000001000 + off, 100 * size}, size));
+            for (uintptr_t off = 0; off < 17; ++off)
+                printf("%d ", lbm::in_place({0x7f0000001000 + off, 100 * size}, size, {0x7f0000000000, 1 << 20}));
     """)
     assert got == [int(off % size == 0) for size in (4, 8) for off in range(17)]
+
+
+def test_arrays_beyond_one_mapped_range_are_left_to_the_copies(tmp_path):
+    """Ranges of 0x10000 bytes at 0x20000 and, unmapped pages between them, at
+    0x40000; also one that ends with the address space."""
+    got = ask(tmp_path, """
+        const lbm::Span first = {0x20000, 0x10000}, last = {~uintptr_t(0) - 0xffff, 0xffff};
+        printf("%d %d %d ", lbm::in_place({0x20000, 0x10000}, 4, first), lbm::in_place({0x2fffc, 4}, 4, first),
+               lbm::in_place({0x23000, 0x1000}, 8, first));
+        printf("%d %d %d %d ", lbm::in_place({0x20000, 0x10004}, 4, first), lbm::in_place({0x2f000, 0x12000}, 4, first),
+               lbm::in_place({0x1f000, 0x2000}, 4, first), lbm::in_place({0x40000, 4}, 4, first));
+        printf("%d %d %d ", lbm::in_place({last.at, 0xfffc}, 4, last), lbm::in_place({last.at + 0x8000, ~size_t(3)}, 4, last),
+               lbm::in_place({0x20000, 4}, 4, {0, 0}));
+    """)
+    assert got == [1, 1, 1, 0, 0, 0, 0, 1, 0, 0]
