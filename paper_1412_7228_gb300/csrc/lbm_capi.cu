@@ -1058,18 +1058,24 @@ template <typename O> int read_fields_t(lbm_ctx* c, int i, O* rho, O* ux, O* uy,
             direct = kind == kPageable && staged <= kStageBytes;
         }
         if (direct && !groups.empty()) {
-            for (size_t k = 0; k < groups.size(); ++k) {
-                const Group& g = groups[k];
-                const lbm::Notice note = k + 1 == groups.size() ? next_notice(c) : lbm::Notice{c->h_red, nullptr, 0};
-                void* dev[4] = {};
-                for (int f : g.f) dev[f] = to[f];
-                if (g.flow)
-                    CK(c, lbm::aux_flow(c->h[i], c->d_inst + i, c->parity, 0, ny, dev, f32, note, c->stream));
-                else
-                    CK(c, lbm::aux_field(c->h[i], c->d_inst + i, c->parity, g.f[0], 0, ny, dev[g.f[0]], f32, note,
-                                         c->stream));
+            auto issue = [&]() -> int {
+                for (size_t k = 0; k < groups.size(); ++k) {
+                    const Group& g = groups[k];
+                    const lbm::Notice note = k + 1 == groups.size() ? next_notice(c) : lbm::Notice{c->h_red, nullptr, 0};
+                    void* dev[4] = {};
+                    for (int f : g.f) dev[f] = to[f];
+                    if (g.flow)
+                        CK(c, lbm::aux_flow(c->h[i], c->d_inst + i, c->parity, 0, ny, dev, f32, note, c->stream));
+                    else
+                        CK(c, lbm::aux_field(c->h[i], c->d_inst + i, c->parity, g.f[0], 0, ny, dev[g.f[0]], f32, note,
+                                             c->stream));
+                }
+                return wait_notice(c);
+            };
+            if ((rc = issue())) {   // no write into the caller's arrays may outlive the call
+                cudaStreamSynchronize(c->stream);
+                return rc;
             }
-            if ((rc = wait_notice(c))) return rc;
             for (int f = 0; f < 4; ++f)
                 if (outs[f] && reinterpret_cast<char*>(to[f]) >= c->h_stage &&
                     reinterpret_cast<char*>(to[f]) < c->h_stage + kStageBytes)
