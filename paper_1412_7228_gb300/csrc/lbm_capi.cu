@@ -247,7 +247,8 @@ struct lbm_ctx {
     double* d_partials = nullptr;
     double* d_result = nullptr;
     unsigned* d_ticket = nullptr;           // of the reductions' last block; zero between launches
-    lbm::Reduced* h_red = nullptr;          // pinned, mapped: the device writes results and the status here
+    lbm::Pinned pinned;
+    lbm::Reduced* h_red = nullptr;          // in it (pinned, mapped): the device writes results and the status here
     unsigned call = 0;                      // number of the last call that waits for them (h_red->call)
     char* h_stage = nullptr;                // behind it, kStageBytes: small fields on their way to pageable memory
     double* d_scratch = nullptr;
@@ -1299,7 +1300,8 @@ int lbm_batch_create(lbm_ctx** out, int n, const int* nx, const int* ny, int pre
         c->owns = true;
         c->buf_bytes = c->L.total;
     }
-    void* const red = lbm::pinned_get(256 + kStageBytes);
+    c->pinned = lbm::pinned_get(256 + kStageBytes);
+    void* const red = c->pinned.p;
     if (!red) {
         lbm_destroy(c);
         return LBM_ENOMEM;
@@ -1359,7 +1361,7 @@ void lbm_destroy(lbm_ctx* c) {
     }
     for (auto& e : c->band_done)
         if (e) cudaEventDestroy(e);
-    lbm::pinned_put(c->h_red);
+    lbm::pinned_put(c->pinned);
     if (c->owns && c->buf) cudaFree(c->buf);
     delete c;
 }

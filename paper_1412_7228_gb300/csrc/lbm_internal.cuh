@@ -18,6 +18,7 @@
 #include <stdint.h>
 
 #include "../../include/lbm.h"
+#include "lbm_pinned_pool.h"
 
 namespace lbm {
 
@@ -358,11 +359,12 @@ bool cluster_supported(int prec, int nx, int ny);
 cudaError_t cluster_run(const Inst& host, int parity, int nsteps, cudaStream_t st);
 
 // Pinned host memory, mapped for every device (lbm_pinned.cu): up to
-// kPinnedBlock bytes come from a small slab, more straight from the driver.
-// NULL when there is none.  Given back once nothing uses it any more.
+// kPinnedBlock bytes come from a small slab of the current CUDA context, more
+// straight from the driver.  p NULL when there is none.  Given back once
+// nothing uses it any more.
 constexpr size_t kPinnedBlock = (size_t(1) << 16) + 256;
-void* pinned_get(size_t bytes);
-void pinned_put(void* p);
+Pinned pinned_get(size_t bytes);
+void pinned_put(const Pinned& b);
 // An attribute of the memory at p, as the driver has it (out: of the
 // attribute's type); false when p is not known to it.
 bool pointer_attribute(CUpointer_attribute what, const void* p, void* out);

@@ -675,7 +675,8 @@ struct lbm_mlp {
     float* loss[2] = {};
     void* stage = nullptr;   // the memory these are in
     cudaEvent_t done[2] = {};
-    float* h_io = nullptr;   // pinned and mapped: NI + NO floats of up to io_n samples (or the parameters), for the kernels
+    lbm::Pinned pinned;
+    float* h_io = nullptr;   // in it (pinned and mapped): NI + NO floats of up to io_n samples (or the parameters), for the kernels
     int io_n = 0;
     int cap = 0;             // samples (and minibatches) each of them holds
     int adam_t = 0;
@@ -854,7 +855,8 @@ int lbm_mlp_create(lbm_mlp** out, int max_samples, unsigned long long seed, void
         return c.used;
     };
     const bool ok = cudaMalloc(&m->dev, cut({nullptr, 0})) == cudaSuccess &&
-                    (m->h_io = static_cast<float*>(lbm::pinned_get(io_bytes(m)))) != nullptr;
+                    (m->pinned = lbm::pinned_get(io_bytes(m))).p != nullptr;
+    m->h_io = static_cast<float*>(m->pinned.p);
     cut({ok ? static_cast<char*>(m->dev) : nullptr, 0});
     if (!ok) {
         cudaGetLastError();
@@ -891,7 +893,7 @@ void lbm_mlp_destroy(lbm_mlp* m) {
     if (m->P) cudaStreamSynchronize(m->st);   // also: nothing uses the pinned memory any more
     if (m->dev) cudaFree(m->dev);
     if (m->stage) cudaFreeHost(m->stage);
-    lbm::pinned_put(m->h_io);
+    lbm::pinned_put(m->pinned);
     for (cudaEvent_t e : m->done)
         if (e) cudaEventDestroy(e);
     delete m;
