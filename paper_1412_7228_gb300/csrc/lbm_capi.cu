@@ -42,9 +42,20 @@ constexpr int kGraphLevels = 5;                            // captured graphs of
 constexpr int kGraphSteps = 2 << (kGraphLevels - 1);       // the longest: 32 steps
 constexpr int kReadBands = 8;                              // row bands of a large field's transfers
 constexpr size_t kReadBandMin = size_t(1) << 20;           // nodes from which the read-back is banded
-// Pinned stage of a context for small fields.  Read of rho into pageable memory:
-// 64^2 FP32 17.2 -> 12.7 us staged, 256^2 19.0 -> 27.0 (the host's copy takes over).
+// Pinned stage that a read-back of small fields borrows.  Read of rho into pageable
+// memory: 64^2 FP32 17.2 -> 12.7 us staged, 256^2 19.0 -> 27.0 (the host's copy takes over).
 constexpr size_t kStageBytes = size_t(1) << 16;
+static_assert(kStageBytes <= lbm::kPinnedBlock, "the stage is a block of the pool");
+struct Stage {
+    lbm::Pinned block;
+    Stage() = default;
+    Stage(const Stage&) = delete;
+    ~Stage() { lbm::pinned_put(block); }
+    char* get() {
+        if (!block.p) block = lbm::pinned_get(kStageBytes);
+        return static_cast<char*>(block.p);
+    }
+};
 
 // The TMA tensor maps of one instance's two time levels (host copies; the
 // kernels receive them in their argument blocks).
@@ -250,7 +261,6 @@ struct lbm_ctx {
     lbm::Pinned pinned;
     lbm::Reduced* h_red = nullptr;          // in it (pinned, mapped): the device writes results and the status here
     unsigned call = 0;                      // number of the last call that waits for them (h_red->call)
-    char* h_stage = nullptr;                // behind it, kStageBytes: small fields on their way to pageable memory
     double* d_scratch = nullptr;
     int parity = 0;
     long long steps = 0, launches = 0;
@@ -1042,21 +1052,23 @@ template <typename O> int read_fields_t(lbm_ctx* c, int i, O* rho, O* ux, O* uy,
     }
     c->h_red->status = 0;
     // where they can, the kernels write straight to where the host reads: the
-    // caller's arrays if they are pinned, else (small ones) the context's
+    // caller's arrays if they are pinned, else (small ones) a pinned
     // stage; no copy is enqueued and no stream waited for (rho into pinned
     // memory, FP32: 64^2 15.3 -> 11.3 us per call, 512^2 29.3 -> 19.0, 1024^2 in
     // bands 67 -> 40 us)
     {
+        Stage stage;   // given back at the end: the kernels are done with it on every way out
         O* to[4] = {};
         size_t staged = 0;
-        bool direct = true;
+        bool direct = true, through[4] = {};
         for (int f = 0; f < 4 && direct; ++f) {
             if (!outs[f]) continue;
             const HostKind kind = host_kind(outs[f], N, true, &to[f]);
             if (kind == kPinned) continue;
-            to[f] = reinterpret_cast<O*>(c->h_stage + staged);
+            const size_t at = staged;
             staged += (N * sizeof(O) + 15) / 16 * 16;
-            direct = kind == kPageable && staged <= kStageBytes;
+            direct = through[f] = kind == kPageable && staged <= kStageBytes && stage.get();
+            if (direct) to[f] = reinterpret_cast<O*>(stage.get() + at);
         }
         if (direct && !groups.empty()) {
             auto issue = [&]() -> int {
@@ -1078,9 +1090,7 @@ template <typename O> int read_fields_t(lbm_ctx* c, int i, O* rho, O* ux, O* uy,
                 return rc;
             }
             for (int f = 0; f < 4; ++f)
-                if (outs[f] && reinterpret_cast<char*>(to[f]) >= c->h_stage &&
-                    reinterpret_cast<char*>(to[f]) < c->h_stage + kStageBytes)
-                    std::memcpy(outs[f], to[f], N * sizeof(O));
+                if (through[f]) std::memcpy(outs[f], to[f], N * sizeof(O));
             return status_code(c->h_red->status);
         }
     }
@@ -1300,16 +1310,14 @@ int lbm_batch_create(lbm_ctx** out, int n, const int* nx, const int* ny, int pre
         c->owns = true;
         c->buf_bytes = c->L.total;
     }
-    c->pinned = lbm::pinned_get(256 + kStageBytes);
-    void* const red = c->pinned.p;
-    if (!red) {
+    static_assert(sizeof(lbm::Reduced) <= lbm::kPinnedSmall, "one of the small blocks");
+    c->pinned = lbm::pinned_get(sizeof(lbm::Reduced));
+    if (!c->pinned.p) {
         lbm_destroy(c);
         return LBM_ENOMEM;
     }
-    std::memset(red, 0, sizeof(lbm::Reduced));
-    static_assert(sizeof(lbm::Reduced) <= 256, "the stage lies behind the results");
-    c->h_red = static_cast<lbm::Reduced*>(red);
-    c->h_stage = static_cast<char*>(red) + 256;
+    std::memset(c->pinned.p, 0, sizeof(lbm::Reduced));
+    c->h_red = static_cast<lbm::Reduced*>(c->pinned.p);
     if (cudaMemsetAsync(c->buf, 0, c->L.total, c->stream) != cudaSuccess || cudaStreamSynchronize(c->stream) != cudaSuccess) {
         lbm_destroy(c);
         return LBM_ECUDA;

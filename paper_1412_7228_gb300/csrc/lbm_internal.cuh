@@ -359,10 +359,10 @@ bool cluster_supported(int prec, int nx, int ny);
 cudaError_t cluster_run(const Inst& host, int parity, int nsteps, cudaStream_t st);
 
 // Pinned host memory, mapped for every device (lbm_pinned.cu): up to
-// kPinnedBlock bytes come from a small slab of the current CUDA context, more
-// straight from the driver.  p NULL when there is none.  Given back once
-// nothing uses it any more.
-constexpr size_t kPinnedBlock = (size_t(1) << 16) + 256;
+// kPinnedSmall and up to kPinnedBlock bytes come from slabs of the current
+// CUDA context, more straight from the driver.  p NULL when there is none.
+// Given back once nothing uses it any more.
+constexpr size_t kPinnedSmall = 256, kPinnedBlock = (size_t(1) << 16) + 256;
 Pinned pinned_get(size_t bytes);
 void pinned_put(const Pinned& b);
 // An attribute of the memory at p, as the driver has it (out: of the

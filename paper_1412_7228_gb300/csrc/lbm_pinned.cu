@@ -1,16 +1,15 @@
 // lbm_pinned.cu -- pinned host memory, mapped for the devices, of the contexts
-// and networks.  Allocating and freeing it takes the driver about 100 and 180 us,
-// three times what making a small context takes otherwise, so the first
-// owner allocates a slab of kBlocks blocks of one size, which serves up to
-// that many owners at a time and is given back at exit; further owners, and
-// larger requests, go to the driver.  A block's owner has waited for its
-// stream before it lets go.  The bookkeeping is lbm_pinned_pool.h's.
+// and networks.  It comes in slabs: of 256 blocks for what each context keeps
+// (64 KB), and of 8 for the networks and for the stage that a read-back borrows
+// while it lasts (half a megabyte), so that making a context costs no
+// allocation by the driver however many are open (64 of 64^2 at once: 23.3 us to
+// make and 1.1 to close each; with an allocation of its own for each beyond the
+// eighth 30.0 and 6.7).  Larger requests go to the driver.  A block's owner has waited
+// for its stream before it lets go.  The bookkeeping is lbm_pinned_pool.h's.
 #include "lbm_internal.cuh"
 
 namespace lbm {
 namespace {
-
-constexpr int kBlocks = 8;   // half a megabyte
 
 // A function of the driver, which the library does not link.
 template <class F> F driver_function(const char* name) {
@@ -46,8 +45,12 @@ struct CudaDriver {
         return pointer_attribute(CU_POINTER_ATTRIBUTE_BUFFER_ID, p, &v) ? v : 0;
     }
 };
+PinnedPool<CudaDriver>& small_pool() {
+    static PinnedPool<CudaDriver> p(kPinnedSmall, 256);
+    return p;
+}
 PinnedPool<CudaDriver>& pool() {
-    static PinnedPool<CudaDriver> p(kPinnedBlock, kBlocks);
+    static PinnedPool<CudaDriver> p(kPinnedBlock, 8);
     return p;
 }
 
@@ -58,8 +61,17 @@ bool pointer_attribute(CUpointer_attribute what, const void* p, void* out) {
     return get && get(out, what, reinterpret_cast<CUdeviceptr>(p)) == CUDA_SUCCESS;
 }
 
-Pinned pinned_get(size_t bytes) { return pool().get(bytes); }
+Pinned pinned_get(size_t bytes) {
+    if (bytes <= kPinnedSmall) return small_pool().get();
+    if (bytes <= kPinnedBlock) return pool().get();
+    Pinned b;
+    b.p = CudaDriver().allocate(bytes);
+    return b;
+}
 
-void pinned_put(const Pinned& b) { pool().put(b); }
+void pinned_put(const Pinned& b) {
+    if (b.slab) small_pool().put(b) || pool().put(b);
+    else if (b.p) CudaDriver().release(b.p);
+}
 
 }  // namespace lbm

@@ -25,6 +25,10 @@ struct Pinned {
 // Driver: void* allocate(size_t); void release(void*); the process-wide ids
 // unsigned long long context() of the current context and
 // unsigned long long id(void*) of the live allocation at an address (0: none).
+//
+// A context whose slabs are all taken gets another, and one that becomes empty
+// is given back unless it is the context's only empty one: the pinned memory
+// follows the owners that are alive, and a slab's cost is spread over them.
 template <class Driver> class PinnedPool {
 public:
     PinnedPool(size_t block, int blocks) : block_(block), blocks_(blocks) {}
@@ -32,24 +36,26 @@ public:
         for (Slab& s : slabs_)
             if (alive(s)) driver_.release(s.base);
     }
-    Pinned get(size_t bytes) {
-        if (bytes <= block_) {
-            const Pinned b = take();
-            if (b.p) return b;
-        }
-        Pinned b;
-        b.p = driver_.allocate(bytes);
+    // a block, or where there is no slab for it memory of its own
+    Pinned get() {
+        Pinned b = take();
+        if (!b.p) b.p = driver_.allocate(block_);
         return b;
     }
-    void put(const Pinned& b) {
-        if (!b.p) return;
-        if (!b.slab) {
-            driver_.release(b.p);
-            return;
-        }
+    // whether b was one of this pool's slabs' blocks, now free again
+    bool put(const Pinned& b) {
         std::lock_guard<std::mutex> lock(mu_);
-        for (Slab& s : slabs_)
-            if (s.id == b.slab) s.used[static_cast<size_t>(static_cast<char*>(b.p) - s.base) / block_] = 0;
+        const auto from = std::find_if(slabs_.begin(), slabs_.end(), [&](const Slab& s) { return s.id == b.slab; });
+        if (from == slabs_.end()) return false;
+        from->used[static_cast<size_t>(static_cast<char*>(b.p) - from->base) / block_] = 0;
+        if (--from->taken) return true;
+        for (const Slab& s : slabs_)
+            if (s.id != from->id && s.context == from->context && !s.taken) {
+                if (alive(*from)) driver_.release(from->base);
+                slabs_.erase(from);
+                break;
+            }
+        return true;
     }
     Driver& driver() { return driver_; }
 
@@ -58,17 +64,18 @@ private:
         char* base;
         unsigned long long id, context;
         std::vector<char> used;
+        int taken;
     };
     bool alive(const Slab& s) { return driver_.id(s.base) == s.id; }
-    // a free block of the current context's slab, or none
+    // a free block of the current context's slabs, or none
     Pinned take() {
         std::lock_guard<std::mutex> lock(mu_);
         slabs_.erase(std::remove_if(slabs_.begin(), slabs_.end(), [&](const Slab& s) { return !alive(s); }), slabs_.end());
         const unsigned long long context = driver_.context();
-        Slab* mine = nullptr;
+        Slab* from = nullptr;
         for (Slab& s : slabs_)
-            if (s.context == context) mine = &s;
-        if (!mine) {
+            if (s.context == context && s.taken < blocks_) from = &s;
+        if (!from) {
             void* const base = driver_.allocate(block_ * blocks_);
             if (!base) return {};
             const unsigned long long id = driver_.id(base);
@@ -76,18 +83,16 @@ private:
                 driver_.release(base);
                 return {};
             }
-            slabs_.push_back({static_cast<char*>(base), id, context, std::vector<char>(blocks_, 0)});
-            mine = &slabs_.back();
+            slabs_.push_back({static_cast<char*>(base), id, context, std::vector<char>(blocks_, 0), 0});
+            from = &slabs_.back();
         }
-        for (int k = 0; k < blocks_; ++k)
-            if (!mine->used[k]) {
-                mine->used[k] = 1;
-                Pinned b;
-                b.p = mine->base + k * block_;
-                b.slab = mine->id;
-                return b;
-            }
-        return {};
+        const size_t k = std::find(from->used.begin(), from->used.end(), 0) - from->used.begin();
+        from->used[k] = 1;
+        ++from->taken;
+        Pinned b;
+        b.p = from->base + k * block_;
+        b.slab = from->id;
+        return b;
     }
 
     const size_t block_;

@@ -68,15 +68,12 @@ def test_blocks_are_distinct_and_used_again(tmp_path):
     lbm::PinnedPool<Fake> pool(256, 4);
     Pinned b[6];
     std::set<void*> seen;
-    for (auto& x : b) { x = pool.get(200); assert(x.p && seen.insert(x.p).second); memset(x.p, 1, 200); }
-    Pinned big = pool.get(5000);
-    assert(big.p && big.slab == 0);
-    pool.put(big);
-    for (auto& x : b) pool.put(x);
-    Pinned again = pool.get(256);
-    assert(again.slab == b[0].slab && again.p == b[0].p);
-    pool.put(again);
-    pool.put({});
+    for (auto& x : b) { x = pool.get(); assert(x.p && x.slab && seen.insert(x.p).second); memset(x.p, 1, 256); }
+    for (auto& x : b) assert(pool.put(x));
+    Pinned again = pool.get();
+    assert(seen.count(again.p));
+    assert(pool.put(again));
+    assert(!pool.put({}));
     """)
 
 
@@ -85,13 +82,13 @@ def test_a_lost_context_takes_its_slab_with_it(tmp_path):
     that now lies where it did."""
     check(tmp_path, """
     lbm::PinnedPool<Fake> pool(256, 4);
-    Pinned old = pool.get(256);
+    Pinned old = pool.get();
     pool.driver().lose(1);
-    Pinned young = pool.get(256);
+    Pinned young = pool.get();
     assert(young.p == old.p && young.slab != old.slab);       // the same address
     assert(pool.driver().id(young.p) == young.slab);          // and live
     pool.put(old);
-    Pinned other = pool.get(256);
+    Pinned other = pool.get();
     assert(other.p != young.p);
     pool.put(young);
     pool.put(other);
@@ -101,14 +98,14 @@ def test_a_lost_context_takes_its_slab_with_it(tmp_path):
 def test_each_context_has_its_own_slab(tmp_path):
     check(tmp_path, """
     lbm::PinnedPool<Fake> pool(256, 4);
-    Pinned a = pool.get(256);
+    Pinned a = pool.get();
     pool.driver().now = 2;
-    Pinned b = pool.get(256);
+    Pinned b = pool.get();
     assert(a.slab != b.slab);
     pool.driver().lose(1);
     memset(b.p, 1, 256);
     assert(pool.driver().id(static_cast<char*>(b.p)) == b.slab);   // the second context's is still there
-    Pinned c = pool.get(256);
+    Pinned c = pool.get();
     assert(c.slab == b.slab && c.p != b.p);
     pool.put(a); pool.put(b); pool.put(c);
     """)
@@ -118,29 +115,54 @@ def test_no_memory_and_no_ids(tmp_path):
     check(tmp_path, """
     lbm::PinnedPool<Fake> pool(256, 4);
     pool.driver().fail = 1;
-    assert(!pool.get(256).p && !pool.get(5000).p);
+    assert(!pool.get().p);
     pool.driver().fail = 0;
-    Pinned a = pool.get(256);
+    Pinned a = pool.get();
     assert(a.p);
     pool.put(a);
     struct NoId : Fake { unsigned long long id(void*) { return 0; } };
     lbm::PinnedPool<NoId> blind(256, 4);
-    Pinned b = blind.get(256);
+    Pinned b = blind.get();
     assert(b.p && b.slab == 0 && blind.driver().live.size() == 1);
-    blind.put(b);
-    assert(blind.driver().live.empty());
+    assert(!blind.put(b));                                    // the owner's to release
+    """)
+
+
+def test_many_owners_share_slabs_which_are_given_back(tmp_path):
+    """No owner beyond a slab's blocks pays for memory of its own, and no
+    more than one empty slab stays."""
+    check(tmp_path, """
+    lbm::PinnedPool<Fake> pool(256, 8);
+    std::vector<Pinned> b(100);
+    for (int round = 0; round < 3; ++round) {
+        const int before = pool.driver().allocations;
+        for (auto& x : b) { x = pool.get(); assert(x.p && x.slab); }
+        assert(pool.driver().live.size() == 13 && pool.driver().allocations - before == (round ? 12 : 13));
+        for (size_t k = 0; k < b.size(); ++k) assert(pool.put(b[(k * 37) % 100]));
+        assert(pool.driver().live.size() == 1);
+    }
+    for (int k = 0; k < 50; ++k) {                            // one owner after another, at a full slab's edge too
+        for (int i = 0; i < 8; ++i) b[i] = pool.get();
+        const int before = pool.driver().allocations;
+        for (int i = 0; i < 5; ++i) assert(pool.put(pool.get()));
+        assert(pool.driver().allocations - before == 1 && pool.driver().live.size() == 2);
+        for (int i = 0; i < 8; ++i) assert(pool.put(b[i]));
+        assert(pool.driver().live.size() <= 2);
+        b[8] = pool.get(); b[9] = pool.get();
+        assert(pool.put(b[8]) && pool.put(b[9]));
+    }
     """)
 
 
 def test_threads(tmp_path):
     check(tmp_path, """
     lbm::PinnedPool<Fake> pool(256, 16);
-    Pinned first = pool.get(256);                              // the slab is there: threads only share its blocks
+    Pinned first = pool.get();                              // the slab is there: threads only share its blocks
     std::vector<std::thread> t;
     for (int k = 0; k < 8; ++k)
         t.emplace_back([&, k] {
             for (int i = 0; i < 2000; ++i) {
-                Pinned b = pool.get(256);
+                Pinned b = pool.get();
                 memset(b.p, k + 1, 256);
                 std::this_thread::yield();
                 for (int j = 0; j < 256; ++j) assert(static_cast<char*>(b.p)[j] == k + 1);
