@@ -723,13 +723,19 @@ int status_of(lbm_ctx* c, int i, int* code) {
 // The results of a kernel enqueued with a Notice have reached h_red (and
 // mapped arrays).  The host watches the call's number there, which arrives
 // some microseconds before the end of the stream's work is known, and asks
-// the stream only now and then (so that an error ends the wait).
+// the stream only now and then (so that an error ends the wait).  Where the
+// device is set to yield or to block (cudaSetDeviceFlags), a wait longer than
+// the first such round of polls is left to the stream, which does so.
 lbm::Notice next_notice(lbm_ctx* c) { return {c->h_red, c->d_ticket, ++c->call}; }
 template <typename Here> int wait_for(lbm_ctx* c, Here here) {
     for (unsigned it = 1;; ++it) {
         if (here()) return LBM_OK;
         if (it & 2047u) continue;
-        const cudaError_t e = cudaStreamQuery(c->stream);
+        unsigned flags = 0;
+        cudaError_t e = it == 2048u ? cudaGetDeviceFlags(&flags) : cudaSuccess;
+        if (e == cudaSuccess)
+            e = (flags & (cudaDeviceScheduleYield | cudaDeviceScheduleBlockingSync)) ? cudaStreamSynchronize(c->stream)
+                                                                                     : cudaStreamQuery(c->stream);
         if (e == cudaErrorNotReady) continue;
         if (e != cudaSuccess) return cuda_fail(c, e, "waiting for the results");
         return here() ? LBM_OK : fail(c, LBM_ECUDA, "the stream ended without the results%s");

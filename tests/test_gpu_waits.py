@@ -1,5 +1,5 @@
-"""When results are waited for: a status is that of all the work issued so
-far."""
+"""When and how results are waited for: a status is that of all the work issued
+so far, and a device set to block leaves the core to others."""
 import numpy as np
 import pytest
 
@@ -38,3 +38,34 @@ def test_a_status_asked_for_is_that_of_all_the_work_issued(P):
         lat.init_density(good)
         assert lat.read_fields(which=()) == {}
     lat.close()
+
+
+BLOCKING = r"""
+import ctypes, sys, time
+cu = ctypes.CDLL("libcuda.so.1")
+assert cu.cuInit(0) == 0 and cu.cuDevicePrimaryCtxSetFlags_v2(0, 4) == 0     # CU_CTX_SCHED_BLOCKING_SYNC
+import numpy as np
+import paper_1412_7228_gb300 as P
+eos = P.Eos(kind=P.LBM_EOS_CS, a=1.0, b=4.0, R=1.0, K=1.0, T=0.066)
+lat = P.Lattice(1024, 1024, P.LBM_FP64)
+lat.set_params(eos, -0.85, 0.3, rho_ref=0.2)
+lat.init_density(np.full((1024, 1024), 0.2))
+for call in (lambda: lat.measure(0, 512.0, 512.0, 100.0, 200.0), lat.stats, lambda: lat.read_fields(which=("rho",))):
+    lat.step(10)
+    call()
+    lat.step(1500)
+    w, c = time.perf_counter(), time.thread_time()
+    call()
+    w, c = time.perf_counter() - w, time.thread_time() - c
+    print("%.4f %.4f" % (w, c))
+    assert w > 0.1 and c < 0.3 * w, (w, c)
+"""
+
+
+def test_long_waits_leave_the_core_where_the_device_is_set_to_block(P):
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", BLOCKING], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
