@@ -265,6 +265,7 @@ struct lbm_ctx {
     int parity = 0;
     long long steps = 0, launches = 0;
     int cfg = 0, sched = 0;
+    int cluster = -1;                       // schedule 4: the cluster's configuration
     bool use_graphs = false;
     cudaGraphExec_t gexec[2][kGraphLevels] = {};   // [start parity][level]: 2 << level steps
     lbm::StepArgs<float> one_f{};    // kernel argument block of a one-lattice context
@@ -606,10 +607,12 @@ cudaError_t launch_step(lbm_ctx* c, int parity) {
 int apply_schedule(lbm_ctx* c, int cfg, int sched) {
     if (sched == 3 && !lbm::run_supported(c->prec, cfg))
         return fail(c, LBM_EINVAL, "the multi-step schedule needs a tile configuration of one box per CTA%s");
-    if (sched == 4 && (c->n != 1 || !lbm::cluster_supported(c->prec, c->nx[0], c->ny[0])))
+    const int cluster = sched == 4 && c->n == 1 ? lbm::cluster_pick(c->prec, c->nx[0], c->ny[0]) : -1;
+    if (sched == 4 && cluster < 0)
         return fail(c, LBM_EINVAL, "the cluster schedule needs one lattice that fits one cluster's shared memory%s");
     c->cfg = cfg;
     c->sched = sched;
+    c->cluster = cluster;
     drop_graphs(c);
     CK(c, lbm::step_prepare(c->prec, cfg));
     int rc = encode_maps(c);
@@ -800,7 +803,7 @@ int sync_all(lbm_ctx* c) {
 // one launch, which also writes the ghost cells of the last time level.
 int cluster_steps(lbm_ctx* c, int n) {
     if (n <= 0) return LBM_OK;
-    CK(c, lbm::cluster_run(c->h[0], c->parity, n, c->stream));
+    CK(c, lbm::cluster_run(c->h[0], c->cluster, c->parity, n, c->stream));
     c->parity ^= (n & 1);
     c->steps += n;
     c->launches += 1;
@@ -1761,7 +1764,7 @@ int lbm_autotune(lbm_ctx* c, int steps, int* tile_config, int* schedule, double*
             // one lattice: the one-step launch (0), the multi-step one (3) or
             // the cluster (4, one tile configuration stands for all)
             if ((c->n == 1 && s != 0 && s < 3) || (s == 3 && !lbm::run_supported(c->prec, k))) continue;
-            if (s == 4 && (k > 0 || c->n != 1 || !lbm::cluster_supported(c->prec, c->nx[0], c->ny[0]))) continue;
+            if (s == 4 && (k > 0 || c->n != 1 || lbm::cluster_pick(c->prec, c->nx[0], c->ny[0]) < 0)) continue;
             float ms = 0;
             bool timed_out = false;
             rc = time_one(k, s, &ms, &timed_out);

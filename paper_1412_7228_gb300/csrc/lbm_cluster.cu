@@ -25,6 +25,7 @@
 // is the hardware's, every CTA of the cluster runs the same number of steps
 // and none leaves early, and a CTA's shared memory is only written by the
 // others between two barriers that it takes part in.
+#include "lbm_host_rules.h"
 #include "lbm_step_kernels.cuh"
 
 namespace lbm {
@@ -209,25 +210,36 @@ __global__ void __launch_bounds__(NT, 1) k_cluster(const __grid_constant__ Clust
     if (__syncthreads_or(bad) && tid == 0) atomicOr(a.status, ST_UNSTABLE);
 }
 
+template <typename T> ClusterArgs<T> cluster_args(const Inst& h, int parity, int nsteps) {
+    ClusterArgs<T> a;
+    if constexpr (sizeof(T) == 4) a.P = h.pf;
+    else a.P = h.pd;
+    a.src = static_cast<const T*>(h.pop[parity]);
+    a.dst = static_cast<T*>(h.pop[parity ^ (nsteps & 1)]);
+    a.plane = h.plane;
+    a.pitch = h.pitch;
+    a.nx = h.nx;
+    a.ny = h.ny;
+    a.nsteps = nsteps;
+    a.status = h.status;
+    return a;
+}
+
 // A cluster configuration: strips of BY rows of at most BX nodes, NT threads.
 template <typename T, int BX, int BY, int NT> struct ClusterCfg {
     using Gm = Geom<T, BX, BY, NT, 1>;
     static constexpr size_t smem = 2 * Gm::buf_stride + Gm::psi_stride;
     static_assert(smem <= 232448, "two boxes and the psi tile must fit in a CTA's shared memory");
-    static constexpr int max_ctas = 16;
-    static bool fits(int nx, int ny) {
-        const int C = (ny + BY - 1) / BY;
-        return nx >= 2 && nx <= BX && C <= max_ctas && ny - (C - 1) * BY >= 2;
-    }
+    static constexpr ClusterShape shape = {BX, BY};
     // the launch of one cluster of C CTAs
-    static void config(unsigned C, cudaStream_t st, cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr) {
+    static void config(int C, cudaStream_t st, cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr) {
         cfg = {};
-        cfg.gridDim = dim3(C);
+        cfg.gridDim = dim3(static_cast<unsigned>(C));
         cfg.blockDim = dim3(NT);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = st;
         attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = C;
+        attr.val.clusterDim.x = static_cast<unsigned>(C);
         attr.val.clusterDim.y = 1;
         attr.val.clusterDim.z = 1;
         cfg.attrs = &attr;
@@ -240,18 +252,19 @@ template <typename T, int BX, int BY, int NT> struct ClusterCfg {
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess ||
             cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
             return false;
-        const unsigned C = static_cast<unsigned>((ny + BY - 1) / BY);
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr;
         int n = 0;
-        config(C, nullptr, cfg, attr);
-        return cudaOccupancyMaxActiveClusters(&n, &k_cluster<T, BX, BY, NT>, &cfg) == cudaSuccess && n > 0;
+        config(shape.ctas(ny), nullptr, cfg, attr);
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, &k_cluster<T, BX, BY, NT>, &cfg);
+        if (e != cudaSuccess) cudaGetLastError();   // not the next launch's error
+        return e == cudaSuccess && n > 0;
     }
-    static cudaError_t run(const ClusterArgs<T>& args, cudaStream_t st) {
+    static cudaError_t run(const Inst& h, int parity, int nsteps, cudaStream_t st) {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr;
-        config(static_cast<unsigned>((args.ny + BY - 1) / BY), st, cfg, attr);
-        return cudaLaunchKernelEx(&cfg, &k_cluster<T, BX, BY, NT>, args);
+        config(shape.ctas(h.ny), st, cfg, attr);
+        return cudaLaunchKernelEx(&cfg, &k_cluster<T, BX, BY, NT>, cluster_args<T>(h, parity, nsteps));
     }
 };
 
@@ -263,55 +276,32 @@ template <typename T, int BX, int BY, int NT> struct ClusterCfg {
 // up to 64 high, else 8, up to 64 nodes wide.  Clocks of a 64^2 FP32 step:
 // psi ring 610, collision 590, images and edge rows 590, cluster barrier with
 // the remote stores' arrival 1000.
-using CF32s = ClusterCfg<float, 64, 4, 256>;
-using CF32m = ClusterCfg<float, 64, 8, 512>;
-using CF32a = ClusterCfg<float, 64, 16, 1024>;
-using CF32b = ClusterCfg<float, 128, 8, 1024>;
-using CF64a = ClusterCfg<double, 64, 4, 256>;
-using CF64b = ClusterCfg<double, 64, 8, 512>;
-
-template <typename T>
-ClusterArgs<T> cluster_args(const Inst& h, const Phys<T>& P, int parity, int nsteps) {
-    ClusterArgs<T> a;
-    a.P = P;
-    a.src = static_cast<const T*>(h.pop[parity]);
-    a.dst = static_cast<T*>(h.pop[parity ^ (nsteps & 1)]);
-    a.plane = h.plane;
-    a.pitch = h.pitch;
-    a.nx = h.nx;
-    a.ny = h.ny;
-    a.nsteps = nsteps;
-    a.status = h.status;
-    return a;
-}
+template <class... Cfg> struct ClusterTable {
+    static constexpr int count = sizeof...(Cfg);
+    static constexpr ClusterShape shapes[] = {Cfg::shape...};
+    static int pick(int nx, int ny) {
+        static constexpr bool (*launchable[])(int) = {&Cfg::launchable...};
+        return pick_cluster(shapes, count, nx, ny, [&](int k) { return launchable[k](ny); });
+    }
+    static cudaError_t run(int which, const Inst& h, int parity, int nsteps, cudaStream_t st) {
+        static constexpr cudaError_t (*runs[])(const Inst&, int, int, cudaStream_t) = {&Cfg::run...};
+        return which >= 0 && which < count ? runs[which](h, parity, nsteps, st) : cudaErrorInvalidValue;
+    }
+};
+using ClusterF32 = ClusterTable<ClusterCfg<float, 64, 4, 256>, ClusterCfg<float, 64, 8, 512>,
+                                ClusterCfg<float, 64, 16, 1024>, ClusterCfg<float, 128, 8, 1024>>;
+using ClusterF64 = ClusterTable<ClusterCfg<double, 64, 4, 256>, ClusterCfg<double, 64, 8, 512>>;
 
 }  // namespace
 
-bool cluster_supported(int prec, int nx, int ny) {
-    if (prec == LBM_FP32) {
-        if (CF32s::fits(nx, ny)) return CF32s::launchable(ny);
-        if (CF32m::fits(nx, ny)) return CF32m::launchable(ny);
-        if (CF32a::fits(nx, ny)) return CF32a::launchable(ny);
-        return CF32b::fits(nx, ny) && CF32b::launchable(ny);
-    }
-    if (CF64a::fits(nx, ny)) return CF64a::launchable(ny);
-    return CF64b::fits(nx, ny) && CF64b::launchable(ny);
+int cluster_pick(int prec, int nx, int ny) {
+    return prec == LBM_FP32 ? ClusterF32::pick(nx, ny) : ClusterF64::pick(nx, ny);
 }
 
-cudaError_t cluster_run(const Inst& h, int parity, int nsteps, cudaStream_t st) {
+cudaError_t cluster_run(const Inst& h, int which, int parity, int nsteps, cudaStream_t st) {
     if (nsteps <= 0) return cudaSuccess;
-    if (h.prec == LBM_FP32) {
-        const ClusterArgs<float> a = cluster_args<float>(h, h.pf, parity, nsteps);
-        if (CF32s::fits(h.nx, h.ny)) return CF32s::run(a, st);
-        if (CF32m::fits(h.nx, h.ny)) return CF32m::run(a, st);
-        if (CF32a::fits(h.nx, h.ny)) return CF32a::run(a, st);
-        if (CF32b::fits(h.nx, h.ny)) return CF32b::run(a, st);
-        return cudaErrorInvalidValue;
-    }
-    const ClusterArgs<double> a = cluster_args<double>(h, h.pd, parity, nsteps);
-    if (CF64a::fits(h.nx, h.ny)) return CF64a::run(a, st);
-    if (CF64b::fits(h.nx, h.ny)) return CF64b::run(a, st);
-    return cudaErrorInvalidValue;
+    return h.prec == LBM_FP32 ? ClusterF32::run(which, h, parity, nsteps, st)
+                              : ClusterF64::run(which, h, parity, nsteps, st);
 }
 
 }  // namespace lbm

@@ -352,11 +352,12 @@ cudaError_t run_launch(int prec, int k, const Inst* d_insts, const void* args, b
                        unsigned long long timeout_ns, cudaStream_t st);
 
 // One lattice held in the shared memory of a thread-block cluster for n
-// steps (lbm_cluster.cu; schedule 4): whether this device can run it for an
-// nx x ny lattice of precision prec, and the launch (host: the descriptor;
-// the caller refills the ghost cells of the time level written last).
-bool cluster_supported(int prec, int nx, int ny);
-cudaError_t cluster_run(const Inst& host, int parity, int nsteps, cudaStream_t st);
+// steps (lbm_cluster.cu; schedule 4): the configuration that this device can
+// run for an nx x ny lattice of precision prec (-1: none; sets its kernel's
+// attributes), and the launch of that configuration (host: the descriptor),
+// which writes the ghost cells of the last time level too.
+int cluster_pick(int prec, int nx, int ny);
+cudaError_t cluster_run(const Inst& host, int which, int parity, int nsteps, cudaStream_t st);
 
 // Pinned host memory, mapped for every device (lbm_pinned.cu): up to
 // kPinnedSmall and up to kPinnedBlock bytes come from slabs of the current

@@ -45,3 +45,33 @@ def test_arrays_beyond_one_mapped_range_are_left_to_the_copies(tmp_path):
                lbm::in_place({0x20000, 4}, 4, {0, 0}));
     """)
     assert got == [1, 1, 1, 0, 0, 0, 0, 1, 0, 0]
+
+
+SHAPES = "const lbm::ClusterShape s[4] = {{64, 4}, {64, 8}, {64, 16}, {128, 8}};"   # as in lbm_cluster.cu, FP32
+
+
+def test_a_lattice_takes_the_first_cluster_that_the_device_can_hold(tmp_path):
+    """64^2 in 16, 8 or 4 CTAs; a refusal of one leaves the next."""
+    got = ask(tmp_path, SHAPES + """
+        for (int most : {16, 15, 8, 7, 4, 3})
+            printf("%d ", lbm::pick_cluster(s, 4, 64, 64, [&](int k) { return s[k].ctas(64) <= most; }));
+        printf("%d %d ", lbm::pick_cluster(s, 4, 65, 64, [&](int k) { return s[k].ctas(64) <= 8; }),
+               lbm::pick_cluster(s, 4, 65, 64, [&](int k) { return s[k].ctas(64) <= 7; }));
+    """)
+    assert got == [0, 1, 1, 2, 2, -1, 3, -1]
+
+
+def test_the_lattices_that_fit_a_cluster(tmp_path):
+    """FP32: up to 64 x 256 or 128 x 128, the last strip of 4, 8 or 16 rows (8 beyond
+    64 wide) at least two rows high."""
+    sizes = [(nx, ny) for nx in (1, 2, 64, 65, 128, 129) for ny in range(2, 260)]
+    got = ask(tmp_path, SHAPES + """
+        for (int nx : {1, 2, 64, 65, 128, 129})
+            for (int ny = 2; ny < 260; ++ny) printf("%d ", lbm::pick_cluster(s, 4, nx, ny, [](int) { return true; }));
+    """)
+    for (nx, ny), k in zip(sizes, got):
+        fits = [(bx, by) for bx, by in ((64, 4), (64, 8), (64, 16), (128, 8))
+                if 2 <= nx <= bx and ny <= 16 * by and (ny % by == 0 or ny % by >= 2)]
+        assert (k >= 0) == bool(fits), (nx, ny)
+        if fits:
+            assert ((64, 4), (64, 8), (64, 16), (128, 8))[k] == fits[0]
