@@ -656,25 +656,10 @@ int config_of(int prec, int bx, int by, int threads, int stages) {
     return 0;
 }
 
-// The tile configuration a context starts with, by its nodes: large tiles
-// reload the least halo, small ones fill the SMs.  One-step launches from
-// graphs, us per step.  FP32: 128 x 16 from 2 M nodes on (2500 x 1200 40.0, with
-// 32 x 16 44.2), 64 x 16 from 1.1 M (1531 x 1117 24.3, with 128 x 16 25.4), below
-// persistent 32 x 16 tiles (1000 x 900 14.8 and 16.5, 400^2 6.0 and 7.6, 256^2 4.0
-// and 6.6).  FP64: 32 x 32 from 0.9 M (1024^2 308, with 32 x 8 315), 32 x 8 from
-// 0.45 M (700^2 153, with 16 x 8 156, with 32 x 32 177), below 16 x 8 (400^2 55.8, with
-// 32 x 8 60.9; 100^2 9.4 and 15.6).
+// The tile configuration a context starts with.
 int default_config(const lbm_ctx* c) {
-    long long N = 0;
-    for (int i = 0; i < c->n; ++i) N += static_cast<long long>(c->nx[i]) * c->ny[i];
-    if (c->prec == LBM_FP32) {
-        if (N >= 2000000) return config_of(c->prec, 128, 16, 512, 1);
-        if (N >= 1100000) return config_of(c->prec, 64, 16, 256, 1);
-        return config_of(c->prec, 32, 16, 256, 2);
-    }
-    if (N >= 900000) return config_of(c->prec, 32, 32, 256, 1);
-    if (N >= 450000) return config_of(c->prec, 32, 8, 256, 1);
-    return config_of(c->prec, 16, 8, 128, 1);
+    const lbm::StartTile t = lbm::start_tile(c->prec == LBM_FP64, c->n, c->nx.data(), c->ny.data());
+    return config_of(c->prec, t.bx, t.by, t.threads, t.stages);
 }
 
 template <typename T> void fill_phys(lbm::Phys<T>& P, const HostParams& hp) {

@@ -75,3 +75,29 @@ def test_the_lattices_that_fit_a_cluster(tmp_path):
         assert (k >= 0) == bool(fits), (nx, ny)
         if fits:
             assert ((64, 4), (64, 8), (64, 16), (128, 8))[k] == fits[0]
+
+
+W, M, N = (128, 16), (64, 16), (32, 16)
+
+
+@pytest.mark.parametrize("fp64,n,nx,ny,tile", [
+    # one FP32 lattice: by its nodes, and wide ones of few rows
+    (0, 1, 2, 2, N), (0, 1, 1000, 900, N), (0, 1, 1531, 1117, M), (0, 1, 4096, 4096, W), (0, 1, 50000, 12, W),
+    (0, 1, 1 << 20, 1 << 20, W),
+    # FP32 batches: full 128 x 16 tiles or not, few of them, large lattices, one tile wide, few rows
+    (0, 60, 128, 128, W), (0, 8, 128, 128, N), (0, 15, 256, 256, W), (0, 8, 300, 300, N), (0, 4, 512, 512, M),
+    (0, 60, 70, 70, W), (0, 100, 96, 96, N), (0, 300, 64, 64, M), (0, 1000, 128, 4, N), (0, 60, 256, 256, W),
+    # FP64
+    (1, 6, 128, 4, (16, 8)), (1, 200, 128, 4, (32, 8)), (1, 2000, 128, 4, (32, 8)), (1, 1, 400, 400, (16, 8)),
+    (1, 1, 512, 512, (32, 8)), (1, 1, 600, 600, (16, 8)), (1, 1, 1024, 1024, (32, 32)), (1, 1, 65536, 16, (32, 8)),
+    (1, 1, 100, 10000, (16, 8)), (1, 195, 128, 8, (32, 8)), (1, 1, 1 << 20, 1 << 20, (32, 32))])
+def test_the_tile_a_context_starts_with(tmp_path, fp64, n, nx, ny, tile):
+    """The faster of the tiles on both sides of each line of the rule (the
+    times stand beside it)."""
+    got = ask(tmp_path, """
+        static int nx[2000], ny[2000];
+        for (int i = 0; i < %d; ++i) { nx[i] = %d; ny[i] = %d; }
+        const lbm::StartTile t = lbm::start_tile(%d, %d, nx, ny);
+        printf("%%d %%d ", t.bx, t.by);
+    """ % (n, nx, ny, fp64, n))
+    assert tuple(got) == tile
