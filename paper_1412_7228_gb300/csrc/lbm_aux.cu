@@ -219,12 +219,13 @@ template <typename T> __device__ __forceinline__ void node_pops(const Inst* I, c
 }
 
 // A float as a double, by moving its bits: the conversion instruction holds
-// the FP64 pipe as long as an addition.  Denormals become zero.
+// the FP64 pipe as long as an addition.  A denormal is first made normal (by an
+// exact product with 2^64); the value is below infinity.
 __device__ __forceinline__ double widen(float v) {
-    const unsigned u = __float_as_uint(v), sign = u & 0x80000000u;
-    const bool tiny = (u & 0x7f800000u) == 0;
-    return __hiloint2double(static_cast<int>(tiny ? sign : sign | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
-                            static_cast<int>(tiny ? 0u : u << 29));
+    const bool tiny = (__float_as_uint(v) & 0x7f800000u) == 0;
+    const unsigned u = __float_as_uint(tiny ? __fmul_rn(v, 0x1p64f) : v), mag = u & 0x7fffffffu;
+    const unsigned hi = mag ? (mag >> 3) + (tiny ? 0x38000000u - (64u << 20) : 0x38000000u) : 0u;
+    return __hiloint2double(static_cast<int>((u & 0x80000000u) | hi), static_cast<int>(u << 29));
 }
 
 // Sum of N floats in FP64 accuracy with three FP64 additions: the sum as an

@@ -1,5 +1,5 @@
 """Fields and statistics at the edges of their arguments: densities
-beyond the law's pole.
+beyond the law's pole, FP32 populations below the normal range.
 
 Tolerances.  psi^2 is a difference of terms of the size of the pressure; with
 |1 - b rho| >= 0.09 and 2^-53 per operation over some 40 operations its
@@ -67,4 +67,24 @@ def test_an_fp64_step_across_the_pole_is_the_oracle_s(P, kind):
     O.step(op, f, 1)
     lat.step(1)
     assert np.abs(lat.read_populations() - f).max() <= 1e-12 * np.abs(f).max()
+    lat.close()
+
+
+def test_denormal_populations_are_read_as_they_are(P):
+    """Multiples of 2^-149 below 2^-99: sums of a few are exact in FP64, and
+    the velocity is one division of two of them (within 2 ulp)."""
+    nx, ny = 67, 41
+    rng = np.random.default_rng(11)
+    eos, A = _law(P, "cs")
+    lat = P.Lattice(nx, ny, P.LBM_FP32)
+    lat.set_params(eos, A, 0.0, G=0.0, rho_ref=0.0)
+    lat.init_density(10.0 ** rng.uniform(-42, -31, (ny, nx)), rng.uniform(-0.1, 0.1, (ny, nx)), rng.uniform(-0.1, 0.1, (ny, nx)))
+    f = lat.read_populations()
+    rho, jx, jy = f.sum(0), f[1] - f[3] + f[5] - f[6] - f[7] + f[8], f[2] - f[4] + f[5] + f[6] - f[7] - f[8]
+    assert (np.abs(f) < 1e-38).any() and (rho > 0.0).all()
+    got = lat.read_fields()
+    assert np.array_equal(got["rho"], rho)
+    assert np.array_equal(lat.read_fields(which=("rho",))["rho"], rho)
+    assert (np.abs(got["ux"] - jx / rho) <= 2.0 ** -51 * np.abs(jx / rho)).all()
+    assert (np.abs(got["uy"] - jy / rho) <= 2.0 ** -51 * np.abs(jy / rho)).all()
     lat.close()
