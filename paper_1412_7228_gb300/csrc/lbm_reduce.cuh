@@ -148,13 +148,18 @@ __device__ __forceinline__ double axis2(int v, double c, int n, double inv_n) {
     return d * d;
 }
 
-// num / den rounded like the division up to the last bit's ties: a reciprocal
-// refined to its rounding, then one residual step.  Seven FP64 instructions;
-// the general division's special cases (overflowing or denormal quotients)
-// are not needed for den in (0, 1].
+// num / den rounded like the division up to the last bit's ties: Newton's
+// reciprocal (Fast<double>::rcp), then one residual step (Markstein's, on the
+// quotient).  Six FP64 instructions.  Where the reciprocal leaves the normal
+// range (den zero, denormal, above 2^1021 or not finite) or the residual is no
+// number (an infinite quotient or num), the division decides; the tests for that
+// are integer ones.
+__device__ __noinline__ double divide(double num, double den) { return num / den; }
 __device__ __forceinline__ double quotient(double num, double inv_den, double den) {
-    const double q = num * inv_den;
-    return fma(fma(-q, den, num), inv_den, q);
+    const double q = num * inv_den, r = fma(fma(-q, den, num), inv_den, q);
+    const unsigned exponent = (static_cast<unsigned>(__double2hiint(den)) >> 20) & 0x7ffu;
+    const bool nan = (__double2hiint(r) & 0x7fffffff) > 0x7ff00000;
+    return exponent - 1u >= 2044u || nan ? divide(num, den) : r;
 }
 
 // The pressure law with its constants folded, p = rho [K R T h(rho) - K a rho]

@@ -1,5 +1,6 @@
 """Fields and statistics at the edges of their arguments: densities
-beyond the law's pole, FP32 populations below the normal range.
+beyond the law's pole, FP32 populations below the normal range, FP64 ones at
+both ends of theirs, a density on the pole.
 
 Tolerances.  psi^2 is a difference of terms of the size of the pressure; with
 |1 - b rho| >= 0.09 and 2^-53 per operation over some 40 operations its
@@ -87,4 +88,37 @@ def test_denormal_populations_are_read_as_they_are(P):
     assert np.array_equal(lat.read_fields(which=("rho",))["rho"], rho)
     assert (np.abs(got["ux"] - jx / rho) <= 2.0 ** -51 * np.abs(jx / rho)).all()
     assert (np.abs(got["uy"] - jy / rho) <= 2.0 ** -51 * np.abs(jy / rho)).all()
+    lat.close()
+
+
+@pytest.mark.parametrize("lo,hi", [(-309, -305), (-2, 2), (304, 307)])
+def test_velocities_at_both_ends_of_the_fp64_range(P, lo, hi):
+    """u is the quotient of the read populations' sums, within 2 ulp of the
+    division (of denormal sums: of its own rounding), also where the
+    reciprocal of the density is no normal number."""
+    nx, ny = 43, 39
+    rng = np.random.default_rng(17)
+    eos, A = _law(P, "cs")
+    lat = P.Lattice(nx, ny, P.LBM_FP64)
+    lat.set_params(eos, A, 0.0, G=0.0, rho_ref=0.0)
+    lat.init_density(10.0 ** rng.uniform(lo, hi, (ny, nx)), rng.uniform(-0.1, 0.1, (ny, nx)), rng.uniform(-0.1, 0.1, (ny, nx)))
+    f = lat.read_populations()
+    rho = sum(f[a] for a in range(9))
+    jx, jy = f[1] - f[3] + f[5] - f[6] - f[7] + f[8], f[2] - f[4] + f[5] + f[6] - f[7] - f[8]
+    got = lat.read_fields()
+    assert np.array_equal(got["rho"], rho) and np.isfinite(rho).all()
+    for k, j in (("ux", jx), ("uy", jy)):
+        assert (np.abs(got[k] - j / rho) <= 2.0 ** -51 * np.abs(j / rho)).all(), k
+    lat.close()
+
+
+def test_pressure_of_a_density_on_the_pole(P):
+    """Without the interaction any positive density is allowed: on the pole
+    the law is infinite, and the sample says so."""
+    eos, A = _law(P, "cs")
+    lat = P.Lattice(40, 24, P.LBM_FP64)
+    lat.set_params(eos, A, 0.0, G=0.0, rho_ref=1.0)       # 4 / b
+    lat.init_density(np.ones((24, 40)))
+    m = lat.measure(0, 20.0, 12.0, 5.0, 8.0)
+    assert m["rho_in"] == 1.0 and m["p_in"] == np.inf and m["p_out"] == np.inf
     lat.close()
