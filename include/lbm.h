@@ -93,8 +93,10 @@ int lbm_eos_maxwell(const lbm_eos* eos, double* rho_g, double* rho_l, double* p0
 int lbm_laplace_fit(int n, const double* dp, const double* R, double* sigma, double* icpt,
                     double* r2);
 
-/* Self-check of the FP64 step's reciprocal, division and square root (one
- * third-order, resp. two Goldschmidt, steps from the hardware estimates)
+/* Self-check of the FP64 reciprocal (one third-order step from the hardware
+ * estimate; the step and the read-backs), division (that and one residual
+ * step; read-backs, statistics and samples) and square root (two Goldschmidt
+ * steps; the FP64 kernels fold theirs, of psi, into one reciprocal root)
  * against IEEE-rounded 1/d, a/d and sqrt(d) on the current device: n values
  * of d spread evenly over [lo, hi], numerators a in [0.37, 0.87).  Writes
  * result[0..2] = the largest distances in units in the last place (rcp, div,

@@ -471,7 +471,7 @@ dim3 grid_2d(int nx, int ny) {
     return dim3(static_cast<unsigned>(gx), static_cast<unsigned>(gy));
 }
 
-// ---- the FP64 step's division, reciprocal and square root against IEEE --
+// ---- FP64 reciprocal, division and square root against IEEE --------------
 // Distance in units in the last place; values of opposite sign or NaN count
 // as infinitely far.
 __device__ __forceinline__ unsigned long long ulp_distance(double a, double b) {
@@ -481,8 +481,8 @@ __device__ __forceinline__ unsigned long long ulp_distance(double a, double b) {
     return static_cast<unsigned long long>(x > y ? x - y : y - x);
 }
 
-// out[0..2]: largest distance of Fast<double>::rcp(d), div(a, d), sqrt(d)
-// from 1/d, a/d, sqrt(d) (IEEE-rounded: this file keeps nvcc's default
+// out[0..2]: largest distance of Fast<double>::rcp(d), quotient(a, rcp(d), d)
+// and Fast<double>::sqrt(d) from 1/d, a/d, sqrt(d) (IEEE-rounded: this file keeps nvcc's default
 // -prec-div and -prec-sqrt) over n values of d spread evenly over [lo, hi],
 // a in [0.37, 0.87); out[3] = 1 if sqrt keeps +0, -0 and gives NaN for -1.
 __global__ void k_math_check(long long n, double lo, double hi, unsigned long long* out) {
@@ -491,8 +491,9 @@ __global__ void k_math_check(long long n, double lo, double hi, unsigned long lo
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n; i += stride) {
         const double d = lo + (hi - lo) * (static_cast<double>(i) / static_cast<double>(n));
         const double a = 0.37 + 0.5 * static_cast<double>((i * 2654435761ll) & 0xffff) / 65536.0;
-        m0 = max(m0, ulp_distance(Fast<double>::rcp(d), 1.0 / d));
-        m1 = max(m1, ulp_distance(Fast<double>::div(a, d), a / d));
+        const double inv = Fast<double>::rcp(d);
+        m0 = max(m0, ulp_distance(inv, 1.0 / d));
+        m1 = max(m1, ulp_distance(quotient(a, inv, d), a / d));
         m2 = max(m2, ulp_distance(Fast<double>::sqrt(d), sqrt(d)));
     }
     atomicMax(&out[0], m0);

@@ -193,7 +193,7 @@ template <typename T> __device__ __forceinline__ const Phys<T>& phys(const Inst*
 template <> __device__ __forceinline__ const Phys<float>& phys<float>(const Inst* I) { return I->pf; }
 template <> __device__ __forceinline__ const Phys<double>& phys<double>(const Inst* I) { return I->pd; }
 
-// Division, reciprocal and square root of the fused step.  FP32 uses the
+// Reciprocal, division and square root of the kernels.  FP32 uses the
 // hardware approximations (a couple of ulp, far inside the FP32 error budget
 // of the stored populations).  FP64 refines the hardware estimates
 // (rcp.approx / rsqrt.approx, accurate to about 2^-22) until only the rounding
@@ -201,10 +201,11 @@ template <> __device__ __forceinline__ const Phys<double>& phys<double>(const In
 // r <- r + r (e + e^2), which leaves e^3), sqrt(x) by two steps of
 // Goldschmidt's coupled iteration (g -> sqrt(x), h -> 1/(2 sqrt(x)):
 // r = 1/2 - g h, g <- g + g r, h <- h + h r).  Both stay within 1 ulp of the
-// IEEE-rounded 1/d and sqrt(x), a * rcp(d) within 1 ulp of a/d
-// (lbm_fp64_math_check measures this on the device); they take fewer FP64
-// operations than the IEEE sequences, and the FP64 step is bound by its FP64
-// pipe.  sqrt keeps sqrt(+-0) = +-0 and NaN for x < 0.
+// IEEE-rounded 1/d and sqrt(x) (lbm_fp64_math_check measures this on the
+// device); they take fewer FP64 operations than the IEEE sequences, and what
+// FP64 does is bound by its pipe.  sqrt keeps sqrt(+-0) = +-0 and NaN for x < 0;
+// the FP64 kernels themselves need roots of quotients only (psi_fold_fp64), and
+// their divisions are quotient's (lbm_reduce.cuh).
 template <typename T> struct Fast;
 template <> struct Fast<float> {
     static __device__ __forceinline__ float div(float a, float b) { return __fdividef(a, b); }
@@ -222,7 +223,6 @@ template <> struct Fast<double> {
         const double e = fma(-d, r, 1.0);
         return fma(r, fma(e, e, e), r);
     }
-    static __device__ __forceinline__ double div(double a, double b) { return a * rcp(b); }
     static __device__ __forceinline__ double sqrt(double x) {
         double y;
         asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));

@@ -122,3 +122,24 @@ def test_pressure_of_a_density_on_the_pole(P):
     m = lat.measure(0, 20.0, 12.0, 5.0, 8.0)
     assert m["rho_in"] == 1.0 and m["p_in"] == np.inf and m["p_out"] == np.inf
     lat.close()
+
+
+@pytest.mark.parametrize("kind", ["cs", "vdw", "pr"])
+def test_psi_is_accurate_to_a_few_ulp(P, kind):
+    """psi from the folded reciprocal square root against the square root in
+    extended precision, hot and repulsive (G = 1), where no terms cancel: W
+    and D carry up to 14 roundings, of which the root halves the effect, and
+    the fold 2.5 more, so 9.5 x 2^-53 < 1.1e-15; the constants' 4 make 1.4e-15."""
+    eos, A = _law(P, kind)
+    eos.T *= 40.0
+    lat = P.Lattice(61, 47, P.LBM_FP64)
+    lat.set_params(eos, A, 0.0, G=1.0, s=[1.0] * 9)
+    rng = np.random.default_rng(23)
+    top = 0.2 if kind == "cs" else 0.2 / eos.b
+    lat.init_density(rng.uniform(1e-3 * top, top, (47, 61)))
+    got = lat.read_fields()
+    for field in (got["psi"], lat.read_fields(which=("psi",))["psi"]):
+        r = got["rho"].astype(np.longdouble)
+        want = np.sqrt(2 * (_pressure(P, eos, r) - r / 3))
+        assert np.abs(field / want - 1).max() <= 1.4e-15
+    lat.close()
