@@ -443,11 +443,11 @@ __device__ __forceinline__ bool collide_rows(const float* sf, const float* sp, c
 // ---- the FP64 node ---------------------------------------------------------
 // FP64 is bound by its pipe (19 clocks of an SM per warp instruction, an
 // addition, a product or a fused one alike), so its node is written for the
-// fewest FP64 instructions rather than for the mirror symmetry that the FP32
-// node keeps to the last bit: about 146 with the psi ring's share instead of
+// fewest FP64 instructions: about 146 with the psi ring's share instead of
 // 205 (FP64, 1024^2, per step: 410 -> 289 us multi-step with 32 x 32 tiles, 447 ->
-// 315 us one-step with 32 x 8; 64^2 in a cluster 18.7 -> 13.5 us).  The method is
-// the same:
+// 315 us one-step with 32 x 8; 64^2 in a cluster 18.7 -> 13.5 us).  Its sums too
+// map onto themselves (or their negatives) under the mirrors x -> -x and
+// y -> -y, to the last bit.  The method is the same:
 //  - Eq. 9 and Eq. 23 are linear in g_a = -(G/12) [(1-A) psi(x) psi_a + (A/2)
 //    psi_a^2], so the nine g_a are formed first and each lattice sum once:
 //    F = sum 12 w_a g_a e_a, and Q from the same g with the factor -kappa/2

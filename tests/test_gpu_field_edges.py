@@ -143,3 +143,22 @@ def test_psi_is_accurate_to_a_few_ulp(P, kind):
         want = np.sqrt(2 * (_pressure(P, eos, r) - r / 3))
         assert np.abs(field / want - 1).max() <= 1.4e-15
     lat.close()
+
+
+def test_the_mirrors_hold_to_the_last_bit_in_fp64(P):
+    """As in FP32: a centred drop stays symmetric under x -> -x and y -> -y."""
+    import lbm_inputs as I
+    eos, A = _law(P, "cs")
+    rg, rl, _ = P.lbm_eos_maxwell(eos)
+    n = 64
+    mx, my, xs = [0, 3, 2, 1, 4, 6, 5, 8, 7], [0, 1, 4, 3, 2, 8, 7, 6, 5], (-np.arange(64)) % 64
+    for sched in (0, 4):
+        lat = P.Lattice(n, n, P.LBM_FP64)
+        lat.set_params(eos, A, 0.3, rho_ref=rg)
+        lat.set_schedule(0, sched)
+        lat.init_density(I.droplet_density(n, n, 15, rl, rg))
+        lat.step(1000)
+        f = lat.read_populations()
+        lat.close()
+        for a in range(9):
+            assert np.array_equal(f[a], f[mx[a]][:, xs]) and np.array_equal(f[a], f[my[a]][xs, :]), a
