@@ -17,11 +17,12 @@
  *    the call.  Device memory belongs to the context, unless the caller hands
  *    in dev_buf, which the library then uses but never frees.
  *  - Work is enqueued on the context's CUDA stream.  lbm_step() is
- *    asynchronous; every call that returns data to the host synchronises the
- *    stream.  Device-side faults of the method (a density outside the EOS's
+ *    asynchronous; every call that returns data to the host waits for all the
+ *    work enqueued before it and for its own results (the last kernel of the
+ *    call itself may still be retiring on the stream when it returns).
+ *    Device-side faults of the method (a density outside the EOS's
  *    psi domain, NaN, a bounded wait that gave up) set a sticky per-instance
- *    status that the next synchronising call returns as LBM_EUNSTABLE or
- *    LBM_ETIMEOUT.
+ *    status that the next such call returns as LBM_EUNSTABLE or LBM_ETIMEOUT.
  *  - A context holds one or more independent lattices ("instances"); the
  *    single-lattice calls act on instance 0, the lbm_batch_* calls on
  *    instance i, and lbm_step() advances every instance.
@@ -181,10 +182,10 @@ int lbm_batch_set_viscosity(lbm_ctx* ctx, int i, int enable, double nu_gas, doub
 /* Initial state f_a = M^-1 m_eq(rho, u) (Eq. 4) from host fields of nx*ny
  * doubles; ux, uy may be NULL (zero velocity).  Resets the step counter and
  * the instance's status.  The fields are checked on the device (copied there,
- * or read in place where they lie in pinned memory): a density that is not finite, positive and below the EOS's
- * upper limit (4/b Carnahan-Starling, 1/b otherwise; any positive density
- * when G = 0) or a velocity that is not finite returns LBM_EINVAL and leaves
- * the instance as it was.  A context of one lattice writes the populations
+ * or read in place where they lie aligned in pinned memory): a density that is
+ * not finite, positive and below the EOS's upper limit (4/b Carnahan-Starling,
+ * 1/b otherwise; any positive density when G = 0) or a velocity that is not
+ * finite returns LBM_EINVAL and leaves the instance as it was.  A context of one lattice writes the populations
  * into its other time level while it checks the fields, one of 2^20 nodes or
  * more from pageable memory in row bands, each while the next is copied.
  * Synchronous. */

@@ -21,10 +21,11 @@
 // The per-node arithmetic is that of the one-step kernels on the same box
 // contents, so every schedule gives the same bits.  Nothing goes to global
 // memory between steps: the populations are read once at the start and
-// written once at the end, ghost cells included.  No wait in this kernel spins in software: the cluster barrier
-// is the hardware's, every CTA of the cluster runs the same number of steps
-// and none leaves early, and a CTA's shared memory is only written by the
-// others between two barriers that it takes part in.
+// written once at the end, ghost cells included.  No wait in this kernel spins
+// in software: the cluster barrier is the hardware's, every CTA of the cluster
+// runs the same number of steps and none leaves early, and a CTA's shared
+// memory is only written by the others between two barriers that it takes part
+// in.
 #include "lbm_host_rules.h"
 #include "lbm_step_kernels.cuh"
 

@@ -149,8 +149,8 @@ __device__ __forceinline__ double axis2(int v, double c, int n, double inv_n) {
 }
 
 // num / den rounded like the division up to the last bit's ties: Newton's
-// reciprocal (Fast<double>::rcp), then one residual step (Markstein's, on the
-// quotient).  Six FP64 instructions.  Where the reciprocal leaves the normal
+// reciprocal (Fast<double>::rcp), then one residual step (Markstein, IBM J.
+// Res. Dev. 34, 1990).  Six FP64 instructions.  Where the reciprocal leaves the normal
 // range (den zero, denormal, above 2^1021 or not finite) or the residual is no
 // number (an infinite quotient or num), the division decides; the tests for that
 // are integer ones.

@@ -977,11 +977,13 @@ __device__ __forceinline__ void run_body(const Inst* __restrict__ insts, unsigne
 
 // The kernels.  FP32 launches ask for 1024 resident threads per SM (two
 // CTAs of 512), which caps their registers at 64 (except the batched
-// persistent variant, which would spill); FP64 leaves the register count to
-// the compiler, except for one-tile-per-CTA tiles of one node row per thread
-// (k_step_row), which ask for three resident CTAs: they fit in 85 registers
-// without spilling, and the compiler's own choice for the batched variant
-// (94-98) would leave two.
+// persistent variant, which would spill).  FP64 asks for two resident CTAs of
+// 256 threads, which caps theirs at 128 (the 64 x 16 shapes spill 8 bytes in the
+// batched one-step launch, 12 and 24 in the multi-step ones), and for three with
+// one-tile-per-CTA tiles of one node row per thread (k_step_row, k_run_row:
+// 72 to 80 registers with 256 threads; left alone, the batched variant's 94 to 98
+// would leave two; the 16 x 8 tiles of 128 threads take 94, 149 batched, 150 to
+// 154 multi-step).
 template <typename T, bool ONE> using ArgsOf = typename std::conditional<ONE, StepArgs<T>, BatchArgs<T>>::type;
 
 template <typename T, int BX, int BY, int NT, int NBUF, bool ONE>
