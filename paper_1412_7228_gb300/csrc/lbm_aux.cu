@@ -347,7 +347,7 @@ __device__ __forceinline__ void flow_tile(const Inst* I, const T* p, int x0, int
             jy = fma(0.5, fma(4.0, g(1, 0) - g(-1, 0), a57 - a86), jy);
         }
         const double inv = Fast<double>::rcp(r);
-        use(x, y, r, quotient(jx, inv, r), quotient(jy, inv, r), ps);
+        use(x, y, r, quotient_any(jx, inv, r), quotient_any(jy, inv, r), ps);
     }
     if (interact) __syncthreads();   // before the next tile's psi
 }
@@ -414,12 +414,12 @@ __device__ __forceinline__ void give(const Notice& to, double total, const Inst*
 // no copy and no wait for the stream.  About 22 FP64 instructions per node (nine
 // additions in FP64, the square root and the divisions by the lattice's size
 // are gone).  Per call, FP32: 256^2 88 -> 18 us, 1024^2 236 -> 72 us.
-template <typename T>
+template <typename T, bool EXACT>
 __global__ void __launch_bounds__(kLapThreads) k_measure(const Inst* __restrict__ I, int parity, Discs D, int rpt,
                                                        double* __restrict__ partials, Notice to) {
     __shared__ AxisTable A;
     const T* p = popk<T>(I, parity);
-    LaplaceSums L;
+    LaplaceSums<EXACT> L;
     laplace_tiles(L, LawFp64(I->pd, false), D, I->nx, I->ny, rpt, A,
                   [&](int x, int y) { return node_rho<T>(I, p, x, y); });
     double total;
@@ -673,16 +673,18 @@ cudaError_t aux_flow(const Inst& h, const Inst* d, int parity, int y0, int y1, v
 }
 
 cudaError_t aux_measure(const Inst& h, const Inst* d, int parity, double cxc, double cyc, double r_in,
-                        double r_out, double* partials, int rows, const Notice& to, cudaStream_t st) {
+                        double r_out, bool exact, double* partials, int rows, const Notice& to, cudaStream_t st) {
     if (rows > kResident) rows = kResident;
     const Discs D = make_discs(h.nx, h.ny, cxc, cyc, r_in, r_out);
     const int rpt = tile_rpt(h.nx, h.ny);
     const long long tiles = tile_count(h.nx, h.ny, rpt);
     const int g = static_cast<int>(tiles < rows ? tiles : rows);
-    if (h.prec == LBM_FP32) k_measure<float><<<g, kLapThreads, 0, st>>>(d, parity, D, rpt, partials, to);
-    else k_measure<double><<<g, kLapThreads, 0, st>>>(d, parity, D, rpt, partials, to);
+    auto go = [&](auto k) { k<<<g, kLapThreads, 0, st>>>(d, parity, D, rpt, partials, to); };
+    if (h.prec == LBM_FP32) exact ? go(k_measure<float, true>) : go(k_measure<float, false>);
+    else exact ? go(k_measure<double, true>) : go(k_measure<double, false>);
     return cudaGetLastError();
 }
+bool aux_measure_again(const double (&sums)[kReduceSlots]) { return on_the_pole(sums); }
 
 cudaError_t aux_stats(const Inst& h, const Inst* d, int parity, double* partials, int rows, const Notice& to,
                       cudaStream_t st) {

@@ -884,26 +884,17 @@ int ensure_copy_stream(lbm_ctx* c) {
 // they also take an array at any address, the kernels only whole values).
 enum HostKind { kPinned, kPageable, kOther };
 template <typename O> HostKind host_kind(O* p, size_t n, bool write, O** dev) {
-    cudaPointerAttributes a, b;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaPointerGetAttributes(&b, p + n - 1) != cudaSuccess) {
-        cudaGetLastError();
-        return kOther;
-    }
-    if (a.type == cudaMemoryTypeUnregistered && b.type == cudaMemoryTypeUnregistered) return kPageable;
+    const lbm::HostMemory m = lbm::host_memory(p);
+    if (!m.known) return lbm::host_memory(p + n - 1).known ? kOther : kPageable;
     // pinned, in one mapped range, and not read-only
-    if (a.type != cudaMemoryTypeHost || !a.devicePointer) return kOther;
-    lbm::Span range = {};
-    if (!lbm::pointer_attribute(CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, a.devicePointer, &range.at) ||
-        !lbm::pointer_attribute(CU_POINTER_ATTRIBUTE_RANGE_SIZE, a.devicePointer, &range.bytes) ||
-        !lbm::in_place({reinterpret_cast<uintptr_t>(a.devicePointer), n * sizeof(O)}, sizeof(O), range))
-        return kOther;
+    if (!m.pinned || !lbm::in_place({reinterpret_cast<uintptr_t>(m.device), n * sizeof(O)}, sizeof(O), m.range)) return kOther;
     unsigned flags = 0;
     if (write && (cudaHostGetFlags(&flags, const_cast<std::remove_const_t<O>*>(p)) != cudaSuccess ||
                   (flags & cudaHostRegisterReadOnly))) {
         cudaGetLastError();
         return kOther;
     }
-    *dev = static_cast<O*>(a.devicePointer);
+    *dev = static_cast<O*>(m.device);
     return kPinned;
 }
 
@@ -1535,10 +1526,13 @@ int lbm_batch_measure(lbm_ctx* c, int i, double cxc, double cyc, double r_in, do
     if (!c->inited[i] || !c->hp[i].set) return fail(c, LBM_EINVAL, "instance not initialised%s");
     Range range("lbm_batch_measure");
     CK(c, cudaSetDevice(c->device));
-    CK(c, lbm::aux_measure(c->h[i], c->d_inst + i, c->parity, cxc, cyc, r_in, r_out, partial_rows(c).first,
-                           partial_rows(c).second, next_reduction(c), c->stream));
     double s[lbm::kReduceSlots];
-    if ((rc = wait_reduction(c, s))) return rc;
+    for (bool exact : {false, true}) {
+        CK(c, lbm::aux_measure(c->h[i], c->d_inst + i, c->parity, cxc, cyc, r_in, r_out, exact, partial_rows(c).first,
+                               partial_rows(c).second, next_reduction(c), c->stream));
+        if ((rc = wait_reduction(c, s))) return rc;
+        if (!lbm::aux_measure_again(s)) break;
+    }
     const double N = static_cast<double>(c->nx[i]) * c->ny[i];
     const double p_in = s[3] > 0 ? s[1] / s[3] : NAN, rho_in = s[3] > 0 ? s[2] / s[3] : NAN;
     const double p_out = s[6] > 0 ? s[4] / s[6] : NAN, rho_out = s[6] > 0 ? s[5] / s[6] : NAN;

@@ -18,6 +18,7 @@
 #include <stdint.h>
 
 #include "../../include/lbm.h"
+#include "lbm_host_rules.h"
 #include "lbm_pinned_pool.h"
 
 namespace lbm {
@@ -217,6 +218,13 @@ template <> struct Fast<float> {
     }
 };
 template <> struct Fast<double> {
+    // Of 1 / d, where that is infinite or zero; rarely reached, and volatile
+    // so that it is not computed ahead of the branch to it.
+    static __device__ __forceinline__ double estimate(double d) {
+        double r;
+        asm volatile("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+        return r;
+    }
     static __device__ __forceinline__ double rcp(double d) {
         double r;
         asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
@@ -366,9 +374,15 @@ cudaError_t cluster_run(const Inst& host, int which, int parity, int nsteps, cud
 constexpr size_t kPinnedSmall = 256, kPinnedBlock = (size_t(1) << 16) + 256;
 Pinned pinned_get(size_t bytes);
 void pinned_put(const Pinned& b);
-// An attribute of the memory at p, as the driver has it (out: of the
-// attribute's type); false when p is not known to it.
-bool pointer_attribute(CUpointer_attribute what, const void* p, void* out);
+// What the driver knows about the memory at p: whether it is pinned host
+// memory (and not managed), its address for kernels and the mapped range that
+// address is in; known: whether it knows p at all.
+struct HostMemory {
+    bool known, pinned;
+    void* device;
+    Span range;
+};
+HostMemory host_memory(const void* p);
 
 // What a call reads back besides its arrays, written by the device into
 // pinned host memory mapped for it: the sums of a reduction with its status
@@ -421,8 +435,9 @@ cudaError_t aux_math_check(long long n, double lo, double hi, unsigned long long
 cudaError_t aux_fp64_fma_rate(int iters, cudaStream_t st, double* flops_per_s, double* seconds);
 constexpr int kReduceBlocks = 304;   // rows of partial sums that every context has; larger lattices use their field scratch
 // partials: device doubles for the partial sums of `rows` blocks (kReduceSlots each)
-cudaError_t aux_measure(const Inst& host, const Inst* d_inst, int parity, double cx, double cy,
-                        double r_in, double r_out, double* partials, int rows, const Notice& to, cudaStream_t st);
+cudaError_t aux_measure(const Inst& host, const Inst* d_inst, int parity, double cx, double cy, double r_in,
+                        double r_out, bool exact, double* partials, int rows, const Notice& to, cudaStream_t st);
+bool aux_measure_again(const double (&sums)[kReduceSlots]);   // with exact set
 cudaError_t aux_stats(const Inst& host, const Inst* d_inst, int parity, double* partials, int rows, const Notice& to,
                       cudaStream_t st);
 

@@ -28,21 +28,20 @@ struct CudaDriver {
         return nullptr;
     }
     void release(void* p) { cudaFreeHost(p); }
-    unsigned long long context() {
+    const void* context() {
         static const auto current = driver_function<CUresult (*)(CUcontext*)>("cuCtxGetCurrent");
-        static const auto id_of = driver_function<CUresult (*)(CUcontext, unsigned long long*)>("cuCtxGetId");
         CUcontext c = nullptr;
-        unsigned long long id = 0;
-        if (!current || !id_of) return 0;
-        if (current(&c) == CUDA_SUCCESS && !c) {   // the runtime makes its own current on first use
+        if (current && current(&c) == CUDA_SUCCESS && !c) {   // the runtime makes its own current on first use
             cudaFree(nullptr);
             current(&c);
         }
-        return c && id_of(c, &id) == CUDA_SUCCESS ? id : 0;
+        return c;
     }
     unsigned long long id(void* p) {
+        static const auto get =
+            driver_function<CUresult (*)(void*, CUpointer_attribute, CUdeviceptr)>("cuPointerGetAttribute");
         unsigned long long v = 0;
-        return pointer_attribute(CU_POINTER_ATTRIBUTE_BUFFER_ID, p, &v) ? v : 0;
+        return get && get(&v, CU_POINTER_ATTRIBUTE_BUFFER_ID, reinterpret_cast<CUdeviceptr>(p)) == CUDA_SUCCESS ? v : 0;
     }
 };
 PinnedPool<CudaDriver>& small_pool() {
@@ -56,9 +55,22 @@ PinnedPool<CudaDriver>& pool() {
 
 }  // namespace
 
-bool pointer_attribute(CUpointer_attribute what, const void* p, void* out) {
-    static const auto get = driver_function<CUresult (*)(void*, CUpointer_attribute, CUdeviceptr)>("cuPointerGetAttribute");
-    return get && get(out, what, reinterpret_cast<CUdeviceptr>(p)) == CUDA_SUCCESS;
+HostMemory host_memory(const void* p) {
+    static const auto get =
+        driver_function<CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr)>("cuPointerGetAttributes");
+    HostMemory m = {};
+    unsigned type = 0, managed = 0;   // type 0: unknown
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                  CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* to[] = {&type, &managed, &m.device, &m.range.at, &m.range.bytes};
+    if (!get || get(5, what, to, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) {
+        m.known = true;   // left to the copies
+        return m;
+    }
+    m.known = type != 0 || managed != 0;
+    m.pinned = type == CU_MEMORYTYPE_HOST && !managed && m.device;
+    return m;
 }
 
 Pinned pinned_get(size_t bytes) {

@@ -12,6 +12,7 @@
 #include <stddef.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <mutex>
 #include <vector>
 
@@ -22,9 +23,10 @@ struct Pinned {
     unsigned long long slab = 0;   // 0: straight from the driver
 };
 
-// Driver: void* allocate(size_t); void release(void*); the process-wide ids
-// unsigned long long context() of the current context and
-// unsigned long long id(void*) of the live allocation at an address (0: none).
+// Driver: void* allocate(size_t); void release(void*); const void* context(),
+// the current context (one made later may have the handle of a lost one), and
+// unsigned long long id(void*), the process-wide id of the live allocation at
+// an address (0: none).
 //
 // A context whose slabs are all taken gets another, and one that becomes empty
 // is given back unless it is the context's only empty one: the pinned memory
@@ -62,7 +64,8 @@ public:
 private:
     struct Slab {
         char* base;
-        unsigned long long id, context;
+        unsigned long long id;
+        const void* context;
         std::vector<char> used;
         int taken;
     };
@@ -70,11 +73,14 @@ private:
     // a free block of the current context's slabs, or none
     Pinned take() {
         std::lock_guard<std::mutex> lock(mu_);
-        slabs_.erase(std::remove_if(slabs_.begin(), slabs_.end(), [&](const Slab& s) { return !alive(s); }), slabs_.end());
-        const unsigned long long context = driver_.context();
+        const void* const context = driver_.context();
         Slab* from = nullptr;
-        for (Slab& s : slabs_)
-            if (s.context == context && s.taken < blocks_) from = &s;
+        for (size_t k = 0; k < slabs_.size() && !from;) {
+            Slab& s = slabs_[k];
+            if (s.context != context || s.taken == blocks_) ++k;
+            else if (alive(s)) from = &s;
+            else slabs_.erase(slabs_.begin() + static_cast<std::ptrdiff_t>(k));   // its context is gone
+        }
         if (!from) {
             void* const base = driver_.allocate(block_ * blocks_);
             if (!base) return {};

@@ -150,22 +150,34 @@ __device__ __forceinline__ double axis2(int v, double c, int n, double inv_n) {
 
 // num / den rounded like the division up to the last bit's ties: Newton's
 // reciprocal (Fast<double>::rcp), then one residual step (Markstein, IBM J.
-// Res. Dev. 34, 1990).  Six FP64 instructions.  Where the reciprocal leaves the normal
-// range (den zero, denormal, above 2^1021 or not finite) or the residual is no
-// number (an infinite quotient or num), the division decides; the tests for that
-// are integer ones.
-__device__ __noinline__ double divide(double num, double den) { return num / den; }
+// Res. Dev. 34, 1990).  Six FP64 instructions.  NaN where den is zero or not
+// finite or the quotient is infinite.
 __device__ __forceinline__ double quotient(double num, double inv_den, double den) {
-    const double q = num * inv_den, r = fma(fma(-q, den, num), inv_den, q);
-    const unsigned exponent = (static_cast<unsigned>(__double2hiint(den)) >> 20) & 0x7ffu;
-    const bool nan = (__double2hiint(r) & 0x7fffffff) > 0x7ff00000;
-    return exponent - 1u >= 2044u || nan ? divide(num, den) : r;
+    const double q = num * inv_den;
+    return fma(fma(-q, den, num), inv_den, q);
+}
+// Where that is no number, or the reciprocal leaves the normal range (den
+// zero, denormal, from 2^1022 on or not finite): num and den scaled by a power
+// of two first, and the product with the reciprocal's estimate (infinite or
+// zero then) where the quotient still is none.  The tests are integer ones, and
+// calling the division instead would cost the kernels registers (48 -> 56).
+__device__ __forceinline__ bool not_a_number(double v) { return (__double2hiint(v) & 0x7fffffff) > 0x7ff00000; }
+__device__ __forceinline__ double quotient_any(double num, double inv_den, double den) {
+    double r = quotient(num, inv_den, den);
+    if ((static_cast<unsigned>(__double2hiint(den)) << 1) - (1u << 21) >= 2044u << 21) {
+        const double scale = (__double2hiint(den) & 0x7fffffff) < 0x3ff00000 ? 0x1p200 : 0x1p-200;
+        num *= scale;
+        den *= scale;
+        r = quotient(num, Fast<double>::rcp(den), den);
+    }
+    return not_a_number(r) ? num * Fast<double>::estimate(den) : r;
 }
 
 // The pressure law with its constants folded, p = rho [K R T h(rho) - K a rho]
 // (h = num / q^3 for Carnahan-Starling), and psi = W / sqrt(W D) with Eq.
 // 10's radicand (2/G)(p - rho/3) = W / D: 16 (with the sum) and 17 FP64
-// instructions.
+// instructions.  On its pole the pressure is infinite, which quotient does not
+// give; EXACT: by the division.
 struct LawFp64 {
     int eos;
     double b, c1, c2, c3;   // p: K R T, K a (K a alpha), 0; psi: those and 1/3, times 2/G
@@ -178,11 +190,11 @@ struct LawFp64 {
         c3 = psi ? s * (1.0 / 3.0) : 0.0;
     }
     // p / rho
-    __device__ __forceinline__ double pressure_over_rho(double rho) const {
+    template <bool EXACT> __device__ __forceinline__ double pressure_over_rho(double rho) const {
         const double n = b * rho, q = 1.0 - n;
-        if (eos == LBM_EOS_CS) return c1 * div(fma(n, fma(n, q, 1.0), 1.0), q * q * q) - c2 * rho;
-        if (eos == LBM_EOS_VDW) return div(c1, q) - c2 * rho;
-        return div(c1, q) - div(c2 * rho, fma(n, 2.0 - n, 1.0));
+        if (eos == LBM_EOS_CS) return c1 * div<EXACT>(fma(n, fma(n, q, 1.0), 1.0), q * q * q) - c2 * rho;
+        if (eos == LBM_EOS_VDW) return div<EXACT>(c1, q) - c2 * rho;
+        return div<EXACT>(c1, q) - div<EXACT>(c2 * rho, fma(n, 2.0 - n, 1.0));
     }
     __device__ __forceinline__ double psi(double rho) const {
         const double n = b * rho, q = 1.0 - n;
@@ -194,14 +206,16 @@ struct LawFp64 {
         const double e = fma(n, 2.0 - n, 1.0);
         return psi_fold_fp64(rho * fma(-fma(c2, rho, c3 * e), q, c1 * e), q * e);
     }
-    static __device__ __forceinline__ double div(double num, double den) { return quotient(num, Fast<double>::rcp(den), den); }
+    template <bool EXACT> static __device__ __forceinline__ double div(double num, double den) {
+        return EXACT ? num / den : quotient(num, Fast<double>::rcp(den), den);
+    }
 };
 
 // Laplace sums of one thread: {sum rho, sum p_in, sum rho_in, n_in,
 // sum p_out, sum rho_out, n_out, 0}; p = p_EOS(rho).  A node's density is
 // added once: to the disc it belongs to, or to `rest` when it belongs to
 // neither (taken off it when it belongs to both).
-struct LaplaceSums {
+template <bool EXACT> struct LaplaceSums {
     double v[8] = {0, 0, 0, 0, 0, 0, 0, 0}, rest = 0.0;
     int n_in = 0, n_out = 0;
     __device__ __forceinline__ void add(const LawFp64& p_eos, const Discs& D, double r, double d2) {
@@ -209,7 +223,7 @@ struct LaplaceSums {
         const bool in = b <= D.in2, out = b >= D.out2;
         if (in == out) rest += in ? -r : r;
         if (!in && !out) return;
-        const double p = p_eos.pressure_over_rho(r);   // its product with rho goes into the sum
+        const double p = p_eos.template pressure_over_rho<EXACT>(r);   // its product with rho goes into the sum
         if (in) {
             v[1] = fma(r, p, v[1]);
             v[2] += r;
@@ -252,14 +266,18 @@ inline int tile_rpt(int nx, int ny) {
     }
     return best;
 }
+// Whether the sums have to be formed again, by the divisions: a pressure that is
+// no number over densities that are (one of them on the law's pole).
+inline bool on_the_pole(const double (&s)[8]) { return std::isfinite(s[0]) && (std::isnan(s[1]) || std::isnan(s[4])); }
+
 // The sums over the tiles of this block; rho_at(x, y) gives a node's density.
 // A tile's squared distances along x and y are formed once, in shared memory,
 // while the first densities arrive.
 struct AxisTable {
     double x[kTileX], y[kTileRows * kMaxRpt];
 };
-template <typename F>
-__device__ __forceinline__ void laplace_tiles(LaplaceSums& L, const LawFp64& p_eos, const Discs& D, int nx, int ny,
+template <bool EXACT, typename F>
+__device__ __forceinline__ void laplace_tiles(LaplaceSums<EXACT>& L, const LawFp64& p_eos, const Discs& D, int nx, int ny,
                                               int rpt, AxisTable& A, F rho_at) {
     const int rows = kTileRows * rpt, t = threadIdx.x, tx = t % kTileX, ty = t / kTileX;
     const int tiles_x = (nx + kTileX - 1) / kTileX, tiles = tiles_x * ((ny + rows - 1) / rows);

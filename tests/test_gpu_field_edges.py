@@ -122,6 +122,14 @@ def test_pressure_of_a_density_on_the_pole(P):
     m = lat.measure(0, 20.0, 12.0, 5.0, 8.0)
     assert m["rho_in"] == 1.0 and m["p_in"] == np.inf and m["p_out"] == np.inf
     lat.close()
+    import torch
+    field = torch.ones((24, 40), dtype=torch.float64, device="cuda")
+    field[12, 20] = 0.1                                   # p_in over the other nodes too
+    m = P.lbm.lbm_field_pressure_jump_static(field.data_ptr(), 40, 24, eos, 20.0, 12.0, 5.0, 8.0)
+    assert m["p_in"] == np.inf and m["p_out"] == np.inf
+    field[:] = 0.1
+    m = P.lbm.lbm_field_pressure_jump_static(field.data_ptr(), 40, 24, eos, 20.0, 12.0, 5.0, 8.0)
+    assert abs(m["p_in"] - P.lbm_eos_pressure(eos, 0.1)) < 1e-15
 
 
 @pytest.mark.parametrize("kind", ["cs", "vdw", "pr"])

@@ -33,7 +33,7 @@ struct Fake {
         return p;
     }
     void release(void* p) { assert(live.erase(static_cast<char*>(p)) == 1); }
-    unsigned long long context() { return now; }
+    const void* context() { return reinterpret_cast<void*>(static_cast<intptr_t>(now)); }
     unsigned long long id(void* p) {
         auto it = live.find(static_cast<char*>(p));
         return it == live.end() ? 0 : it->second.second.first;
