@@ -105,3 +105,34 @@ def test_pinned_arrays_at_any_address(P, nx, ny, dtype):
     lat.init_density(*views[:3])
     assert np.array_equal(lat.read_populations(), state)
     lat.close()
+
+
+def test_small_reads_of_many_lattices_in_threads(P):
+    """The stage that small pageable fields come through is borrowed for a
+    call: more lattices than a slab has blocks, read by several threads."""
+    import threading
+    lats, wants = [], []
+    for k in range(18):
+        nx, ny = 20 + 3 * k, 40
+        lat = _lattice(P, nx, ny, P.LBM_FP32 if k % 2 else P.LBM_FP64)
+        lat.init_density(*_inputs(nx, ny, np.float64))
+        lat.step(3)
+        lats.append(lat)
+        wants.append((lat.read_fields(which=("rho", "psi")), lat.measure(0, 10.0, 20.0, 4.0, 9.0)))
+    wrong = []
+
+    def work(mine):
+        for _ in range(40):
+            for k in mine:
+                got, m = lats[k].read_fields(which=("rho", "psi")), lats[k].measure(0, 10.0, 20.0, 4.0, 9.0)
+                if not (all(np.array_equal(got[f], wants[k][0][f]) for f in got) and m == wants[k][1]):
+                    wrong.append(k)
+
+    threads = [threading.Thread(target=work, args=(range(t, 18, 6),)) for t in range(6)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
+    for lat in lats:
+        lat.close()
