@@ -42,20 +42,11 @@ constexpr int kGraphLevels = 5;                            // captured graphs of
 constexpr int kGraphSteps = 2 << (kGraphLevels - 1);       // the longest: 32 steps
 constexpr int kReadBands = 8;                              // row bands of a large field's transfers
 constexpr size_t kReadBandMin = size_t(1) << 20;           // nodes from which the read-back is banded
-// Pinned stage that a read-back of small fields borrows.  Read of rho into pageable
-// memory: 64^2 FP32 17.2 -> 12.7 us staged, 256^2 19.0 -> 27.0 (the host's copy takes over).
+// Pinned stage of a context for small fields, from the first read-back on that needs
+// it.  Read of rho into pageable memory: 64^2 FP32 17.2 -> 12.7 us staged, 256^2 19.0
+// -> 27.0 (the host's copy takes over).
 constexpr size_t kStageBytes = size_t(1) << 16;
 static_assert(kStageBytes <= lbm::kPinnedBlock, "the stage is a block of the pool");
-struct Stage {
-    lbm::Pinned block;
-    Stage() = default;
-    Stage(const Stage&) = delete;
-    ~Stage() { lbm::pinned_put(block); }
-    char* get() {
-        if (!block.p) block = lbm::pinned_get(kStageBytes);
-        return static_cast<char*>(block.p);
-    }
-};
 
 // The TMA tensor maps of one instance's two time levels (host copies; the
 // kernels receive them in their argument blocks).
@@ -258,7 +249,7 @@ struct lbm_ctx {
     double* d_partials = nullptr;
     double* d_result = nullptr;
     unsigned* d_ticket = nullptr;           // of the reductions' last block; zero between launches
-    lbm::Pinned pinned;
+    lbm::Pinned pinned, stage;
     lbm::Reduced* h_red = nullptr;          // in it (pinned, mapped): the device writes results and the status here
     unsigned call = 0;                      // number of the last call that waits for them (h_red->call)
     double* d_scratch = nullptr;
@@ -885,7 +876,7 @@ int ensure_copy_stream(lbm_ctx* c) {
 enum HostKind { kPinned, kPageable, kOther };
 template <typename O> HostKind host_kind(O* p, size_t n, bool write, O** dev) {
     const lbm::HostMemory m = lbm::host_memory(p);
-    if (!m.known) return lbm::host_memory(p + n - 1).known ? kOther : kPageable;
+    if (!m.known) return kPageable;
     // pinned, in one mapped range, and not read-only
     if (!m.pinned || !lbm::in_place({reinterpret_cast<uintptr_t>(m.device), n * sizeof(O)}, sizeof(O), m.range)) return kOther;
     unsigned flags = 0;
@@ -1037,12 +1028,11 @@ template <typename O> int read_fields_t(lbm_ctx* c, int i, O* rho, O* ux, O* uy,
     }
     c->h_red->status = 0;
     // where they can, the kernels write straight to where the host reads: the
-    // caller's arrays if they are pinned, else (small ones) a pinned
+    // caller's arrays if they are pinned, else (small ones) the context's
     // stage; no copy is enqueued and no stream waited for (rho into pinned
     // memory, FP32: 64^2 15.3 -> 11.3 us per call, 512^2 29.3 -> 19.0, 1024^2 in
     // bands 67 -> 40 us)
     {
-        Stage stage;   // given back at the end: the kernels are done with it on every way out
         O* to[4] = {};
         size_t staged = 0;
         bool direct = true, through[4] = {};
@@ -1052,8 +1042,10 @@ template <typename O> int read_fields_t(lbm_ctx* c, int i, O* rho, O* ux, O* uy,
             if (kind == kPinned) continue;
             const size_t at = staged;
             staged += (N * sizeof(O) + 15) / 16 * 16;
-            direct = through[f] = kind == kPageable && staged <= kStageBytes && stage.get();
-            if (direct) to[f] = reinterpret_cast<O*>(stage.get() + at);
+            direct = through[f] = kind == kPageable && staged <= kStageBytes;
+            if (direct && !c->stage.p) c->stage = lbm::pinned_get(kStageBytes);
+            if (!c->stage.p) direct = false;   // none to be had: the copies
+            if (direct) to[f] = reinterpret_cast<O*>(static_cast<char*>(c->stage.p) + at);
         }
         if (direct && !groups.empty()) {
             auto issue = [&]() -> int {
@@ -1355,6 +1347,7 @@ void lbm_destroy(lbm_ctx* c) {
     for (auto& e : c->band_done)
         if (e) cudaEventDestroy(e);
     lbm::pinned_put(c->pinned);
+    lbm::pinned_put(c->stage);
     if (c->owns && c->buf) cudaFree(c->buf);
     delete c;
 }

@@ -1,7 +1,7 @@
 // lbm_pinned.cu -- pinned host memory, mapped for the devices, of the contexts
 // and networks.  It comes in slabs: of 256 blocks for what each context keeps
-// (64 KB), and of 8 for the networks and for the stage that a read-back borrows
-// while it lasts (half a megabyte), so that making a context costs no
+// (64 KB), and of 8 for the networks and for the stage of small pageable
+// read-backs (half a megabyte), so that making a context costs no
 // allocation by the driver however many are open (64 of 64^2 at once: 23.3 us to
 // make and 1.1 to close each; with an allocation of its own for each beyond the
 // eighth 30.0 and 6.7).  Larger requests go to the driver.  A block's owner has waited

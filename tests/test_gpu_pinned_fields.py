@@ -108,8 +108,8 @@ def test_pinned_arrays_at_any_address(P, nx, ny, dtype):
 
 
 def test_small_reads_of_many_lattices_in_threads(P):
-    """The stage that small pageable fields come through is borrowed for a
-    call: more lattices than a slab has blocks, read by several threads."""
+    """Small pageable fields come through a stage from a slab of blocks: more
+    lattices than a slab has, read by several threads."""
     import threading
     lats, wants = [], []
     for k in range(18):
