@@ -285,8 +285,8 @@ __device__ __forceinline__ void node_j(const double (&v)[9], double& jx, double&
 
 // Tiles of the kernels that need the force (velocity fields, statistics):
 // psi of the tile and its 1-node ring (periodic) goes to shared memory once,
-// so a node costs 1.25 densities and psi instead of nine, and about 65 FP64
-// instructions instead of 700 (the FP64 pipe is the bound: 19 clocks of an
+// so a node costs 1.25 densities and psi instead of nine, and 64 FP64
+// instructions (FP32 velocities; statistics 76) instead of 700 (the FP64 pipe is the bound: 19 clocks of an
 // SM per warp instruction).  32 x 16 nodes: two per thread, a ring of 612
 // nodes in 20 warp passes for 16 of the tile's own.  FP32 statistics of
 // 1024^2: 1113 -> 177 us per call, of 256^2: 149 -> 27; the two velocity

@@ -50,8 +50,8 @@ std::mutex g_mu;
 double* g_ptr[kMaxDevices] = {};
 
 // The Laplace sums of a field (LaplaceSums) in one launch, bound by the FP64
-// pipe (19 instructions per node; 4096^2: 1970 -> 689 us per call, of which
-// the former second launch was 168).
+// pipe (17.5 instructions per node; 4096^2: 1970 -> 689 us per call, 617 on the
+// device; the former second launch was 168).  EXACT: see LawFp64.
 template <bool EXACT>
 __global__ void __launch_bounds__(kLapThreads)
     k_field_sums(const double* __restrict__ rho, int nx, int ny, Phys<double> P, Discs D, int rpt,
